@@ -2,13 +2,16 @@
 
 Every step of the path (activation quantizer, group-wise weight quantizer and packer, integer
 GEMM with dequantizing epilogue, encoder-layer linear stack) runs in the CUDA kernels behind the C
-ABI declared in ``include/qbert.h``.  torch is used for device buffers and the current stream.
-There is no CPU fallback: if ``libqbert.so`` has not been built, importing works but the first call
-raises ``QbertError``.
+ABI declared in ``include/qbert.h``.  torch is used for device buffers and the current stream.  The calls
+that a model makes on every pass go through ``_qbert.so`` (tensors read, outputs allocated and the stream
+looked up in C++), the others through ctypes.  There is no CPU fallback: if the libraries have not been
+built, importing works but the first call raises ``QbertError``.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 from dataclasses import dataclass
 from pathlib import Path
 from typing import Optional, Sequence
@@ -17,6 +20,7 @@ import torch
 
 _PKG = Path(__file__).resolve().parent
 LIB_PATH = _PKG / "libqbert.so"
+EXT_PATH = _PKG / "_qbert.so"  # the calls made on every pass, marshalled in C++ (csrc/binding.cpp)
 
 QB_OK = 0
 QB_ERR_INVALID = -1
@@ -144,6 +148,24 @@ def lib() -> ctypes.CDLL:
     return L
 
 
+_native = None
+
+
+def _ext():
+    """Load ``_qbert.so`` on the first call that needs it."""
+    global _native
+    lib()
+    if not EXT_PATH.exists():
+        raise QbertError(QB_ERR_CUDA, f"{EXT_PATH} is missing: build it with "
+                                      "`python -m paper_1909_05840_b200.build`; there is no CPU fallback")
+    loader = importlib.machinery.ExtensionFileLoader("_qbert", str(EXT_PATH))
+    mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_qbert", loader))
+    loader.exec_module(mod)
+    mod.set_raise(_check)
+    _native = mod
+    return mod
+
+
 def _check(status: int, what: str) -> None:
     if status != QB_OK:
         L = lib()
@@ -156,7 +178,7 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def version() -> int:
@@ -186,14 +208,7 @@ def read_status(ws: torch.Tensor) -> int:
 def quantize_act(x: torch.Tensor, ws: torch.Tensor, xq: Optional[torch.Tensor] = None,
                  act_scale: Optional[torch.Tensor] = None, rowsum: Optional[torch.Tensor] = None):
     """``qb_quantize_act``: fp32 [M,K] -> (int8 codes [M,K], fp32 scale [1], int32 row sums [M])."""
-    assert x.is_cuda and x.dtype == torch.float32 and x.dim() == 2 and x.is_contiguous()
-    M, K = x.shape
-    xq = torch.empty((M, K), dtype=torch.int8, device=x.device) if xq is None else xq
-    act_scale = torch.empty(1, dtype=torch.float32, device=x.device) if act_scale is None else act_scale
-    rowsum = torch.empty(M, dtype=torch.int32, device=x.device) if rowsum is None else rowsum
-    _check(lib().qb_quantize_act(x.data_ptr(), M, K, xq.data_ptr(), act_scale.data_ptr(), rowsum.data_ptr(),
-                                 ws.data_ptr(), ws.numel(), _stream()), "qb_quantize_act")
-    return xq, act_scale, rowsum
+    return (_native or _ext()).quantize_act(x, ws, xq, act_scale, rowsum)
 
 
 def quantize_pack_weights(w: torch.Tensor, bits: int, groups: int, ws: torch.Tensor,
@@ -201,81 +216,40 @@ def quantize_pack_weights(w: torch.Tensor, bits: int, groups: int, ws: torch.Ten
                           packed: Optional[torch.Tensor] = None, delta: Optional[torch.Tensor] = None,
                           q0: Optional[torch.Tensor] = None):
     """``qb_quantize_pack_weights``: fp32 [N,K] -> (int32-viewed packed words [N, K*bits/32], delta [G], q0 [G])."""
-    assert w.is_cuda and w.dtype == torch.float32 and w.dim() == 2 and w.is_contiguous()
-    N, K = w.shape
-    if packed is None:
-        words_per_row = max(1, K * bits // 32)
-        packed = torch.empty((N, words_per_row), dtype=torch.int32, device=w.device)
-    delta = torch.empty(max(groups, 1), dtype=torch.float32, device=w.device) if delta is None else delta
-    q0 = torch.empty(max(groups, 1), dtype=torch.float32, device=w.device) if q0 is None else q0
-    _check(lib().qb_quantize_pack_weights(w.data_ptr(), N, K, bits, groups, _ptr(range_lo), _ptr(range_hi),
-                                          packed.data_ptr(), delta.data_ptr(), q0.data_ptr(), ws.data_ptr(),
-                                          ws.numel(), _stream()), "qb_quantize_pack_weights")
-    return packed, delta, q0
+    return (_native or _ext()).quantize_pack_weights(w, bits, groups, ws, range_lo, range_hi, packed, delta, q0)
 
 
 def fake_quantize_weights(w: torch.Tensor, bits: int, groups: int, ws: torch.Tensor,
                           range_lo: Optional[torch.Tensor] = None, range_hi: Optional[torch.Tensor] = None,
                           wq: Optional[torch.Tensor] = None):
     """``qb_fake_quantize_weights``: fp32 [N,K] -> (Q(W) fp32 [N,K], delta [G], q0 [G])."""
-    assert w.is_cuda and w.dtype == torch.float32 and w.dim() == 2 and w.is_contiguous()
-    N, K = w.shape
-    wq = torch.empty_like(w) if wq is None else wq
-    delta = torch.empty(groups, dtype=torch.float32, device=w.device)
-    q0 = torch.empty(groups, dtype=torch.float32, device=w.device)
-    _check(lib().qb_fake_quantize_weights(w.data_ptr(), N, K, bits, groups, _ptr(range_lo), _ptr(range_hi),
-                                          wq.data_ptr(), delta.data_ptr(), q0.data_ptr(), ws.data_ptr(), ws.numel(),
-                                          _stream()), "qb_fake_quantize_weights")
-    return wq, delta, q0
+    return (_native or _ext()).fake_quantize_weights(w, bits, groups, ws, range_lo, range_hi, wq)
 
 
 def fake_quantize_weights_batch(items, ws: torch.Tensor) -> None:
     """``qb_fake_quantize_weights_batch`` over ``(w, bits, groups, wq, delta, q0)`` tuples (or a C array whose
     ``packed`` fields point to the fp32 outputs)."""
     arr = items if isinstance(items, ctypes.Array) else make_weight_desc_array(items)
-    _check(lib().qb_fake_quantize_weights_batch(arr, len(arr), ws.data_ptr(), ws.numel(), _stream()),
-           "qb_fake_quantize_weights_batch")
+    (_native or _ext()).fake_quantize_weights_batch(arr, ws)
 
 
 def ste_backward(grad_wq: torch.Tensor, w: torch.Tensor, groups: int, range_lo: Optional[torch.Tensor] = None,
                  range_hi: Optional[torch.Tensor] = None, grad_w: Optional[torch.Tensor] = None) -> torch.Tensor:
     """``qb_ste_backward``: straight-through gradient of the quantizer with respect to the weights."""
-    assert grad_wq.is_cuda and grad_wq.dtype == torch.float32 and grad_wq.is_contiguous() and grad_wq.shape == w.shape
-    N, K = w.shape
-    grad_w = torch.empty_like(w) if grad_w is None else grad_w
-    _check(lib().qb_ste_backward(grad_wq.data_ptr(), w.data_ptr(), N, K, groups, _ptr(range_lo), _ptr(range_hi),
-                                 grad_w.data_ptr(), _stream()), "qb_ste_backward")
-    return grad_w
+    return (_native or _ext()).ste_backward(grad_wq, w, groups, range_lo, range_hi, grad_w)
 
 
 def quantize_embedding(table: torch.Tensor, bits: int, groups: int, ws: torch.Tensor,
                        packed: Optional[torch.Tensor] = None):
     """``qb_quantize_embedding``: fp32 [V,D] -> (int32-viewed packed rows [V, D*bits/32], delta [G], q0 [G])."""
-    assert table.is_cuda and table.dtype == torch.float32 and table.dim() == 2 and table.is_contiguous()
-    V, D = table.shape
-    if packed is None:
-        packed = torch.empty((V, D * bits // 32), dtype=torch.int32, device=table.device)
-    delta = torch.empty(groups, dtype=torch.float32, device=table.device)
-    q0 = torch.empty(groups, dtype=torch.float32, device=table.device)
-    _check(lib().qb_quantize_embedding(table.data_ptr(), V, D, bits, groups, packed.data_ptr(), delta.data_ptr(),
-                                       q0.data_ptr(), ws.data_ptr(), ws.numel(), _stream()), "qb_quantize_embedding")
-    return packed, delta, q0
+    return (_native or _ext()).quantize_embedding(table, bits, groups, ws, packed)
 
 
 def embedding_lookup(ids: torch.Tensor, packed: torch.Tensor, delta: torch.Tensor, q0: torch.Tensor, D: int,
                      bits: int, groups: int, ws: torch.Tensor, out: Optional[torch.Tensor] = None,
                      accumulate: bool = False) -> torch.Tensor:
     """``qb_embedding_lookup``: int32 ids [T] -> fp32 [T,D]; with ``accumulate`` the rows are added to ``out``."""
-    assert ids.is_cuda and ids.dtype == torch.int32 and ids.is_contiguous()
-    T = ids.numel()
-    V = packed.shape[0]
-    if out is None:
-        assert not accumulate
-        out = torch.empty((T, D), dtype=torch.float32, device=ids.device)
-    _check(lib().qb_embedding_lookup(ids.data_ptr(), T, packed.data_ptr(), delta.data_ptr(), q0.data_ptr(), V, D, bits,
-                                     groups, 1 if accumulate else 0, out.data_ptr(), ws.data_ptr(), ws.numel(),
-                                     _stream()), "qb_embedding_lookup")
-    return out
+    return (_native or _ext()).embedding_lookup(ids, packed, delta, q0, D, bits, groups, ws, out, accumulate)
 
 
 def make_act_desc_array(items):
@@ -290,7 +264,7 @@ def make_act_desc_array(items):
 def quantize_act_batch(items, ws: torch.Tensor) -> None:
     """``qb_quantize_act_batch`` over ``(x, xq, act_scale, rowsum)`` tuples (or a prepared C array)."""
     arr = items if isinstance(items, ctypes.Array) else make_act_desc_array(items)
-    _check(lib().qb_quantize_act_batch(arr, len(arr), ws.data_ptr(), ws.numel(), _stream()), "qb_quantize_act_batch")
+    (_native or _ext()).quantize_act_batch(arr, ws)
 
 
 def make_weight_desc_array(items):
@@ -306,8 +280,7 @@ def make_weight_desc_array(items):
 def quantize_pack_weights_batch(items, ws: torch.Tensor) -> None:
     """``qb_quantize_pack_weights_batch`` over ``(w, bits, groups, packed, delta, q0)`` tuples (or a C array)."""
     arr = items if isinstance(items, ctypes.Array) else make_weight_desc_array(items)
-    _check(lib().qb_quantize_pack_weights_batch(arr, len(arr), ws.data_ptr(), ws.numel(), _stream()),
-           "qb_quantize_pack_weights_batch")
+    (_native or _ext()).quantize_pack_weights_batch(arr, ws)
 
 
 def quantize_pack_weights_noalloc(w: torch.Tensor, bits: int, groups: int, packed: torch.Tensor,
@@ -362,52 +335,29 @@ def gemm(xq: torch.Tensor, act_scale: torch.Tensor, rowsum: torch.Tensor, packed
          ws: torch.Tensor, y: Optional[torch.Tensor] = None, acc_out: Optional[torch.Tensor] = None,
          want_acc: bool = False):
     """``qb_gemm``: returns ``y`` fp32 [M,N] (and the int32 accumulators when ``want_acc``)."""
-    assert xq.is_cuda and xq.dtype == torch.int8 and xq.is_contiguous()
-    M, K = xq.shape
-    y = torch.empty((M, N), dtype=torch.float32, device=xq.device) if y is None else y
     if want_acc and acc_out is None:
-        acc_out = torch.empty((M, N), dtype=torch.int32, device=xq.device)
-    _check(lib().qb_gemm(xq.data_ptr(), act_scale.data_ptr(), rowsum.data_ptr(), packed.data_ptr(),
-                         delta.data_ptr(), q0.data_ptr(), _ptr(bias), M, N, K, bits, groups, y.data_ptr(),
-                         _ptr(acc_out), ws.data_ptr(), ws.numel(), _stream()), "qb_gemm")
-    return (y, acc_out) if (want_acc or acc_out is not None) else y
+        acc_out = torch.empty((xq.shape[0], N), dtype=torch.int32, device=xq.device)
+    y = (_native or _ext()).gemm(0, xq, act_scale, rowsum, packed, delta, q0, bias, N, bits, groups, ws, y, acc_out)
+    return (y, acc_out) if acc_out is not None else y
 
 
 def gemm_bf16(xq: torch.Tensor, act_scale: torch.Tensor, rowsum: torch.Tensor, packed: torch.Tensor,
               delta: torch.Tensor, q0: torch.Tensor, bias: Optional[torch.Tensor], N: int, bits: int, groups: int,
               ws: torch.Tensor, y: Optional[torch.Tensor] = None) -> torch.Tensor:
     """``qb_gemm_bf16``: returns ``y`` bfloat16 [M,N]."""
-    assert xq.is_cuda and xq.dtype == torch.int8 and xq.is_contiguous()
-    M, K = xq.shape
-    y = torch.empty((M, N), dtype=torch.bfloat16, device=xq.device) if y is None else y
-    assert y.dtype == torch.bfloat16 and y.is_contiguous()
-    _check(lib().qb_gemm_bf16(xq.data_ptr(), act_scale.data_ptr(), rowsum.data_ptr(), packed.data_ptr(),
-                              delta.data_ptr(), q0.data_ptr(), _ptr(bias), M, N, K, bits, groups, y.data_ptr(),
-                              ws.data_ptr(), ws.numel(), _stream()), "qb_gemm_bf16")
-    return y
+    return (_native or _ext()).gemm(1, xq, act_scale, rowsum, packed, delta, q0, bias, N, bits, groups, ws, y, None)
 
 
 def gemm_i8(xq: torch.Tensor, act_scale: torch.Tensor, rowsum: torch.Tensor, packed: torch.Tensor,
             delta: torch.Tensor, q0: torch.Tensor, bias: Optional[torch.Tensor], N: int, bits: int, groups: int,
             out_scale: torch.Tensor, ws: torch.Tensor, yq: Optional[torch.Tensor] = None) -> torch.Tensor:
     """``qb_gemm_i8``: returns int8 codes [M,N] on the grid of step ``out_scale`` (device fp32 [1])."""
-    assert xq.is_cuda and xq.dtype == torch.int8 and xq.is_contiguous()
-    assert out_scale.is_cuda and out_scale.dtype == torch.float32
-    M, K = xq.shape
-    yq = torch.empty((M, N), dtype=torch.int8, device=xq.device) if yq is None else yq
-    _check(lib().qb_gemm_i8(xq.data_ptr(), act_scale.data_ptr(), rowsum.data_ptr(), packed.data_ptr(),
-                            delta.data_ptr(), q0.data_ptr(), _ptr(bias), M, N, K, bits, groups, out_scale.data_ptr(),
-                            yq.data_ptr(), ws.data_ptr(), ws.numel(), _stream()), "qb_gemm_i8")
-    return yq
+    return (_native or _ext()).gemm(2, xq, act_scale, rowsum, packed, delta, q0, bias, N, bits, groups, ws, yq, out_scale)
 
 
 def rowsum_i8(xq: torch.Tensor, rowsum: Optional[torch.Tensor] = None) -> torch.Tensor:
     """``qb_rowsum_i8``: int32 row sums of int8 codes [M,K]."""
-    assert xq.is_cuda and xq.dtype == torch.int8 and xq.dim() == 2 and xq.is_contiguous()
-    M, K = xq.shape
-    rowsum = torch.empty(M, dtype=torch.int32, device=xq.device) if rowsum is None else rowsum
-    _check(lib().qb_rowsum_i8(xq.data_ptr(), M, K, rowsum.data_ptr(), _stream()), "qb_rowsum_i8")
-    return rowsum
+    return (_native or _ext()).rowsum_i8(xq, rowsum)
 
 
 @dataclass
@@ -440,7 +390,7 @@ def make_desc_array(descs: Sequence[LinearDesc]):
 def layer_linears(descs, ws: torch.Tensor) -> None:
     """``qb_layer_linears`` over a list of ``LinearDesc`` (or an array from ``make_desc_array``)."""
     arr = descs if isinstance(descs, ctypes.Array) else make_desc_array(descs)
-    _check(lib().qb_layer_linears(arr, len(arr), ws.data_ptr(), ws.numel(), _stream()), "qb_layer_linears")
+    (_native or _ext()).layer_linears(arr, ws)
 
 
 def quantize_act_launch_count(count: int) -> int:
@@ -472,5 +422,5 @@ def layer_linears_bf16(descs, ws: torch.Tensor) -> None:
     """``qb_layer_linears_bf16``: as ``layer_linears``, every ``y`` a bfloat16 [M,N] tensor."""
     if not isinstance(descs, ctypes.Array):
         assert all(d.y.dtype == torch.bfloat16 for d in descs)
-    arr = descs if isinstance(descs, ctypes.Array) else make_desc_array(descs)
-    _check(lib().qb_layer_linears_bf16(arr, len(arr), ws.data_ptr(), ws.numel(), _stream()), "qb_layer_linears_bf16")
+        descs = make_desc_array(descs)
+    (_native or _ext()).layer_linears_bf16(descs, ws)
