@@ -102,10 +102,16 @@ struct Problem {
   int32_t bits;        // bit width of this problem's codes (read by the kernels that mix bit widths)
 };
 
-struct GroupedParams {
-  CUtensorMap tmx[kMaxProblems];  // int8 activations, box 128 B x BT tokens, 128-byte swizzle
-  CUtensorMap tmy[kMaxProblems];  // outputs (fp32 or bfloat16), box 32 neurons x 32 tokens
-  Problem prob[kMaxProblems];
+// What a launch gets, in kernel-parameter space.  P: linears it has room for, O: entries of the visiting order.
+// Two sizes exist: a parameter block of 28 KB costs the host 5.3 us per launch, one of 512 bytes 2.2 us
+// (measured), so a single linear, which is what qb_gemm launches and whose tiles need no order, has its own.
+template <int P, int O>
+struct GroupedParamsT {
+  static constexpr int kProblems = P;
+  static constexpr int kOrder = O;
+  CUtensorMap tmx[P];  // int8 activations, box 128 B x BT tokens, 128-byte swizzle
+  CUtensorMap tmy[P];  // outputs (fp32 or bfloat16), box 32 neurons x 32 tokens
+  Problem prob[P];
   void* ws;
   int32_t count;
   int32_t total_tiles;
@@ -114,9 +120,11 @@ struct GroupedParams {
   // the CTAs instead of dealing them round-robin.
   int32_t total_positions;
   int32_t use_order;
-  uint16_t order[kMaxOrder];
-  uint8_t order_prob[kMaxOrder];  // with `order`: the problem that owns order[p] (spares every role the search)
+  uint16_t order[O];
+  uint8_t order_prob[O];  // with `order`: the problem that owns order[p] (spares every role the search)
 };
+typedef GroupedParamsT<kMaxProblems, kMaxOrder> GroupedParams;
+typedef GroupedParamsT<1, 1> SingleParams;
 
 // BT: tokens per tile (the N of the MMA).  CG: CTAs that share one MMA (1, or 2 = a CTA pair of a cluster:
 // the tile is then 256 neurons x BT tokens, each CTA expands its own 128 weight rows, loads its own half
@@ -236,7 +244,13 @@ struct TileCursor {
     pi = 0;
   }
   // move to the CTA's next tile; false when there is none
-  __device__ __forceinline__ bool next(const GroupedParams& gp) {
+  template <class GP>
+  __device__ __forceinline__ bool next(const GP& gp) {
+    if constexpr (GP::kProblems == 1) {  // one linear: no order, no search
+      p += stride;
+      t = p;
+      return p < gp.total_positions;
+    }
     for (;;) {
       p += stride;
       if (p >= gp.total_positions) return false;
@@ -289,9 +303,9 @@ __device__ __forceinline__ bool epilogue_sync_or(bool pred) {
 // even), Y bfloat16 [M][N]; or that result re-quantized to the 8-bit activation grid of step *out_scale,
 // clamp(round_half_even(y * (1 / out_scale)), -127, 127), Y int8 [M][N].
 enum { kOutF32 = 0, kOutBf16 = 1, kOutI8 = 2 };
-template <int BT, int BITS, int OUT, int CG>
+template <int BT, int BITS, int OUT, int CG, class GP>
 __global__ void __launch_bounds__(kGemmThreads, 1)
-qb_gemm_kernel(const __grid_constant__ GroupedParams gp) {
+qb_gemm_kernel(const __grid_constant__ GP gp) {
   using Cfg = GemmCfg<BT, CG>;
   constexpr int kStages = Cfg::kStages;
   // CG == 2: this CTA's rank in its pair (rank 0 issues the MMAs for both and owns the barriers the issuer
@@ -964,10 +978,10 @@ static qb_status make_y_tensormap(CUtensorMap* tm, void* y, int64_t M, int64_t N
 }
 
 // `grid` CTAs; with CG == 2 they are launched as clusters of two (grid is even).
-template <int BT, int BITS, int OUT, int CG>
-static qb_status launch_group_inst(const GroupedParams& gp, int grid, cudaStream_t stream) {
+template <int BT, int BITS, int OUT, int CG, class GP>
+static qb_status launch_group_inst(const GP& gp, int grid, cudaStream_t stream) {
   using Cfg = GemmCfg<BT, CG>;
-  auto kernel = qb_gemm_kernel<BT, BITS, OUT, CG>;
+  auto kernel = qb_gemm_kernel<BT, BITS, OUT, CG, GP>;
   static std::atomic<bool> attr_set[64] = {};
   int dev = 0;
   QB_CUDA_TRY(cudaGetDevice(&dev));
@@ -991,8 +1005,8 @@ static qb_status launch_group_inst(const GroupedParams& gp, int grid, cudaStream
   return QB_OK;
 }
 
-template <int BT, int OUT, int CG>
-static qb_status launch_group_bits(int bits, const GroupedParams& gp, int grid, cudaStream_t stream) {
+template <int BT, int OUT, int CG, class GP>
+static qb_status launch_group_bits(int bits, const GP& gp, int grid, cudaStream_t stream) {
   switch (bits) {
     case 2: return launch_group_inst<BT, 2, OUT, CG>(gp, grid, stream);
     case 3: return launch_group_inst<BT, 3, OUT, CG>(gp, grid, stream);
@@ -1048,8 +1062,73 @@ static qb_status validate_gemm(const int8_t* xq, const float* act_scale, const i
   return QB_OK;
 }
 
-// One launch over descriptors d[idx[0..count)] (count <= kMaxProblems), all with the same bit width, on at
-// most `max_ctas` CTAs.
+// Tiles of unequal length over the CTA groups: longest first, each to the least loaded group (a heap of loads:
+// the 48-linear stack at M = 128 has 648 tiles for 148 groups; scanning all groups for every tile took the
+// host 80 us of the call's 100, the heap 15).  Fills gp.order; leaves it unused when the tiles are all alike (the
+// identity order is as good) or too many for the table.
+static void balance_tiles(GroupedParams& gp, int tiles, int grid, bool mixed_bits) {
+  bool uniform = !mixed_bits;
+  for (int i = 1; i < gp.count; ++i) uniform = uniform && gp.prob[i].K == gp.prob[0].K;
+  if (uniform || tiles > kMaxOrder || tiles >= (int)kNoTile) return;
+  constexpr int kEpilogueCost = 5;  // a tile's fixed cost in units of one K block
+  // the tiles of a problem cost the same: sort the problems, not the tiles
+  int by_cost[kMaxProblems], cost[kMaxProblems];
+  for (int i = 0; i < gp.count; ++i) {
+    by_cost[i] = i;
+    // measured at M = 128: a K block of 3-bit weights takes about 1.2 times, of 8-bit weights about 1.4
+    // times as long as one of 2- or 4-bit weights
+    cost[i] = (gp.prob[i].K / kBlockK + kEpilogueCost) * (gp.prob[i].bits == 3 ? 12 : (gp.prob[i].bits == 8 ? 14 : 10));
+  }
+  std::stable_sort(by_cost, by_cost + gp.count, [&](int a, int b) { return cost[a] > cost[b]; });
+  struct Dealt {
+    uint16_t tile, group;
+    uint16_t rank;  // the group's how-manieth tile
+    uint8_t prob;
+  };
+  std::vector<Dealt> dealt(tiles);
+  std::vector<int> len(grid, 0);
+  // least loaded group first, the lowest index among equals
+  std::vector<uint64_t> heap(grid);
+  for (int g = 0; g < grid; ++g) heap[g] = (uint64_t)g;
+  const auto above = [](uint64_t a, uint64_t b) { return a > b; };
+  int max_len = 0, n = 0;
+  for (int q = 0; q < gp.count; ++q) {
+    const int i = by_cost[q];
+    const Problem& p = gp.prob[i];
+    for (int j = 0; j < p.n_tiles * p.m_tiles; ++j) {
+      std::pop_heap(heap.begin(), heap.end(), above);
+      const int g = (int)(heap.back() & 0xFFFFFFu);
+      heap.back() += (uint64_t)cost[i] << 24;
+      std::push_heap(heap.begin(), heap.end(), above);
+      dealt[n++] = {(uint16_t)(p.tile_begin + j), (uint16_t)g, (uint16_t)len[g], (uint8_t)i};
+      max_len = std::max(max_len, ++len[g]);
+    }
+  }
+  if ((int64_t)max_len * grid > kMaxOrder) return;
+  std::fill(gp.order, gp.order + max_len * grid, kNoTile);
+  // Each CTA visits its own list shortest tile first: the short tile's epilogue then runs under the
+  // long tile's main loop and the launch's first weight reads are spread over more tiles (measured
+  // on a 6-linear mixed stack at M = 128: 5 % less than longest first).
+  for (const Dealt& d : dealt) {
+    const int at = (len[d.group] - 1 - d.rank) * grid + d.group;
+    gp.order[at] = d.tile;
+    gp.order_prob[at] = d.prob;
+  }
+  gp.total_positions = max_len * grid;
+  gp.use_order = 1;
+}
+
+template <int OUT, class GP>
+static qb_status launch_group_out(int bits, int bt, int cg, const GP& gp, int grid, cudaStream_t stream) {
+  if constexpr (GP::kProblems > 1)
+    if (bits == 0) return launch_group_inst<128, 0, OUT, 1>(gp, grid, stream);
+  if (cg == 2) return launch_group_bits<256, OUT, 2>(bits, gp, 2 * grid, stream);
+  return bt == 256 ? launch_group_bits<256, OUT, 1>(bits, gp, grid, stream)
+                   : launch_group_bits<128, OUT, 1>(bits, gp, grid, stream);
+}
+
+// One launch over descriptors d[idx[0..count)] (count <= GP::kProblems), on at most `max_ctas` CTAs.
+template <class GP>
 static qb_status launch_group(const qb_linear_desc* d, const int* idx, int count, int32_t* acc_out, void* ws,
                               int max_ctas, cudaStream_t stream, int out,
                               const float* const* out_scales = nullptr) {
@@ -1064,8 +1143,7 @@ static qb_status launch_group(const qb_linear_desc* d, const int* idx, int count
     bt = 128;
   }
   const int group_n = kTileN * cg;
-  GroupedParams gp;
-  memset(&gp, 0, sizeof(gp));
+  GP gp;  // every field that the kernel reads for `count` linears is written below
   gp.ws = ws;
   gp.count = count;
   int tile = 0;
@@ -1107,70 +1185,12 @@ static qb_status launch_group(const qb_linear_desc* d, const int* idx, int count
   const int grid = tile < max_groups ? tile : max_groups;  // CTA groups
   gp.total_positions = tile;
   gp.use_order = 0;
-  // Tiles of different problems differ in length (K blocks).  When the launch is small enough for the
-  // table, deal the tiles longest first to the least loaded CTA instead of round-robin.
-  {
-    bool uniform = bits != 0;
-    for (int i = 1; i < count; ++i) uniform = uniform && gp.prob[i].K == gp.prob[0].K;
-    if (!uniform && tile <= kMaxOrder && tile < (int)kNoTile) {
-      constexpr int kEpilogueCost = 5;  // a tile's fixed cost in units of one K block
-      std::vector<int> ids(tile), cost(tile);
-      for (int i = 0, t = 0; i < count; ++i)
-        for (int j = 0; j < gp.prob[i].n_tiles * gp.prob[i].m_tiles; ++j, ++t) {
-          ids[t] = t;
-          // measured at M = 128: a K block of 3-bit weights takes about 1.2 times, of 8-bit weights about 1.4
-          // times as long as one of 2- or 4-bit weights
-          cost[t] = (gp.prob[i].K / kBlockK + kEpilogueCost) * (gp.prob[i].bits == 3 ? 12 : (gp.prob[i].bits == 8 ? 14 : 10));
-        }
-      std::stable_sort(ids.begin(), ids.end(), [&](int a, int b) { return cost[a] > cost[b]; });
-      std::vector<std::vector<int>> lists(grid);
-      std::vector<long long> load(grid, 0);
-      size_t max_len = 0;
-      for (int t : ids) {
-        int best = 0;
-        for (int c = 1; c < grid; ++c)
-          if (load[c] < load[best]) best = c;
-        lists[best].push_back(t);
-        load[best] += cost[t];
-        if (lists[best].size() > max_len) max_len = lists[best].size();
-      }
-      if (max_len * (size_t)grid <= (size_t)kMaxOrder) {
-        // Each CTA visits its own list shortest tile first: the short tile's epilogue then runs under the
-        // long tile's main loop and the launch's first weight reads are spread over more tiles (measured
-        // on a 6-linear mixed stack at M = 128: 5 % less than longest first).
-        for (size_t i = 0; i < max_len; ++i)
-          for (int c = 0; c < grid; ++c)
-            gp.order[i * grid + c] = i < lists[c].size() ? (uint16_t)lists[c][lists[c].size() - 1 - i] : kNoTile;
-        // the owner of every listed tile, so that the kernel's roles need not search for it at every tile
-        for (int q = 0; q < (int)(max_len * grid); ++q) {
-          if (gp.order[q] == kNoTile) continue;
-          int pi = 0;
-          while (pi + 1 < count && (int)gp.order[q] >= gp.prob[pi + 1].tile_begin) ++pi;
-          gp.order_prob[q] = (uint8_t)pi;
-        }
-        gp.total_positions = (int32_t)(max_len * grid);
-        gp.use_order = 1;
-      }
-    }
+  if constexpr (GP::kProblems > 1) balance_tiles(gp, tile, grid, bits == 0);
+  switch (out) {
+    case kOutBf16: return launch_group_out<kOutBf16>(bits, bt, cg, gp, grid, stream);
+    case kOutI8: return launch_group_out<kOutI8>(bits, bt, cg, gp, grid, stream);
+    default: return launch_group_out<kOutF32>(bits, bt, cg, gp, grid, stream);
   }
-  if (bits == 0) {
-    if (out == kOutBf16) return launch_group_inst<128, 0, kOutBf16, 1>(gp, grid, stream);
-    if (out == kOutI8) return launch_group_inst<128, 0, kOutI8, 1>(gp, grid, stream);
-    return launch_group_inst<128, 0, kOutF32, 1>(gp, grid, stream);
-  }
-  if (cg == 2) {
-    if (out == kOutBf16) return launch_group_bits<256, kOutBf16, 2>(bits, gp, 2 * grid, stream);
-    if (out == kOutI8) return launch_group_bits<256, kOutI8, 2>(bits, gp, 2 * grid, stream);
-    return launch_group_bits<256, kOutF32, 2>(bits, gp, 2 * grid, stream);
-  }
-  if (out == kOutBf16)
-    return bt == 256 ? launch_group_bits<256, kOutBf16, 1>(bits, gp, grid, stream)
-                     : launch_group_bits<128, kOutBf16, 1>(bits, gp, grid, stream);
-  if (out == kOutI8)
-    return bt == 256 ? launch_group_bits<256, kOutI8, 1>(bits, gp, grid, stream)
-                     : launch_group_bits<128, kOutI8, 1>(bits, gp, grid, stream);
-  return bt == 256 ? launch_group_bits<256, kOutF32, 1>(bits, gp, grid, stream)
-                   : launch_group_bits<128, kOutF32, 1>(bits, gp, grid, stream);
 }
 
 struct StackGroup {
@@ -1223,7 +1243,10 @@ static qb_status launch_stack(const qb_linear_desc* d, int count, void* ws, int 
   std::vector<StackGroup> groups;
   plan_stack(d, count, sm_count, order, groups);
   for (const StackGroup& g : groups) {
-    qb_status st = launch_group(d, order.data() + g.begin, g.count, nullptr, ws, sm_count, stream, out, out_scales);
+    const int* idx = order.data() + g.begin;
+    qb_status st = g.count == 1
+                       ? launch_group<SingleParams>(d, idx, 1, nullptr, ws, sm_count, stream, out, out_scales)
+                       : launch_group<GroupedParams>(d, idx, g.count, nullptr, ws, sm_count, stream, out, out_scales);
     if (st != QB_OK) return st;
   }
   return QB_OK;
@@ -1256,7 +1279,7 @@ static qb_status gemm_entry(const int8_t* xq, const float* act_scale, const int3
   d.groups = groups;
   d.y = static_cast<float*>(y);
   const int idx = 0;
-  return qb::launch_group(&d, &idx, 1, acc_out, ws, sms, (cudaStream_t)cuda_stream, out, out_scale ? &out_scale : nullptr);
+  return qb::launch_group<qb::SingleParams>(&d, &idx, 1, acc_out, ws, sms, (cudaStream_t)cuda_stream, out, out_scale ? &out_scale : nullptr);
 }
 
 static qb_status stack_entry(const char* who, const qb_linear_desc* descs, int32_t count, void* ws, size_t ws_bytes,
