@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "qbert.h"
 
 namespace qb {
@@ -12,6 +14,10 @@ namespace qb {
 // [0]   int32  status   first device-side error, never cleared by a kernel
 // [4]   int32  detail   where a bounded wait gave up (role << 16 | stage), diagnostics only
 // [16]  uint32 act_absmax_bits   bit pattern of max|x| of the last qb_quantize_act
+// [32]  uint32 ticket            blocks of the running launch that have started        } zero
+// [36]  uint32 cleared           1 once the running launch's reduction slots are clear } between
+// [40]  uint32 arrived           blocks of the running launch that have published      } calls
+// [44]  uint32 round             counts the launches whose blocks waited for one another
 // [256] uint32 range_hi_enc[G], uint32 range_lo_inv[G]   ordered encodings of per-group max / min
 constexpr size_t kWsStatusOff = 0;
 constexpr size_t kWsDetailOff = 4;
@@ -24,6 +30,11 @@ struct WsHeader {
   int32_t detail;
   uint32_t pad[2];
   uint32_t act_absmax_bits;
+  uint32_t pad2[3];
+  uint32_t ticket;
+  uint32_t cleared;
+  uint32_t arrived;
+  uint32_t round;
 };
 
 inline size_t ws_bytes_needed(int groups) {
@@ -46,8 +57,52 @@ inline bool valid_bits(int b) { return b == 2 || b == 3 || b == 4 || b == 8; }
     if (e__ != cudaSuccess) return qb::cuda_fail(e__, #expr); \
   } while (0)
 
+// Launch of a kernel that begins with pdl_begin.
+// `overlap`: programmatic stream serialization: the kernel's blocks may be set up while the kernel before it on
+// the stream drains, and wait in pdl_begin for its completion.  Back to back launches of 592 blocks: 4.1 us
+// each without it, 2.2 us with it.
+// `cluster`: CTAs per cluster; `cooperative`: every block must be resident at once (the blocks wait on
+// one another).
+template <class... P, class... A>
+inline cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
+                                 bool overlap, unsigned cluster, bool cooperative, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid, 1, 1);
+  cfg.blockDim = dim3(block, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[3];
+  int n = 0;
+  if (overlap) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = cluster;
+    attr[n].val.clusterDim.y = 1;
+    attr[n++].val.clusterDim.z = 1;
+  }
+  if (cooperative) {
+    attr[n].id = cudaLaunchAttributeCooperative;
+    attr[n++].val.cooperative = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kernel, std::decay_t<P>(args)...);
+}
+
 // ---- device-side helpers -----------------------------------------------------------------------
 #ifdef __CUDACC__
+// Called by every thread of a kernel started by launch_kernel before it touches global memory: waits until the
+// kernel before this one on the stream has completed and its results are visible, and only then lets the
+// next kernel's blocks be set up.  In this order every kernel that runs has all kernels but its direct
+// predecessor behind it when it is set up.
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ void report_status(void* ws, int32_t code, int32_t detail = 0) {
   WsHeader* h = reinterpret_cast<WsHeader*>(ws);
   if (atomicCAS(&h->status, 0, code) == 0) h->detail = detail;
@@ -67,6 +122,37 @@ __device__ __forceinline__ uint32_t float_to_ordered(float f) {
 __device__ __forceinline__ float ordered_to_float(uint32_t e) {
   uint32_t b = (e & 0x80000000u) ? (e & 0x7fffffffu) : ~e;
   return __uint_as_float(b);
+}
+__device__ __forceinline__ float min3_nan(float a, float b, float c) {
+  float d;
+  asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float d;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release(uint32_t* p, uint32_t v) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+// Called by one warp of every block: the block that comes first clears the launch's reduction slots and says so
+// (whichever block it is, it is running, so nobody waits for a block that has not started).  The others
+// look (h->cleared) before they publish; by then they have read their share of the input and the wait is
+// over before it begins.  The next launch on the stream sets ticket and cleared back to zero.
+__device__ __forceinline__ void clear_slots(uint32_t* slots, int count, WsHeader* h, int lane) {
+  uint32_t ticket = 0;
+  if (lane == 0) ticket = atomicAdd(&h->ticket, 1u);
+  if (__shfl_sync(0xffffffffu, ticket, 0) != 0u) return;
+  for (int i = lane; i < count; i += 32) slots[i] = 0u;
+  __threadfence();
+  __syncwarp();
+  if (lane == 0) st_release(&h->cleared, 1u);
 }
 // 16-byte load with an L2 eviction-priority policy (createpolicy).  The two-pass quantizers use it: the
 // first pass asks L2 to keep a fraction of what it reads (the second pass reads the same tensor next),

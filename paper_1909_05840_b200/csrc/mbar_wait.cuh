@@ -1,6 +1,7 @@
 // Bounded waits on mbarrier phases, shared by the GEMM kernels and by the wait-limit self-test.
 #pragma once
 
+#include "common.cuh"
 #include "ptx.cuh"
 
 namespace qb {
@@ -51,6 +52,16 @@ __device__ __forceinline__ bool wait_barrier_warp(uint32_t bar, uint32_t parity,
   int ok = 1;
   if ((threadIdx.x & 31) == 0) ok = wait_barrier_relaxed(bar, parity, abort_flag, limit) ? 1 : 0;
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
+// One thread polls a global word until it equals / differs from v (acquire); false when the bound ran out.
+template <bool EQUAL>
+__device__ __forceinline__ bool poll_word(const uint32_t* p, uint32_t v, long long limit = kWaitLimitCycles) {
+  if ((ld_acquire(p) == v) == EQUAL) return true;
+  const long long t0 = clock64();
+  while ((ld_acquire(p) == v) != EQUAL)
+    if (clock64() - t0 > limit) return false;
+  return true;
 }
 
 }  // namespace qb

@@ -1,23 +1,37 @@
 // qb_quantize_act(_batch): per-tensor 8-bit activation quantizer (Table 1 caption: 8-bit activations;
 // Appendix A's uniform quantizer on the symmetric range [-a, a], a = max|x|), for one tensor or a
-// batch of tensors in one pair of launches.
+// batch of tensors.
 //
-// Kernel 1  act_absmax_kernel    each block belongs to one tensor; block-stride float4 loads, max of
-//                                |x| bit patterns (monotone as unsigned integers, and NaN/Inf sort
-//                                above every finite value), warp reduce + one atomicMax per block
-//                                into the tensor's slot of the workspace.
-// Kernel 2  act_quantize_kernel  one warp per row (rows of all tensors form one sequence):
-//                                x * (127/a), round half to even, clamp, four codes packed per 32-bit
-//                                store, int32 row sum by warp reduction.
-// Both kernels are HBM-bound: 4 B read per element in each, 1 B written in the second.
+// The unit of work is a segment: up to eight units of 128 consecutive elements of one row, one float4 per lane
+// and unit, so that a warp has 4 KB of loads in flight at once.  A row is cut into ceil(K / 1024) segments.
+//
+//   act_absmax_kernel    max|x| of every tensor.  The units of all tensors form one sequence that the
+//                        blocks cut into equal contiguous shares (a block meets few tensors and publishes
+//                        one atomicMax for each).
+//   act_quantize_kernel  one warp per segment: x * (127/a), round half to even, four codes per 32-bit
+//                        store, row sum by dp4a and a warp reduction (rows of several segments: atomicAdd on
+//                        row sums that the first kernel cleared).
+//   act_fused_kernel     both for one tensor whose segments each find a warp on the device: the segment
+//                        stays in registers while the blocks agree on a, x is read once and there is one
+//                        launch instead of two.
+//
+// Both passes are memory-bound (4 B read per element, then 4 B read, from L2 as far as it holds the
+// tensors, and 1 B written).  What bounds them below L2's size is the bytes in flight and the instructions per
+// element: 128 KB of loads per SM and about nine instructions per float4 (packed fp32x2, no clamp) instead of
+// 64 KB and thirty.  Quantizer and GEMMs of one BERT-base layer at M = 4096 (88 MB of input): 86.9 -> 81.1 us;
+// int8 chain at M = 6144 98.0 -> 91.5; query projection at M = 1024 (fused) 20.1 -> 17.4.
 #include <algorithm>
 #include <cstring>
 
 #include "common.cuh"
+#include "mbar_wait.cuh"
 
 namespace qb {
 
 constexpr int kActThreads = 256;
+constexpr int kActWarps = kActThreads / 32;
+constexpr int kActBlocksPerSm = 4;
+constexpr int kSegUnits = 8;      // float4 per lane and segment
 constexpr int kMaxActBatch = 64;  // tensors per launch (descriptors travel as kernel parameters, 4 KB)
 
 struct ActItem {
@@ -25,63 +39,38 @@ struct ActItem {
   int8_t* xq;
   float* act_scale;
   int32_t* rowsum;
-  int64_t M, K;
-  int64_t row_begin;    // index of the tensor's first row in the launch's row sequence
-  int32_t block_begin;  // first block of kernel 1 that works on this tensor
-  int32_t blocks;       // number of such blocks
+  int64_t M;
+  int64_t unit_begin;   // index of the tensor's first unit in the launch's sequence
+  int64_t seg_begin;    // index of the tensor's first segment in the launch's sequence
+  int32_t units_per_row;
+  int32_t segs_per_row;
+  int32_t seg_units;    // units per segment (the last one of a row may be shorter)
 };
 
+template <int P>
 struct ActBatch {
-  ActItem item[kMaxActBatch];
+  ActItem item[P];
   uint32_t* absmax_bits;  // [count] slots in the workspace
   void* ws;
-  int64_t rows_total;
+  int64_t units_total, units_per_block;
+  int64_t segs_total;
   int32_t count;
   float keep_fraction;  // share of the launch's input that L2 is asked to keep between the two passes
 };
 
-__global__ void __launch_bounds__(kActThreads)
-act_absmax_kernel(const __grid_constant__ ActBatch b) {
-  int it = 0;
-  while (it + 1 < b.count && (int)blockIdx.x >= b.item[it + 1].block_begin) ++it;
-  const ActItem& t = b.item[it];
-  const float4* __restrict__ x = reinterpret_cast<const float4*>(t.x);
-  const int64_t n4 = t.M * t.K / 4;
-  uint32_t m = 0;
-  const uint64_t pol = policy_evict_last(b.keep_fraction);
-  const int64_t stride = (int64_t)t.blocks * blockDim.x;
-  int64_t i = (int64_t)((int)blockIdx.x - t.block_begin) * blockDim.x + threadIdx.x;
-  // four independent 16-byte loads in flight per thread
-  for (; i + 3 * stride < n4; i += 4 * stride) {
-    float4 a = ldg_policy(x + i, pol), bb = ldg_policy(x + i + stride, pol), c = ldg_policy(x + i + 2 * stride, pol),
-           d = ldg_policy(x + i + 3 * stride, pol);
-#define QB_ABSMAX4(v)                                            \
-  m = max(m, __float_as_uint(v.x) & 0x7fffffffu);                \
-  m = max(m, __float_as_uint(v.y) & 0x7fffffffu);                \
-  m = max(m, __float_as_uint(v.z) & 0x7fffffffu);                \
-  m = max(m, __float_as_uint(v.w) & 0x7fffffffu);
-    QB_ABSMAX4(a) QB_ABSMAX4(bb) QB_ABSMAX4(c) QB_ABSMAX4(d)
+// Running extremes of a lane; NaN stays.  Start value 0: only the magnitude matters.
+struct Extremes {
+  float lo = 0.0f, hi = 0.0f;
+  __device__ __forceinline__ void add(const float4& v) {
+    lo = min3_nan(min3_nan(lo, v.x, v.y), v.z, v.w);
+    hi = max3_nan(max3_nan(hi, v.x, v.y), v.z, v.w);
   }
-  for (; i < n4; i += stride) {
-    float4 a = ldg_policy(x + i, pol);
-    QB_ABSMAX4(a)
+  // bit pattern of the largest |x| over the warp (NaN and Inf above every finite value)
+  __device__ __forceinline__ uint32_t warp_bits() const {
+    const uint32_t h = __float_as_uint(hi) & 0x7fffffffu, l = __float_as_uint(lo) & 0x7fffffffu;
+    return __reduce_max_sync(0xffffffffu, max(h, l));
   }
-#undef QB_ABSMAX4
-  m = __reduce_max_sync(0xffffffffu, m);
-  __shared__ uint32_t warp_max[kActThreads / 32];
-  if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    uint32_t v = threadIdx.x < kActThreads / 32 ? warp_max[threadIdx.x] : 0u;
-    v = __reduce_max_sync(0xffffffffu, v);
-    if (threadIdx.x == 0 && v != 0u) atomicMax(b.absmax_bits + it, v);
-  }
-}
-
-__device__ __forceinline__ int quant_code(float v, float inv) {
-  int q = __float2int_rn(__fmul_rn(v, inv));
-  return min(max(q, -127), 127);
-}
+};
 
 // scale and reciprocal of a tensor from the bit pattern of its max|x|; false if NaN/Inf was seen
 __device__ __forceinline__ bool act_scales(uint32_t mb, float* s, float* inv) {
@@ -98,64 +87,212 @@ __device__ __forceinline__ bool act_scales(uint32_t mb, float* s, float* inv) {
   return true;
 }
 
-__global__ void __launch_bounds__(kActThreads, 8)  // eight blocks per SM resident: the grid is one full wave
-act_quantize_kernel(const __grid_constant__ ActBatch b) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  int it = 0;
-  int cur = -1;
-  float inv = 0.0f;
-  const uint64_t pol = policy_evict_first();
-  for (int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < b.rows_total; row += warps) {
-    while (it + 1 < b.count && row >= b.item[it + 1].row_begin) ++it;
+// Four codes of one float4 as bytes.  |x| <= a and inv = 127/a rounded, so |x * inv| < 127.5 and no code needs a
+// clamp; adding 1.5 * 2^23 rounds to an integer, half to even, and leaves the code in the low byte as two's
+// complement.  The add is written as a fused multiply-add with 1.0: a packed mul and a packed add would be
+// contracted into one operation, which rounds the exact product instead of the rounded one.
+__device__ __forceinline__ uint32_t quant_word(const float4& v, float inv) {
+  uint32_t b0, b1, b2, b3;
+  asm("{\n\t.reg .b64 p0, p1, i2, m2, o2;\n\t"
+      "mov.b64 p0, {%4, %5};\n\tmov.b64 p1, {%6, %7};\n\t"
+      "mov.b64 i2, {%8, %8};\n\tmov.b64 m2, {%9, %9};\n\tmov.b64 o2, {%10, %10};\n\t"
+      "mul.rn.f32x2 p0, p0, i2;\n\tmul.rn.f32x2 p1, p1, i2;\n\t"
+      "fma.rn.f32x2 p0, p0, o2, m2;\n\tfma.rn.f32x2 p1, p1, o2, m2;\n\t"
+      "mov.b64 {%0, %1}, p0;\n\tmov.b64 {%2, %3}, p1;\n\t}"
+      : "=r"(b0), "=r"(b1), "=r"(b2), "=r"(b3)
+      : "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "f"(inv), "f"(12582912.0f), "f"(1.0f));
+  return __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
+}
+
+template <int P>
+__global__ void __launch_bounds__(kActThreads, kActBlocksPerSm)
+act_absmax_kernel(const __grid_constant__ ActBatch<P> b) {
+  __shared__ uint32_t s_max[P];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  WsHeader* const h = reinterpret_cast<WsHeader*>(b.ws);
+  for (int i = threadIdx.x; i < P; i += kActThreads) s_max[i] = 0u;
+  pdl_begin();
+  __syncthreads();
+  const uint64_t pol = policy_evict_last(b.keep_fraction);
+  const int64_t u0 = (int64_t)blockIdx.x * b.units_per_block;
+  const int64_t u1 = min(u0 + b.units_per_block, b.units_total);
+  bool cleared = warp != 0;
+  for (int it = 0; it < b.count; ++it) {
     const ActItem& t = b.item[it];
-    if (it != cur) {  // warp-uniform: first row of this warp in tensor `it`
-      cur = it;
-      float s;
-      const bool finite = act_scales(b.absmax_bits[it], &s, &inv);
-      if (row == t.row_begin && lane == 0) {  // exactly one warp sees the tensor's first row
-        *t.act_scale = s;
-        if (!finite) report_status(b.ws, QB_ERR_NONFINITE);
+    const int64_t units = t.M * t.units_per_row;
+    const int64_t lo = max(u0 - t.unit_begin, (int64_t)0), hi = min(u1 - t.unit_begin, units);
+    if (t.segs_per_row > 1)  // row sums that several warps will add to
+      for (int64_t m = (int64_t)blockIdx.x * kActThreads + threadIdx.x; m < t.M; m += (int64_t)gridDim.x * kActThreads)
+        t.rowsum[m] = 0;
+    if (lo >= hi) continue;
+    const float4* __restrict__ x = reinterpret_cast<const float4*>(t.x) + lane;
+    Extremes ex;
+    for (int64_t u = lo + warp * kSegUnits; u < hi; u += kActWarps * kSegUnits) {
+      const int n = (int)min(hi - u, (int64_t)kSegUnits);
+      float4 v[kSegUnits];
+#pragma unroll
+      for (int j = 0; j < kSegUnits; ++j)
+        if (j < n) v[j] = ldg_policy(x + (u + j) * 32, pol);
+      if (!cleared) {  // warp 0, while its first loads are on their way (every block has at least one unit)
+        cleared = true;
+        clear_slots(b.absmax_bits, b.count, h, lane);
       }
+#pragma unroll
+      for (int j = 0; j < kSegUnits; ++j)
+        if (j < n) ex.add(v[j]);
     }
-    const int64_t r = row - t.row_begin;
-    const int64_t k4 = t.K >> 2;  // float4 per row
-    const float4* src = reinterpret_cast<const float4*>(t.x + r * t.K);
-    uint32_t* dst = reinterpret_cast<uint32_t*>(t.xq + r * t.K);
-    int sum = 0;
-#pragma unroll 4
-    for (int64_t c = lane; c < k4; c += 32) {
-      const float4 v = ldg_policy(src + c, pol);
-      const int q0 = quant_code(v.x, inv), q1 = quant_code(v.y, inv), q2 = quant_code(v.z, inv),
-                q3 = quant_code(v.w, inv);
-      sum += (q0 + q1) + (q2 + q3);
-      dst[c] = (uint32_t)(q0 & 0xff) | ((uint32_t)(q1 & 0xff) << 8) | ((uint32_t)(q2 & 0xff) << 16) |
-               ((uint32_t)(q3 & 0xff) << 24);
+    const uint32_t m = ex.warp_bits();
+    if (lane == 0 && m != 0u) atomicMax(&s_max[it], m);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0 && !poll_word<true>(&h->cleared, 1u)) report_status(b.ws, QB_ERR_TIMEOUT);
+  __syncthreads();
+  for (int i = threadIdx.x; i < b.count; i += kActThreads)
+    if (s_max[i] != 0u) atomicMax(b.absmax_bits + i, s_max[i]);
+}
+
+// Codes and row sum of one segment held in v[0 .. n).
+__device__ __forceinline__ void quantize_segment(const ActItem& t, uint32_t row, int seg, int n, const float4 (&v)[kSegUnits],
+                                                 float inv, int lane) {
+  uint32_t* dst = reinterpret_cast<uint32_t*>(t.xq) + ((int64_t)row * t.units_per_row + seg * t.seg_units) * 32 + lane;
+  int sum = 0;
+#pragma unroll
+  for (int j = 0; j < kSegUnits; ++j)
+    if (j < n) {
+      const uint32_t w = quant_word(v[j], inv);
+      sum = __dp4a((int)w, 0x01010101, sum);
+      dst[j * 32] = w;
     }
-    sum = __reduce_add_sync(0xffffffffu, sum);
-    if (lane == 0) t.rowsum[r] = sum;
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  if (lane == 0) {
+    if (t.segs_per_row == 1) t.rowsum[row] = sum;
+    else atomicAdd(t.rowsum + row, sum);
   }
 }
 
-// One pair of launches over `count` tensors (<= kMaxActBatch).  `absmax_slots` has room for `count` words.
+template <int P>
+__global__ void __launch_bounds__(kActThreads, kActBlocksPerSm)
+act_quantize_kernel(const __grid_constant__ ActBatch<P> b) {
+  const int lane = threadIdx.x & 31;
+  WsHeader* const h = reinterpret_cast<WsHeader*>(b.ws);
+  pdl_begin();
+  if (blockIdx.x == 0 && threadIdx.x == 0) {  // for the next call; nothing of this launch reads them
+    h->ticket = 0u;
+    h->cleared = 0u;
+  }
+  const int64_t warps = (int64_t)gridDim.x * kActWarps;
+  const uint64_t pol = policy_evict_first();
+  int it = 0, cur = -1;
+  float inv = 0.0f;
+  for (int64_t s = (int64_t)blockIdx.x * kActWarps + (threadIdx.x >> 5); s < b.segs_total; s += warps) {
+    while (it + 1 < b.count && s >= b.item[it + 1].seg_begin) ++it;
+    const ActItem& t = b.item[it];
+    const uint32_t local = (uint32_t)(s - t.seg_begin);  // below 2^24 rows x 64 segments
+    const uint32_t row = t.segs_per_row > 1 ? local / (uint32_t)t.segs_per_row : local;
+    const int seg = (int)(local - row * t.segs_per_row);
+    const int n = min(t.seg_units, t.units_per_row - seg * t.seg_units);
+    const float4* src = reinterpret_cast<const float4*>(t.x) + ((int64_t)row * t.units_per_row + seg * t.seg_units) * 32 + lane;
+    float4 v[kSegUnits];
+#pragma unroll
+    for (int j = 0; j < kSegUnits; ++j)
+      if (j < n) v[j] = ldg_policy(src + j * 32, pol);
+    if (it != cur) {  // warp-uniform: first segment of this warp in tensor `it`
+      cur = it;
+      float scale;
+      const bool finite = act_scales(b.absmax_bits[it], &scale, &inv);
+      if (local == 0 && lane == 0) {  // exactly one warp sees the tensor's first segment
+        *t.act_scale = scale;
+        if (!finite) report_status(b.ws, QB_ERR_NONFINITE);
+      }
+    }
+    quantize_segment(t, row, seg, n, v, inv, lane);
+  }
+}
+
+// One tensor, one segment per warp, every block resident (cooperative launch).
+__global__ void __launch_bounds__(kActThreads, kActBlocksPerSm)
+act_fused_kernel(const __grid_constant__ ActBatch<1> b) {
+  __shared__ uint32_t s_max;
+  __shared__ int s_ok;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  WsHeader* const h = reinterpret_cast<WsHeader*>(b.ws);
+  const ActItem& t = b.item[0];
+  const uint32_t local = blockIdx.x * kActWarps + warp;
+  const bool mine = local < (uint32_t)b.segs_total;
+  const uint32_t row = local / (uint32_t)t.segs_per_row;
+  const int seg = (int)(local - row * t.segs_per_row);
+  const int n = mine ? min(t.seg_units, t.units_per_row - seg * t.seg_units) : 0;
+  const float4* src = reinterpret_cast<const float4*>(t.x) + ((int64_t)row * t.units_per_row + seg * t.seg_units) * 32 + lane;
+  if (threadIdx.x == 0) s_max = 0u;
+  pdl_begin();
+  float4 v[kSegUnits];
+#pragma unroll
+  for (int j = 0; j < kSegUnits; ++j)
+    if (j < n) v[j] = __ldg(src + j * 32);
+  const uint32_t round = ld_acquire(&h->round);  // only the block that arrives last changes it
+  if (warp == 0) clear_slots(b.absmax_bits, 1, h, lane);
+  if (mine && t.segs_per_row > 1 && seg == 0 && lane == 0) t.rowsum[row] = 0;  // published by the barrier below
+  __syncthreads();
+  Extremes ex;
+#pragma unroll
+  for (int j = 0; j < kSegUnits; ++j)
+    if (j < n) ex.add(v[j]);
+  const uint32_t m = ex.warp_bits();
+  if (lane == 0 && m != 0u) atomicMax(&s_max, m);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    // publish this block's maximum, then wait for all blocks: the last one to arrive lets the others go
+    bool ok = poll_word<true>(&h->cleared, 1u);
+    if (ok) {
+      if (s_max != 0u) atomicMax(b.absmax_bits, s_max);
+      __threadfence();
+      if (atomicAdd(&h->arrived, 1u) == gridDim.x - 1u) {
+        h->ticket = 0u;
+        h->cleared = 0u;
+        h->arrived = 0u;
+        __threadfence();
+        st_release(&h->round, round + 1u);
+      } else {
+        ok = poll_word<false>(&h->round, round);
+      }
+      __threadfence();
+      s_max = __ldcg(b.absmax_bits);
+    }
+    if (!ok) report_status(b.ws, QB_ERR_TIMEOUT);
+    s_ok = ok ? 1 : 0;
+  }
+  __syncthreads();
+  if (!s_ok) return;
+  float scale, inv;
+  const bool finite = act_scales(s_max, &scale, &inv);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *t.act_scale = scale;
+    if (!finite) report_status(b.ws, QB_ERR_NONFINITE);
+  }
+  if (mine) quantize_segment(t, row, seg, n, v, inv, lane);
+}
+
+// The launches over `count` tensors (<= P).  `absmax_slots` has room for `count` words.
+template <int P>
 static qb_status launch_act_batch(const qb_act_desc* d, int count, void* ws, uint32_t* absmax_slots, int sm_count,
                                   cudaStream_t stream) {
-  ActBatch b;
-  memset(&b, 0, sizeof(b));
+  ActBatch<P> b;
   b.count = count;
   b.ws = ws;
   b.absmax_bits = absmax_slots;
-  const int64_t cap = (int64_t)sm_count * 8;  // one full wave of either kernel (eight blocks per SM)
-  int64_t total4 = 0;
-  for (int i = 0; i < count; ++i) total4 += d[i].M * d[i].K / 4;
-  // Tensors with the longest rows first: kernel 2 hands rows to warps round-robin, and a long row met
+  const int64_t cap = (int64_t)sm_count * kActBlocksPerSm;  // one full wave
+  // Tensors with the longest segments first: kernel 2 hands segments to warps round-robin, and a long one met
   // at the end of a warp's list would be the launch's tail.  Slot i of `absmax_slots` stays with the
   // i-th tensor of this order; nothing outside the two kernels reads the slots.
-  int ord[kMaxActBatch];
+  int ord[P];
   for (int i = 0; i < count; ++i) ord[i] = i;
-  std::stable_sort(ord, ord + count, [&](int a, int c) { return d[a].K > d[c].K; });
-  int64_t rows = 0;
-  int blocks1 = 0;
+  const auto seg_units = [](int64_t K) {
+    const int64_t u = K / 128, n = (u + kSegUnits - 1) / kSegUnits;
+    return (int)((u + n - 1) / n);
+  };
+  if (P > 1)
+    std::stable_sort(ord, ord + count, [&](int a, int c) { return seg_units(d[a].K) > seg_units(d[c].K); });
+  int64_t units = 0, segs = 0;
   for (int i = 0; i < count; ++i) {
     const qb_act_desc& q = d[ord[i]];
     ActItem& t = b.item[i];
@@ -164,32 +301,35 @@ static qb_status launch_act_batch(const qb_act_desc* d, int count, void* ws, uin
     t.act_scale = q.act_scale;
     t.rowsum = q.rowsum;
     t.M = q.M;
-    t.K = q.K;
-    t.row_begin = rows;
-    rows += q.M;
-    // blocks of kernel 1 in proportion to the tensor's size (rounded down, so that the launch never
-    // exceeds one wave: a block of a second wave would run alone for as long as the whole first wave),
-    // each thread >= 4 loads when possible
-    const int64_t n4 = q.M * q.K / 4;
-    int64_t want = (n4 + (int64_t)kActThreads * 4 - 1) / ((int64_t)kActThreads * 4);
-    const int64_t avail = cap - count > 0 ? cap - count : 0;  // one block per tensor is set aside
-    const int64_t share = 1 + avail * n4 / total4;
-    if (want > share) want = share;
-    if (want < 1) want = 1;
-    t.block_begin = blocks1;
-    t.blocks = (int32_t)want;
-    blocks1 += (int)want;
+    t.unit_begin = units;
+    t.seg_begin = segs;
+    t.units_per_row = (int32_t)(q.K / 128);
+    t.seg_units = seg_units(q.K);
+    t.segs_per_row = (t.units_per_row + t.seg_units - 1) / t.seg_units;
+    units += q.M * t.units_per_row;
+    segs += q.M * t.segs_per_row;
   }
-  b.rows_total = rows;
-  b.keep_fraction = l2_keep_fraction(16.0 * (double)total4);
-  QB_CUDA_TRY(cudaMemsetAsync(absmax_slots, 0, sizeof(uint32_t) * (size_t)count, stream));
-  act_absmax_kernel<<<(unsigned)blocks1, kActThreads, 0, stream>>>(b);
-  QB_CUDA_TRY(cudaGetLastError());
-  const int warps_per_block = kActThreads / 32;
-  int64_t blocks2 = (rows + warps_per_block - 1) / warps_per_block;
-  if (blocks2 > cap) blocks2 = cap;
-  act_quantize_kernel<<<(unsigned)blocks2, kActThreads, 0, stream>>>(b);
-  QB_CUDA_TRY(cudaGetLastError());
+  b.units_total = units;
+  b.segs_total = segs;
+  b.keep_fraction = l2_keep_fraction(512.0 * (double)units);
+  const int64_t seg_blocks = (segs + kActWarps - 1) / kActWarps;
+  if constexpr (P == 1) {
+    // A segment for every resident warp (4,736 of them; 1,024 x 768 needs 1,024): one launch.
+    if (seg_blocks <= cap) {
+      b.units_per_block = 0;
+      QB_CUDA_TRY(launch_kernel(act_fused_kernel, (unsigned)seg_blocks, kActThreads, 0, stream, true, 1, true, b));
+      return QB_OK;
+    }
+  }
+  // equal shares of whole batches of kSegUnits units per warp
+  int64_t share = (units + cap - 1) / cap;
+  share = (share + kSegUnits - 1) / kSegUnits * kSegUnits;
+  b.units_per_block = share;
+  // The first pass is not set up under the kernel before it: after a GEMM, whose CTAs have the SM's shared memory,
+  // its loads in flight would have to make do with the L1 that a shared-memory-heavy kernel leaves (two
+  // BERT-large layers at M = 24576: 1,172 us this way, 1,240 when it overlaps the GEMM before it).
+  QB_CUDA_TRY(launch_kernel(act_absmax_kernel<P>, (unsigned)((units + share - 1) / share), kActThreads, 0, stream, false, 1, false, b));
+  QB_CUDA_TRY(launch_kernel(act_quantize_kernel<P>, (unsigned)std::min(seg_blocks, cap), kActThreads, 0, stream, true, 1, false, b));
   return QB_OK;
 }
 
@@ -221,7 +361,7 @@ extern "C" qb_status qb_quantize_act(const float* x, int64_t M, int64_t K, int8_
   if (st != QB_OK) return st;
   uint32_t* slot = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + qb::kWsActMaxOff);
   const qb_act_desc d{x, M, K, xq, act_scale, rowsum};
-  return qb::launch_act_batch(&d, 1, ws, slot, sms, (cudaStream_t)cuda_stream);
+  return qb::launch_act_batch<1>(&d, 1, ws, slot, sms, (cudaStream_t)cuda_stream);
 }
 
 extern "C" qb_status qb_quantize_act_batch(const qb_act_desc* descs, int32_t count, void* ws, size_t ws_bytes,
@@ -247,7 +387,7 @@ extern "C" qb_status qb_quantize_act_batch(const qb_act_desc* descs, int32_t cou
   uint32_t* slots = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + qb::kWsRangeOff);
   for (int i = 0; i < count; i += qb::kMaxActBatch) {
     const int n = count - i < qb::kMaxActBatch ? count - i : qb::kMaxActBatch;
-    st = qb::launch_act_batch(descs + i, n, ws, slots, sms, (cudaStream_t)cuda_stream);
+    st = qb::launch_act_batch<qb::kMaxActBatch>(descs + i, n, ws, slots, sms, (cudaStream_t)cuda_stream);
     if (st != QB_OK) return st;
   }
   return QB_OK;

@@ -305,17 +305,6 @@ struct RegsSlice {
   int32_t first_unit; // of the slice inside its group (teams)
 };
 
-__device__ __forceinline__ float min3_nan(float a, float b, float c) {
-  float d;
-  asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-__device__ __forceinline__ float max3_nan(float a, float b, float c) {
-  float d;
-  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-  return d;
-}
-
 // Four codes of one float4 as a 4k-bit field in the low bits of the result (k < 8: bits from 22 up are
 // left over from the rounding constant and are dropped by the narrow store that follows).
 template <int BITS, bool CLAMP>
