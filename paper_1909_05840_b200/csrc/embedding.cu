@@ -27,6 +27,7 @@ __device__ __forceinline__ bool finite_f(float x) { return fabsf(x) <= 3.4028234
 // many loads in flight each take the place of many blocks that would queue on the same 2 D atomics.
 __global__ void emb_range_kernel(const float4* __restrict__ e, int64_t V, int d4, int slots, float keep_fraction,
                                  uint32_t* __restrict__ col_hi, uint32_t* __restrict__ col_lo_inv, void* ws) {
+  pdl_begin();
   const uint64_t pol = policy_evict_last(keep_fraction);
   extern __shared__ uint32_t emb_smem[];  // [slots][2][4 * d4] encoded maxima / inverted minima
   const int q = threadIdx.x % d4, slot = threadIdx.x / d4;
@@ -125,6 +126,7 @@ __global__ void emb_pack_kernel(const float4* __restrict__ e, int64_t V, int d4,
   constexpr int WORDS = 4 * BITS;  // output words per unit of 128 codes
   constexpr int NSRC = BITS == 8 ? 1 : (BITS == 4 ? 2 : 4);
   const int q = threadIdx.x, lane = threadIdx.x & 31, unit = threadIdx.x >> 5;
+  pdl_begin();
   const uint64_t pol = policy_evict_first();
   ColParams p;
 #pragma unroll
@@ -181,6 +183,7 @@ __global__ void emb_lookup_kernel(const int32_t* __restrict__ ids, int64_t T, co
                                   const float* __restrict__ q0, int accumulate, float4* __restrict__ out, void* ws) {
   constexpr uint32_t kMask = BITS == 8 ? 0xFFFFFFFFu : ((1u << (4 * BITS)) - 1u);
   const int q = threadIdx.x;
+  pdl_begin();
   float d[4], z[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
@@ -276,17 +279,13 @@ extern "C" qb_status qb_quantize_embedding(const float* table, int64_t V, int64_
     if (rblocks * slots > V) rblocks = (V + slots - 1) / slots;
     // slots * D <= 4096 columns (blockDim <= 1024 threads of four columns each): at most 32 KB
     const size_t smem = (size_t)slots * 2 * (size_t)D * sizeof(uint32_t);
-    qb::emb_range_kernel<<<(unsigned)rblocks, threads * slots, smem, stream>>>(e4, V, threads, slots, qb::l2_keep_fraction(4.0 * (double)V * (double)D), col_hi, col_lo, ws);
-    QB_CUDA_TRY(cudaGetLastError());
+    QB_CUDA_TRY(qb::launch_kernel(qb::emb_range_kernel, (unsigned)rblocks, (unsigned)(threads * slots), smem, stream, true, 1, false,
+                                  e4, V, threads, slots, qb::l2_keep_fraction(4.0 * (double)V * (double)D), col_hi, col_lo, ws));
   }
   const int cpg = (int)(D / groups);
-  switch (bits) {
-    case 2: qb::emb_pack_kernel<2><<<(unsigned)blocks, threads, 0, stream>>>(e4, V, threads, cpg, col_hi, col_lo, packed, delta, q0); break;
-    case 3: qb::emb_pack_kernel<3><<<(unsigned)blocks, threads, 0, stream>>>(e4, V, threads, cpg, col_hi, col_lo, packed, delta, q0); break;
-    case 4: qb::emb_pack_kernel<4><<<(unsigned)blocks, threads, 0, stream>>>(e4, V, threads, cpg, col_hi, col_lo, packed, delta, q0); break;
-    default: qb::emb_pack_kernel<8><<<(unsigned)blocks, threads, 0, stream>>>(e4, V, threads, cpg, col_hi, col_lo, packed, delta, q0); break;
-  }
-  QB_CUDA_TRY(cudaGetLastError());
+  auto pack = bits == 2 ? qb::emb_pack_kernel<2> : (bits == 3 ? qb::emb_pack_kernel<3> : (bits == 4 ? qb::emb_pack_kernel<4> : qb::emb_pack_kernel<8>));
+  QB_CUDA_TRY(qb::launch_kernel(pack, (unsigned)blocks, (unsigned)threads, 0, stream, true, 1, false, e4, V, threads, cpg, col_hi,
+                                col_lo, packed, delta, q0));
   return QB_OK;
 }
 
@@ -320,12 +319,8 @@ extern "C" qb_status qb_embedding_lookup(const int32_t* ids, int64_t T, const ui
   const int cpg = (int)(D / groups);
   float4* o4 = reinterpret_cast<float4*>(out);
   const int acc = accumulate ? 1 : 0;
-  switch (bits) {
-    case 2: qb::emb_lookup_kernel<2><<<(unsigned)blocks, threads, 0, stream>>>(ids, T, packed, V, threads, cpg, delta, q0, acc, o4, ws); break;
-    case 3: qb::emb_lookup_kernel<3><<<(unsigned)blocks, threads, 0, stream>>>(ids, T, packed, V, threads, cpg, delta, q0, acc, o4, ws); break;
-    case 4: qb::emb_lookup_kernel<4><<<(unsigned)blocks, threads, 0, stream>>>(ids, T, packed, V, threads, cpg, delta, q0, acc, o4, ws); break;
-    default: qb::emb_lookup_kernel<8><<<(unsigned)blocks, threads, 0, stream>>>(ids, T, packed, V, threads, cpg, delta, q0, acc, o4, ws); break;
-  }
-  QB_CUDA_TRY(cudaGetLastError());
+  auto lookup = bits == 2 ? qb::emb_lookup_kernel<2> : (bits == 3 ? qb::emb_lookup_kernel<3> : (bits == 4 ? qb::emb_lookup_kernel<4> : qb::emb_lookup_kernel<8>));
+  QB_CUDA_TRY(qb::launch_kernel(lookup, (unsigned)blocks, (unsigned)threads, 0, stream, true, 1, false, ids, T, packed, V, threads, cpg,
+                                delta, q0, acc, o4, ws));
   return QB_OK;
 }

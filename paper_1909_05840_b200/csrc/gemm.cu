@@ -318,6 +318,7 @@ qb_gemm_kernel(const __grid_constant__ GP gp) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const uint32_t smem_base = ptx::smem_u32(smem);
   if ((smem_base & 1023u) != 0u) {  // never expected; leave without touching anything
+    pdl_begin();
     if (threadIdx.x == 0) report_status(gp.ws, QB_ERR_CUDA, (int)smem_base);
     return;
   }
@@ -364,6 +365,8 @@ qb_gemm_kernel(const __grid_constant__ GP gp) {
   if constexpr (CG == 2) ptx::cluster_sync_all();
   ptx::tcgen05_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
+  // barriers and tensor memory are set up while the kernel before this one drains; its results are read below
+  pdl_begin();
   // the barriers the MMA issuer waits on live in the group's first CTA
   auto full_lead = [&](int s) { return CG == 2 ? ptx::map_to_cta(full(s), 0) : full(s); };
   auto acc_empty_lead = [&](int a) { return CG == 2 ? ptx::map_to_cta(acc_empty(a), 0) : acc_empty(a); };
@@ -989,19 +992,7 @@ static qb_status launch_group_inst(const GP& gp, int grid, cudaStream_t stream) 
     QB_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
     if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_release);
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid, 1, 1);
-  cfg.blockDim = dim3(kGemmThreads, 1, 1);
-  cfg.dynamicSmemBytes = Cfg::kSmemBytes;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = CG;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = CG == 2 ? 1 : 0;
-  QB_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, gp));
+  QB_CUDA_TRY(launch_kernel(kernel, (unsigned)grid, kGemmThreads, Cfg::kSmemBytes, stream, true, CG, false, gp));
   return QB_OK;
 }
 
@@ -1334,6 +1325,7 @@ __global__ void __launch_bounds__(256) rowsum_i8_kernel(const int4* __restrict__
                                                         int32_t* __restrict__ rowsum) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * 8;
+  pdl_begin();
   for (int64_t m = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); m < M; m += warps) {
     int s = 0;
     for (int64_t c = lane; c < k16; c += 32) {
@@ -1363,9 +1355,8 @@ extern "C" qb_status qb_rowsum_i8(const int8_t* xq, int64_t M, int64_t K, int32_
   if (st != QB_OK) return st;
   int64_t blocks = (M + 7) / 8;
   if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
-  qb::rowsum_i8_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)cuda_stream>>>(reinterpret_cast<const int4*>(xq), M,
-                                                                                K / 16, rowsum);
-  QB_CUDA_TRY(cudaGetLastError());
+  QB_CUDA_TRY(qb::launch_kernel(qb::rowsum_i8_kernel, (unsigned)blocks, 256, 0, (cudaStream_t)cuda_stream, true, 1, false,
+                                reinterpret_cast<const int4*>(xq), M, K / 16, rowsum));
   return QB_OK;
 }
 

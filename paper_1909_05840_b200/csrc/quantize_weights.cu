@@ -108,6 +108,7 @@ __device__ __forceinline__ void flush_range(uint32_t* __restrict__ hi_enc, uint3
 __global__ void __launch_bounds__(kWqThreads)
 weight_range_kernel(const __grid_constant__ WeightBatch b) {
   const int lane = threadIdx.x & 31;
+  pdl_begin();
   const uint64_t pol = policy_evict_last(b.keep_fraction);
   const int warp_in_block = threadIdx.x >> 5;
   const int64_t gwarp = (int64_t)blockIdx.x * kWqWarps + warp_in_block;
@@ -230,6 +231,7 @@ __global__ void __launch_bounds__(256)
 ste_backward_kernel(const float4* __restrict__ grad_q, const float4* __restrict__ w, int64_t n4, int64_t k4,
                     int64_t rows_per_group, const float* __restrict__ lo, const float* __restrict__ hi,
                     float4* __restrict__ grad_w) {
+  pdl_begin();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
     const int64_t g = (i / k4) / rows_per_group;
@@ -564,6 +566,7 @@ weight_regs_kernel(const __grid_constant__ RegsBatch b) {
   const int id0 = (int)blockIdx.x / csize, stride = (int)gridDim.x / csize;  // items go to clusters
   int it = 0, prev_it = 0;
   float4 v[kRgUnits];
+  pdl_begin();
   RegsSlice s = regs_slice<CLUSTER>(b, id0, it, warp, lane, crank);
 #pragma unroll
   for (int j = 0; j < kRgUnits; ++j)
@@ -767,8 +770,7 @@ static qb_status launch_two_pass(const HostWeight* m, int count, void* ws, int s
   const int64_t warps = (units + upw - 1) / upw;
   const unsigned blocks = (unsigned)((warps + kWqWarps - 1) / kWqWarps);
 
-  weight_range_kernel<<<blocks, kWqThreads, 0, stream>>>(b);
-  QB_CUDA_TRY(cudaGetLastError());
+  QB_CUDA_TRY(launch_kernel(weight_range_kernel, blocks, kWqThreads, 0, stream, true, 1, false, b));
   HostWeight second[kMaxWeightBatch];
   for (int i = 0; i < count; ++i) {
     second[i] = m[i];
@@ -855,21 +857,8 @@ static qb_status launch_regs_cluster(const HostWeight* m, int count, int cl, voi
     b.ws = ws;
     b.total_items = items;
     b.count = n;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(std::min(items, max_clusters) * cl));
-    cfg.blockDim = dim3(kRgThreads);
-    cfg.stream = stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)cl;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    if (fake)
-      QB_CUDA_TRY(cudaLaunchKernelEx(&cfg, weight_regs_kernel<true, true, false>, b));
-    else
-      QB_CUDA_TRY(cudaLaunchKernelEx(&cfg, weight_regs_kernel<true, false, false>, b));
+    QB_CUDA_TRY(launch_kernel(fake ? weight_regs_kernel<true, true, false> : weight_regs_kernel<true, false, false>,
+                              (unsigned)(std::min(items, max_clusters) * cl), kRgThreads, 0, stream, true, (unsigned)cl, false, b));
   }
   return QB_OK;
 }
@@ -941,18 +930,9 @@ static qb_status launch_regs_single(const HostWeight* m, int count, bool ranged,
     b.total_items = (int32_t)items;
     b.count = n;
     const unsigned grid = (unsigned)std::min<int64_t>(items, sm_count);
-    if (ranged) {
-      if (fake)
-        weight_regs_kernel<false, true, true><<<grid, kRgThreads, 0, stream>>>(b);
-      else
-        weight_regs_kernel<false, false, true><<<grid, kRgThreads, 0, stream>>>(b);
-    } else {
-      if (fake)
-        weight_regs_kernel<false, true, false><<<grid, kRgThreads, 0, stream>>>(b);
-      else
-        weight_regs_kernel<false, false, false><<<grid, kRgThreads, 0, stream>>>(b);
-    }
-    QB_CUDA_TRY(cudaGetLastError());
+    auto kernel = ranged ? (fake ? weight_regs_kernel<false, true, true> : weight_regs_kernel<false, false, true>)
+                         : (fake ? weight_regs_kernel<false, true, false> : weight_regs_kernel<false, false, false>);
+    QB_CUDA_TRY(launch_kernel(kernel, grid, kRgThreads, 0, stream, true, 1, false, b));
   }
   return QB_OK;
 }
@@ -1253,9 +1233,8 @@ extern "C" qb_status qb_ste_backward(const float* grad_wq, const float* w, int64
   const int64_t n4 = N * K / 4;
   int64_t blocks = (n4 + 256 * 4 - 1) / (256 * 4);
   if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
-  qb::ste_backward_kernel<<<(unsigned)blocks, 256, 0, stream>>>(
-      reinterpret_cast<const float4*>(grad_wq), reinterpret_cast<const float4*>(w), n4, K / 4, N / groups, range_lo,
-      range_hi, reinterpret_cast<float4*>(grad_w));
-  QB_CUDA_TRY(cudaGetLastError());
+  QB_CUDA_TRY(qb::launch_kernel(qb::ste_backward_kernel, (unsigned)blocks, 256, 0, stream, true, 1, false,
+                                reinterpret_cast<const float4*>(grad_wq), reinterpret_cast<const float4*>(w), n4, K / 4,
+                                N / groups, range_lo, range_hi, reinterpret_cast<float4*>(grad_w)));
   return QB_OK;
 }
