@@ -75,7 +75,7 @@ size_t qb_packed_words(int64_t N, int64_t K, int bits) {
 
 size_t qb_workspace_bytes(int64_t M, int64_t N, int64_t K, int bits, int groups) {
   (void)M; (void)N; (void)K; (void)bits;
-  return qb::ws_bytes_needed(groups);
+  return qb::ws_bytes_recommended(groups);
 }
 
 qb_status qb_workspace_init(void* ws, size_t ws_bytes, void* cuda_stream) {

@@ -21,13 +21,14 @@
 #include <vector>
 
 #include "common.cuh"
+#include "mbar_wait.cuh"
 #include "ptx.cuh"
 
 namespace qb {
 
 constexpr int kWqThreads = 256;
 constexpr int kWqWarps = kWqThreads / 32;
-constexpr int kMaxWeightBatch = 32;  // matrices per launch (descriptors travel as kernel parameters)
+constexpr int kMaxWeightBatch = 96;  // matrices per launch (descriptors travel as kernel parameters)
 
 struct WeightItem {
   const float4* w;
@@ -352,6 +353,17 @@ __device__ __forceinline__ void rg_next_group(RgGroup& cur, const RgGroup& mine,
   next_start += ug;
 }
 
+// Item `i` of a 3-bit staging area: 32 codes = eight 12-bit fields held in 16-bit cells -> three words.
+__device__ __forceinline__ void store_3bit_item(const uint8_t* stg, uint32_t* __restrict__ out, const int i) {
+  const uint4 q = reinterpret_cast<const uint4*>(stg)[i];
+  const uint32_t f0 = q.x & 0xffffu, f1 = q.x >> 16, f2 = q.y & 0xffffu, f3 = q.y >> 16;
+  const uint32_t f4 = q.z & 0xffffu, f5 = q.z >> 16, f6 = q.w & 0xffffu, f7 = q.w >> 16;
+  uint32_t* o3 = out + i * 3;
+  o3[0] = f0 | (f1 << 12) | (f2 << 24);
+  o3[1] = (f2 >> 8) | (f3 << 4) | (f4 << 16) | (f5 << 28);
+  o3[2] = (f5 >> 4) | (f6 << 8) | (f7 << 20);
+}
+
 // One staging block (units BLK * 6 ... of the slice): fields into the warp's staging area, then out.
 template <int BITS, int BLK, bool MULTI, bool CLAMP>
 __device__ __forceinline__ void regs_pack_block(float4 (&v)[kRgUnits], const int n, RgGroup& cur, const RgGroup& mine,
@@ -382,16 +394,7 @@ __device__ __forceinline__ void regs_pack_block(float4 (&v)[kRgUnits], const int
   const int nu = min(kRgBlock, n - BLK * kRgBlock);
   uint32_t* const o = out + BLK * kRgBlock * 4 * BITS;
   if (BITS == 3) {
-    // 32 codes = eight 12-bit fields held in 16-bit cells -> three words; four such items per unit
-    if (lane < 4 * nu) {
-      const uint4 q = reinterpret_cast<const uint4*>(stg)[lane];
-      const uint32_t f0 = q.x & 0xffffu, f1 = q.x >> 16, f2 = q.y & 0xffffu, f3 = q.y >> 16;
-      const uint32_t f4 = q.z & 0xffffu, f5 = q.z >> 16, f6 = q.w & 0xffffu, f7 = q.w >> 16;
-      uint32_t* o3 = o + lane * 3;
-      o3[0] = f0 | (f1 << 12) | (f2 << 24);
-      o3[1] = (f2 >> 8) | (f3 << 4) | (f4 << 16) | (f5 << 28);
-      o3[2] = (f5 >> 4) | (f6 << 8) | (f7 << 20);
-    }
+    if (lane < 4 * nu) store_3bit_item(stg, o, lane);  // four items per unit
   } else {
     const int n16 = nu * BITS;  // 16 * BITS bytes per unit
     const uint4* pk = reinterpret_cast<const uint4*>(stg);
@@ -714,6 +717,316 @@ weight_regs_kernel(const __grid_constant__ RegsBatch b) {
   if (CLUSTER) ptx::cluster_sync_all();
 }
 
+// ---- shared-memory ring path ------------------------------------------------------------------------------
+// Groups too large for a cluster's registers (one range per matrix, say), read once: one persistent CTA per SM
+// (cooperative launch), every group cut into chunks of 32 units that are dealt round-robin, so that a group of
+// 9 MB is spread over all SMs and its range is known a few chunks after its first chunk was loaded.  A chunk
+// stays in a CTA's ring of twelve 16 KB stages from its load to its rounding:
+//   warp 0         brings chunks in with cp.async.bulk, as far ahead as stages are free
+//   warps 1..4     range: every warp reduces a quarter of each chunk, keeps the extremes over the CTA's run of
+//                  chunks of one group, and hands them over when the run ends
+//   warps 5..12    agents, one lane each, take the CTA's runs in turn: merge the run's range into the group's
+//                  (atomicMax), count the CTA in (release), wait until every CTA that holds a part of the
+//                  group has been counted (acquire), leave the group's parameters in shared memory.  The chain
+//                  takes about 2 us, five chunks' time; eight agents keep eight runs under way.
+//   warps 13..24   rounding: three teams of four warps take every third chunk, round and pack (or
+//                  fake-quantize) it from the ring and free the stage
+// Nobody waits for a later chunk of its own CTA's list, and a group may not span more rounds of the deal than
+// the ring has stages, so the loads and ranges that a team waits for never depend on that team.  One count and
+// two atomicMax per CTA and group, one polling lane per CTA and run: with one per warp and chunk the atomics
+// and polls of all SMs met on three words of one L2 slice and the set below took 299 us.
+// Memory-bound: 4 + k/8 B per weight.
+constexpr int kRingUnits = 32;                 // per chunk: 16 KB
+constexpr int kRingStages = 12;
+constexpr int kRingRangeWarps = 4;
+constexpr int kRingAgents = 8;
+constexpr int kRingRoundTeams = 3;             // of four warps
+constexpr int kRingFirstAgent = 1 + kRingRangeWarps;
+constexpr int kRingFirstRound = kRingFirstAgent + kRingAgents;
+constexpr int kRingThreads = 32 * (kRingFirstRound + 4 * kRingRoundTeams);
+constexpr int kRingWarpUnits = kRingUnits / 4; // of a range or rounding warp
+constexpr int kRingSmemBytes = kRingStages * kRingUnits * 512 + 4 * kRingRoundTeams * kRingWarpUnits * 128;
+// Rounds of the deal that a group may span, so that its last chunk is loaded and reduced while its first one
+// is still held, with two stages left for loads in flight.
+constexpr int kRingMaxSpan = kRingStages - 2;
+static_assert(kRingStages % kRingRoundTeams == 0, "a stage is always rounded by the same team");
+
+struct RingItem {
+  const float4* w;
+  uint32_t* packed;
+  float* delta;
+  float* q0;
+  int32_t ug;                // units per group
+  int32_t chunks_per_group;
+  int32_t chunk_begin;       // of the matrix, in the launch's list
+  int32_t group_begin;       // of the matrix, in the launch's tables
+  int32_t bits;
+};
+
+struct RingBatch {
+  RingItem item[kMaxWeightBatch];
+  uint32_t* hi_enc;    // [groups of the launch], cleared before the launch
+  uint32_t* lo_inv;
+  uint32_t* arrived;
+  void* ws;
+  int32_t chunks_total;
+  int32_t count;
+};
+
+// A chunk of the launch's list.  `it` only moves forward.
+struct RingChunk {
+  int it, group, first_unit, n;  // matrix, group inside it, first unit inside the group, units
+  __device__ __forceinline__ void seek(const RingBatch& b, int c) {
+    while (it + 1 < b.count && c >= b.item[it + 1].chunk_begin) ++it;
+    const RingItem& m = b.item[it];
+    const int local = c - m.chunk_begin;
+    group = local / m.chunks_per_group;
+    first_unit = (local - group * m.chunks_per_group) * kRingUnits;
+    n = min(m.ug - first_unit, kRingUnits);
+  }
+  // chunks of this group that the CTA meets from here on, one every `step` chunks
+  __device__ __forceinline__ int run(const RingBatch& b, int step) const {
+    return (b.item[it].chunks_per_group - first_unit / kRingUnits + step - 1) / step;
+  }
+};
+
+__global__ void __launch_bounds__(256) clear_words_kernel(uint32_t* p, int n) {
+  pdl_begin();
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) p[i] = 0u;
+}
+
+// Codes of the warp's units (n <= kRingWarpUnits) to the packed stream.
+template <int BITS>
+__device__ __forceinline__ void ring_pack(const float4 (&v)[kRingWarpUnits], const int n, const RgGroup& g, uint8_t* stg,
+                                          uint32_t* __restrict__ out, const int lane) {
+#pragma unroll
+  for (int j = 0; j < kRingWarpUnits; ++j)
+    if (j < n) {
+      const uint32_t f = quant_field_open<BITS, false>(v[j], g.lo, g.inv, g.hi);
+      const int fi = j * 32 + lane;
+      if (BITS == 8) reinterpret_cast<uint32_t*>(stg)[fi] = f;
+      if (BITS == 4 || BITS == 3) reinterpret_cast<uint16_t*>(stg)[fi] = (uint16_t)f;
+      if (BITS == 2) stg[fi] = (uint8_t)f;
+    }
+  __syncwarp();
+  if (BITS == 3) {
+    if (lane < 4 * n) store_3bit_item(stg, out, lane);
+  } else {
+    const int n16 = n * BITS;
+#pragma unroll
+    for (int r = 0; r < (kRingWarpUnits * BITS + 31) / 32; ++r) {
+      const int i = r * 32 + lane;
+      if (i < n16) reinterpret_cast<uint4*>(out)[i] = reinterpret_cast<const uint4*>(stg)[i];
+    }
+  }
+  __syncwarp();
+}
+
+template <bool FAKE>
+__global__ void __launch_bounds__(kRingThreads, 1)
+weight_ring_kernel(const __grid_constant__ RingBatch b) {
+  extern __shared__ __align__(1024) uint8_t smem[];
+  // A CTA's runs (its chunks of one group) use slot run % kRingStages: a run holds at least one stage, so at most
+  // kRingStages runs are between their first load and their last rounding.
+  __shared__ __align__(8) uint64_t s_bar[4 * kRingStages];
+  __shared__ uint32_t s_hi[kRingStages][kRingRangeWarps], s_lo[kRingStages][kRingRangeWarps];
+  __shared__ RgGroup s_par[kRingStages];
+  __shared__ volatile int s_abort;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t ring = ptx::smem_u32(smem), bars = ptx::smem_u32(s_bar);
+  auto full = [&](int s) { return bars + 8u * s; };                       // the stage's chunk has landed
+  auto empty = [&](int s) { return bars + 8u * (kRingStages + s); };      // the stage's chunk has been rounded
+  auto ranged = [&](int r) { return bars + 8u * (2 * kRingStages + r); }; // the run's range is in s_hi, s_lo
+  auto ready = [&](int r) { return bars + 8u * (3 * kRingStages + r); };  // the group's parameters are in s_par
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kRingStages; ++s) {
+      ptx::mbar_init(full(s), 1);
+      ptx::mbar_init(empty(s), 4);
+      ptx::mbar_init(ranged(s), kRingRangeWarps);
+      ptx::mbar_init(ready(s), 1);
+    }
+    s_abort = 0;
+    ptx::fence_mbar_init();
+  }
+  pdl_begin();
+  __syncthreads();
+  bool timed_out = false;
+  RingChunk c;
+  c.it = 0;
+  const int step = (int)gridDim.x;
+  if (warp == 0) {
+    if (ptx::elect_one()) {
+      int stage = 0;
+      uint32_t phase = 0;
+      for (int id = blockIdx.x; id < b.chunks_total; id += step) {
+        c.seek(b, id);
+        const RingItem& m = b.item[c.it];
+        if (!wait_barrier_relaxed(empty(stage), phase ^ 1u, &s_abort)) {
+          timed_out = true;
+          break;
+        }
+        ptx::mbar_arrive_expect_tx(full(stage), (uint32_t)c.n * 512u);
+        ptx::bulk_load_1d(ring + stage * kRingUnits * 512, m.w + ((int64_t)c.group * m.ug + c.first_unit) * 32,
+                          (uint32_t)c.n * 512u, full(stage));
+        if (++stage == kRingStages) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+    }
+  } else if (warp < kRingFirstAgent) {
+    const int part = warp - 1;
+    const float kInf = __int_as_float(0x7f800000);
+    int stage = 0, slot = 0, left = 0;  // left: chunks of this CTA left in the run
+    uint32_t phase = 0;
+    float lo = kInf, hi = -kInf;
+    for (int id = blockIdx.x; id < b.chunks_total; id += step) {
+      c.seek(b, id);
+      if (left == 0) left = c.run(b, step);
+      if (!wait_barrier_relaxed(full(stage), phase, &s_abort)) {
+        timed_out = true;
+        break;
+      }
+      const float4* src = reinterpret_cast<const float4*>(smem + stage * kRingUnits * 512) + part * kRingWarpUnits * 32 + lane;
+      const int n = min(c.n - part * kRingWarpUnits, kRingWarpUnits);
+#pragma unroll
+      for (int j = 0; j < kRingWarpUnits; ++j)
+        if (j < n) {
+          const float4 v = src[j * 32];
+          lo = min3_nan(min3_nan(lo, v.x, v.y), v.z, v.w);
+          hi = max3_nan(max3_nan(hi, v.x, v.y), v.z, v.w);
+        }
+      if (--left == 0) {
+        const uint32_t e_hi = __reduce_max_sync(0xffffffffu, float_to_ordered(hi));
+        const uint32_t e_lo = __reduce_max_sync(0xffffffffu, ~float_to_ordered(lo));
+        if (lane == 0) {
+          s_hi[slot][part] = e_hi;
+          s_lo[slot][part] = e_lo;
+          ptx::mbar_arrive(ranged(slot));
+        }
+        lo = kInf;
+        hi = -kInf;
+        if (++slot == kRingStages) slot = 0;
+      }
+      if (++stage == kRingStages) {
+        stage = 0;
+        phase ^= 1u;
+      }
+    }
+  } else if (warp < kRingFirstRound) {
+    if (lane == 0) {
+      const int agent = warp - kRingFirstAgent;
+      int slot = 0;
+      uint32_t phase = 0;
+      int id = blockIdx.x;
+      for (int run = 0; id < b.chunks_total; ++run) {
+        c.seek(b, id);
+        const int len = c.run(b, step);
+        if (run % kRingAgents == agent) {
+          const RingItem& m = b.item[c.it];
+          const int g = m.group_begin + c.group;
+          if (!wait_barrier_relaxed(ranged(slot), phase, &s_abort)) {
+            timed_out = true;
+            break;
+          }
+          uint32_t e_hi = 0, e_lo = 0;
+#pragma unroll
+          for (int i = 0; i < kRingRangeWarps; ++i) {
+            e_hi = max(e_hi, s_hi[slot][i]);
+            e_lo = max(e_lo, s_lo[slot][i]);
+          }
+          atomicMax(b.hi_enc + g, e_hi);
+          atomicMax(b.lo_inv + g, e_lo);
+          asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(b.arrived + g) : "memory");
+          const uint32_t target = (uint32_t)min(m.chunks_per_group, step);  // CTAs that hold a part of the group
+          if (ld_acquire(b.arrived + g) != target) {
+            const long long t0 = clock64();
+            while (ld_acquire(b.arrived + g) != target)
+              if (s_abort != 0 || clock64() - t0 > kWaitLimitCycles) {
+                timed_out = true;
+                break;
+              }
+          }
+          if (timed_out) break;
+          const float g_hi = ordered_to_float(__ldcg(b.hi_enc + g)), g_lo = ordered_to_float(~__ldcg(b.lo_inv + g));
+          const int L = (1 << m.bits) - 1;
+          const bool publish = c.first_unit == 0;
+          if (publish && !(fabsf(g_hi) <= 3.402823466e38f && fabsf(g_lo) <= 3.402823466e38f)) report_status(b.ws, QB_ERR_NONFINITE);
+          const GroupParams gp = finish_group(g_lo, g_hi, false, L, c.group, m.delta, m.q0, publish, b.ws);
+          s_par[slot] = RgGroup{gp.lo, gp.inv, group_step(gp, L), gp.hi};
+          ptx::mbar_arrive(ready(slot));
+        }
+        id += len * step;
+        if (++slot == kRingStages) {
+          slot = 0;
+          phase ^= 1u;
+        }
+      }
+    }
+  } else {
+    const int rw = warp - kRingFirstRound;
+    const int team = rw >> 2, part = rw & 3;
+    uint8_t* const stg = smem + kRingStages * kRingUnits * 512 + rw * kRingWarpUnits * 128;
+    int stage = 0, slot = -1, left = 0, turn = team;
+    uint32_t phase = 0, slot_phase = 1;
+    for (int id = blockIdx.x; id < b.chunks_total; id += step) {
+      c.seek(b, id);
+      if (left == 0) {
+        left = c.run(b, step);
+        if (++slot == kRingStages) slot = 0;
+        if (slot == 0) slot_phase ^= 1u;
+      }
+      --left;
+      if (turn == 0) {
+        turn = kRingRoundTeams;
+        const RingItem& m = b.item[c.it];
+        // In this order: once the chunk has landed, the one twelve chunks before it has been rounded, and with it
+        // every run that used this slot before; a barrier's parity is only told apart one phase at a time.
+        if (!wait_barrier_relaxed(full(stage), phase, &s_abort) || !wait_barrier_relaxed(ready(slot), slot_phase, &s_abort)) {
+          timed_out = true;
+          break;
+        }
+        const RgGroup cur = s_par[slot];
+        const int u0 = part * kRingWarpUnits;
+        const int n = min(c.n - u0, kRingWarpUnits);
+        const float4* src = reinterpret_cast<const float4*>(smem + stage * kRingUnits * 512) + u0 * 32 + lane;
+        float4 v[kRingWarpUnits];
+#pragma unroll
+        for (int j = 0; j < kRingWarpUnits; ++j)
+          if (j < n) v[j] = src[j * 32];
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(empty(stage));  // the warp's part is in registers
+        uint32_t* const out = m.packed + ((int64_t)c.group * m.ug + c.first_unit + u0) * (FAKE ? 128 : 4 * m.bits);
+        if (FAKE) {
+#pragma unroll
+          for (int j = 0; j < kRingWarpUnits; ++j)
+            if (j < n) reinterpret_cast<float4*>(out)[j * 32 + lane] = fake_quant4<false>(v[j], cur);
+        } else {
+          switch (m.bits) {  // team-uniform
+            case 2: ring_pack<2>(v, n, cur, stg, out, lane); break;
+            case 3: ring_pack<3>(v, n, cur, stg, out, lane); break;
+            case 4: ring_pack<4>(v, n, cur, stg, out, lane); break;
+            default: ring_pack<8>(v, n, cur, stg, out, lane); break;
+          }
+        }
+      }
+      --turn;
+      if (++stage == kRingStages) {
+        stage = 0;
+        phase ^= 1u;
+      }
+    }
+  }
+  if (timed_out) {
+    s_abort = 1;
+    report_status(b.ws, QB_ERR_TIMEOUT);
+    // let copies already in flight land before the CTA's shared memory is released
+    const long long t0 = clock64();
+    while (clock64() - t0 < 400000ll) {
+    }
+  }
+}
+
 struct HostWeight {
   const float* w;
   int64_t N, K;
@@ -964,60 +1277,91 @@ static qb_status launch_regs(const HostWeight* m_all, int count_all, void* ws, i
   return launch_regs_single(single.data(), (int)single.size(), false, ws, sm_count, stream, fake, false);
 }
 
-// One pair of launches of the two-pass path: matrices of one bit width (<= kMaxWeightBatch).
-struct WeightJob {
-  HostWeight m[kMaxWeightBatch];
-  int n;
-  int bits;
-};
-
-static void plan_weight_batch(const HostWeight* m, int count, int bits, std::vector<WeightJob>& jobs) {
-  WeightJob j;
-  j.n = count;
-  j.bits = bits;
-  for (int i = 0; i < count; ++i) j.m[i] = m[i];
-  jobs.push_back(j);
+// One pair of launches (clear, ring kernel) over `count` matrices (<= kMaxWeightBatch) whose groups fit the ring.
+// Their tables sit back to back in the workspace: maxima at ws + kWsRangeOff, inverted minima, arrivals.
+template <bool FAKE>
+static qb_status launch_ring_form(const RingBatch& b, unsigned grid, cudaStream_t stream) {
+  static std::atomic<bool> attr_set[64] = {};
+  int dev = 0;
+  QB_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= 64 || !attr_set[dev].load(std::memory_order_acquire)) {
+    QB_CUDA_TRY(cudaFuncSetAttribute(weight_ring_kernel<FAKE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingSmemBytes));
+    if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_release);
+  }
+  QB_CUDA_TRY(launch_kernel(weight_ring_kernel<FAKE>, grid, kRingThreads, kRingSmemBytes, stream, true, 1, true, b));
+  return QB_OK;
+}
+static qb_status launch_ring(const HostWeight* m, int count, void* ws, int sm_count, cudaStream_t stream, bool fake) {
+  RingBatch b;
+  int groups = 0, chunks = 0;
+  for (int i = 0; i < count; ++i) {
+    const HostWeight& h = m[i];
+    RingItem& it = b.item[i];
+    it.w = reinterpret_cast<const float4*>(h.w);
+    it.packed = h.packed;
+    it.delta = h.delta;
+    it.q0 = h.q0;
+    it.ug = (int32_t)group_units(h);
+    it.chunks_per_group = (it.ug + kRingUnits - 1) / kRingUnits;
+    it.chunk_begin = chunks;
+    it.group_begin = groups;
+    it.bits = h.bits;
+    chunks += it.chunks_per_group * h.groups;
+    groups += h.groups;
+  }
+  b.ws = ws;
+  b.hi_enc = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + kWsRangeOff);
+  b.lo_inv = b.hi_enc + groups;
+  b.arrived = b.lo_inv + groups;
+  b.chunks_total = chunks;
+  b.count = count;
+  QB_CUDA_TRY(launch_kernel(clear_words_kernel, (unsigned)std::min((3 * groups + 255) / 256, sm_count), 256, 0, stream, true, 1, false,
+                            b.hi_enc, 3 * groups));
+  const unsigned grid = (unsigned)std::min(chunks, sm_count);
+  return fake ? launch_ring_form<true>(b, grid, stream) : launch_ring_form<false>(b, grid, stream);
 }
 
-// The two-pass jobs of a call, one after the other (they share the range tables at the head of the workspace).
-static qb_status run_weight_jobs(const std::vector<WeightJob>& jobs, void* ws, int sm_count, cudaStream_t stream) {
-  for (const WeightJob& j : jobs) {
-    qb_status st = launch_two_pass(j.m, j.n, ws, sm_count, stream);
-    if (st != QB_OK) return st;
-  }
+// Matrices whose groups do not fit a cluster's registers: the ring as long as a group spans few enough rounds of
+// its deal (up to 148 * 9 chunks of 16 KB, 22 MB), else, and where the workspace has no room for the
+// arrival counts, the two passes.  Both are a pair of launches per kMaxWeightBatch matrices.
+static inline bool ring_eligible(const HostWeight& h, int sm_count) {
+  return (group_units(h) + kRingUnits - 1) / kRingUnits <= (int64_t)(kRingMaxSpan - 1) * sm_count;
+}
+static qb_status launch_large_groups(const std::vector<HostWeight>& m, void* ws, size_t ws_bytes, int sm_count,
+                                     cudaStream_t stream, bool fake) {
+  std::vector<HostWeight> part[2];
+  for (const HostWeight& h : m) part[ring_eligible(h, sm_count) ? 0 : 1].push_back(h);
+  for (int k = 0; k < 2; ++k)
+    for (size_t i = 0; i < part[k].size(); i += kMaxWeightBatch) {
+      const int n = (int)std::min<size_t>(kMaxWeightBatch, part[k].size() - i);
+      size_t groups = 0;
+      for (int j = 0; j < n; ++j) groups += (size_t)part[k][i + j].groups;
+      const bool ring = k == 0 && kWsRangeOff + 12 * groups <= ws_bytes;
+      qb_status st = ring ? launch_ring(part[k].data() + i, n, ws, sm_count, stream, fake)
+                          : launch_two_pass(part[k].data() + i, n, ws, sm_count, stream, fake);
+      if (st != QB_OK) return st;
+    }
   return QB_OK;
 }
 
-static qb_status launch_weight_batch(const HostWeight* m, int count, int bits, void* ws, int sm_count,
-                                     cudaStream_t stream) {
+// All matrices of a call, any bit widths.
+static qb_status launch_weights(const std::vector<HostWeight>& m, void* ws, size_t ws_bytes, int sm_count,
+                                cudaStream_t stream, bool fake) {
   std::vector<HostWeight> regs, rest;
-  for (int i = 0; i < count; ++i) (regs_eligible(m[i]) ? regs : rest).push_back(m[i]);
+  for (const HostWeight& h : m) (regs_eligible(h) ? regs : rest).push_back(h);
   if (!regs.empty()) {
-    qb_status st = launch_regs(regs.data(), (int)regs.size(), ws, sm_count, stream);
+    qb_status st = launch_regs(regs.data(), (int)regs.size(), ws, sm_count, stream, fake);
     if (st != QB_OK) return st;
   }
-  if (rest.empty()) return QB_OK;
-  std::vector<WeightJob> jobs;
-  for (size_t i = 0; i < rest.size(); i += kMaxWeightBatch)
-    plan_weight_batch(rest.data() + i, (int)std::min<size_t>(kMaxWeightBatch, rest.size() - i), bits, jobs);
-  return run_weight_jobs(jobs, ws, sm_count, stream);
-}
-
-// Fake quantization of one matrix: the register-resident kernel where the groups fit it, else the two passes.
-static qb_status launch_fake_quantize(const float* w, int64_t N, int64_t K, int bits, int groups,
-                                      const float* range_lo, const float* range_hi, float* wq, float* delta,
-                                      float* q0, void* ws, int sm_count, cudaStream_t stream) {
-  // `packed` of the descriptor points to the fp32 output
-  const HostWeight h{w, N, K, groups, range_lo, range_hi, reinterpret_cast<uint32_t*>(wq), delta, q0, bits};
-  if (regs_eligible(h)) return launch_regs(&h, 1, ws, sm_count, stream, true);
-  return launch_two_pass(&h, 1, ws, sm_count, stream, true);
+  return launch_large_groups(rest, ws, ws_bytes, sm_count, stream, fake);
 }
 
 qb_status launch_quantize_pack_weights(const float* w, int64_t N, int64_t K, int bits, int groups,
                                        const float* range_lo, const float* range_hi, uint32_t* packed,
-                                       float* delta, float* q0, void* ws, int sm_count, cudaStream_t stream) {
-  const HostWeight m{w, N, K, groups, range_lo, range_hi, packed, delta, q0, bits};
-  return launch_weight_batch(&m, 1, bits, ws, sm_count, stream);
+                                       float* delta, float* q0, void* ws, size_t ws_bytes, int sm_count,
+                                       cudaStream_t stream) {
+  return launch_weights({HostWeight{w, N, K, groups, range_lo, range_hi, packed, delta, q0, bits}}, ws, ws_bytes, sm_count,
+                        stream, false);
 }
 
 static qb_status validate_weight(const char* who, const float* w, int64_t N, int64_t K, int bits, int groups,
@@ -1053,45 +1397,18 @@ extern "C" qb_status qb_quantize_pack_weights(const float* w, int64_t N, int64_t
   int sms = 0;
   st = qb::require_sm100(&sms);
   if (st != QB_OK) return st;
-  return qb::launch_quantize_pack_weights(w, N, K, bits, groups, range_lo, range_hi, packed, delta, q0, ws, sms,
-                                          (cudaStream_t)cuda_stream);
+  return qb::launch_quantize_pack_weights(w, N, K, bits, groups, range_lo, range_hi, packed, delta, q0, ws, ws_bytes,
+                                          sms, (cudaStream_t)cuda_stream);
 }
 
-namespace qb {
-
-// The launch plan of a batch: the matrices of the register-resident path, and the jobs of the others.
-static void plan_batch(const qb_weight_desc* descs, int count, std::vector<HostWeight>& regs,
-                       std::vector<WeightJob>& jobs) {
-  // Matrices that fit the register-resident path (see regs_eligible): all bit widths in the same launches.
-  // The others (own ranges over groups too large for a cluster) take the two passes: launches of one bit
-  // width, at most kMaxWeightBatch matrices each; the range tables of a launch reuse the head of the
-  // workspace (launches on one stream run in order).
-  std::vector<int> order;
+static std::vector<qb::HostWeight> host_weights(const qb_weight_desc* descs, int32_t count) {
+  std::vector<qb::HostWeight> m(count);
   for (int i = 0; i < count; ++i) {
     const qb_weight_desc& d = descs[i];
-    const HostWeight h{d.w, d.N, d.K, d.groups, d.range_lo, d.range_hi, d.packed, d.delta, d.q0, d.bits};
-    if (regs_eligible(h))
-      regs.push_back(h);
-    else
-      order.push_back(i);
+    m[i] = qb::HostWeight{d.w, d.N, d.K, d.groups, d.range_lo, d.range_hi, d.packed, d.delta, d.q0, d.bits};
   }
-  const int rest = (int)order.size();
-  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return descs[a].bits < descs[b].bits; });
-  int i = 0;
-  while (i < rest) {
-    HostWeight m[kMaxWeightBatch];
-    int n = 0;
-    const int bits = descs[order[i]].bits;
-    while (i < rest && n < kMaxWeightBatch && descs[order[i]].bits == bits) {
-      const qb_weight_desc& d = descs[order[i]];
-      m[n++] = HostWeight{d.w, d.N, d.K, d.groups, d.range_lo, d.range_hi, d.packed, d.delta, d.q0, d.bits};
-      ++i;
-    }
-    plan_weight_batch(m, n, bits, jobs);
-  }
+  return m;
 }
-
-}  // namespace qb
 
 extern "C" qb_status qb_quantize_pack_weights_batch(const qb_weight_desc* descs, int32_t count, void* ws,
                                                     size_t ws_bytes, void* cuda_stream) {
@@ -1115,15 +1432,7 @@ extern "C" qb_status qb_quantize_pack_weights_batch(const qb_weight_desc* descs,
   int sms = 0;
   qb_status st = qb::require_sm100(&sms);
   if (st != QB_OK) return st;
-  std::vector<qb::HostWeight> regs;
-  std::vector<qb::WeightJob> jobs;
-  qb::plan_batch(descs, count, regs, jobs);
-  if (!regs.empty()) {
-    st = qb::launch_regs(regs.data(), (int)regs.size(), ws, sms, (cudaStream_t)cuda_stream);
-    if (st != QB_OK) return st;
-  }
-  if (jobs.empty()) return QB_OK;
-  return qb::run_weight_jobs(jobs, ws, sms, (cudaStream_t)cuda_stream);
+  return qb::launch_weights(host_weights(descs, count), ws, ws_bytes, sms, (cudaStream_t)cuda_stream, false);
 }
 
 extern "C" int32_t qb_quantize_pack_weights_launch_count(const qb_weight_desc* descs, int32_t count) {
@@ -1132,20 +1441,22 @@ extern "C" int32_t qb_quantize_pack_weights_launch_count(const qb_weight_desc* d
     const qb_weight_desc& d = descs[i];
     if (d.N <= 0 || d.K <= 0 || d.groups < 1 || d.N % d.groups != 0 || d.K % 128 != 0) return 0;
   }
-  std::vector<qb::HostWeight> regs;
-  std::vector<qb::WeightJob> jobs;
-  qb::plan_batch(descs, count, regs, jobs);
+  int sms = 148;
+  qb::require_sm100(&sms);  // without a device: the plan for a 148-SM part
   int per_cluster[qb::kRgMaxCluster + 1] = {};
-  int ranged = 0;
-  for (const qb::HostWeight& h : regs) {
-    if (h.range_lo != nullptr)
+  int ranged = 0, ring = 0, two_pass = 0;
+  for (const qb::HostWeight& h : host_weights(descs, count)) {
+    if (!qb::regs_eligible(h))
+      ++(qb::ring_eligible(h, sms) ? ring : two_pass);
+    else if (h.range_lo != nullptr)
       ++ranged;
     else
       ++per_cluster[std::max(1, qb::regs_cluster_size(h))];
   }
-  int32_t n = (ranged + qb::kRgMaxBatch - 1) / qb::kRgMaxBatch;
-  for (int cl = 1; cl <= qb::kRgMaxCluster; ++cl) n += (per_cluster[cl] + qb::kRgMaxBatch - 1) / qb::kRgMaxBatch;
-  n += 2 * (int32_t)jobs.size();
+  const auto launches = [](int matrices, int per_launch) { return (matrices + per_launch - 1) / per_launch; };
+  int32_t n = launches(ranged, qb::kRgMaxBatch);
+  for (int cl = 1; cl <= qb::kRgMaxCluster; ++cl) n += launches(per_cluster[cl], qb::kRgMaxBatch);
+  n += 2 * (launches(ring, qb::kMaxWeightBatch) + launches(two_pass, qb::kMaxWeightBatch));
   return n;
 }
 
@@ -1163,8 +1474,9 @@ extern "C" qb_status qb_fake_quantize_weights(const float* w, int64_t N, int64_t
   int sms = 0;
   st = qb::require_sm100(&sms);
   if (st != QB_OK) return st;
-  return qb::launch_fake_quantize(w, N, K, bits, groups, range_lo, range_hi, wq, delta, q0, ws, sms,
-                                  (cudaStream_t)cuda_stream);
+  // `packed` of the descriptor points to the fp32 output
+  return qb::launch_weights({qb::HostWeight{w, N, K, groups, range_lo, range_hi, reinterpret_cast<uint32_t*>(wq), delta, q0, bits}},
+                            ws, ws_bytes, sms, (cudaStream_t)cuda_stream, true);
 }
 
 extern "C" qb_status qb_fake_quantize_weights_batch(const qb_weight_desc* descs, int32_t count, void* ws,
@@ -1189,22 +1501,7 @@ extern "C" qb_status qb_fake_quantize_weights_batch(const qb_weight_desc* descs,
   int sms = 0;
   qb_status st = qb::require_sm100(&sms);
   if (st != QB_OK) return st;
-  std::vector<qb::HostWeight> regs, rest;
-  for (int i = 0; i < count; ++i) {
-    const qb_weight_desc& d = descs[i];
-    const qb::HostWeight h{d.w, d.N, d.K, d.groups, d.range_lo, d.range_hi, d.packed, d.delta, d.q0, d.bits};
-    (qb::regs_eligible(h) ? regs : rest).push_back(h);
-  }
-  if (!regs.empty()) {
-    st = qb::launch_regs(regs.data(), (int)regs.size(), ws, sms, (cudaStream_t)cuda_stream, true);
-    if (st != QB_OK) return st;
-  }
-  for (size_t i = 0; i < rest.size(); i += qb::kMaxWeightBatch) {  // own ranges over groups beyond a cluster: two passes
-    st = qb::launch_two_pass(rest.data() + i, (int)std::min<size_t>(qb::kMaxWeightBatch, rest.size() - i), ws, sms,
-                             (cudaStream_t)cuda_stream, true);
-    if (st != QB_OK) return st;
-  }
-  return QB_OK;
+  return qb::launch_weights(host_weights(descs, count), ws, ws_bytes, sms, (cudaStream_t)cuda_stream, true);
 }
 
 extern "C" qb_status qb_ste_backward(const float* grad_wq, const float* w, int64_t N, int64_t K, int groups,

@@ -22,9 +22,9 @@ namespace qb {
 // defined in quantize_weights.cu
 qb_status launch_quantize_pack_weights(const float* w, int64_t N, int64_t K, int bits, int groups,
                                        const float* range_lo, const float* range_hi, uint32_t* packed,
-                                       float* delta, float* q0, void* ws, int sm_count, cudaStream_t stream);
+                                       float* delta, float* q0, void* ws, size_t ws_bytes, int sm_count, cudaStream_t stream);
 
-constexpr size_t kNoAllocScratchBytes = kWsRangeOff + 8 * (size_t)QB_NOALLOC_MAX_GROUPS;
+constexpr size_t kNoAllocScratchBytes = kWsRangeOff + 12 * (size_t)QB_NOALLOC_MAX_GROUPS;
 
 // Same layout as a caller-provided workspace: status word at offset 0, encoded ranges at kWsRangeOff.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
@@ -85,8 +85,8 @@ extern "C" qb_status qb_quantize_pack_weights_noalloc(const float* w, int64_t N,
   cudaStream_t stream = (cudaStream_t)cuda_stream;
   // the status word is sticky inside one call only: start it at zero (the ranges are cleared by the launcher)
   QB_CUDA_TRY(cudaMemsetAsync(scratch, 0, qb::kWsRangeOff, stream));
-  st = qb::launch_quantize_pack_weights(w, N, K, bits, groups, range_lo, range_hi, packed, delta, q0, scratch, sms,
-                                        stream);
+  st = qb::launch_quantize_pack_weights(w, N, K, bits, groups, range_lo, range_hi, packed, delta, q0, scratch,
+                                        qb::kNoAllocScratchBytes, sms,                                        stream);
   if (st != QB_OK) return st;
   if (status_out != nullptr)
     QB_CUDA_TRY(cudaMemcpyAsync(status_out, scratch, sizeof(int32_t), cudaMemcpyDeviceToDevice, stream));
