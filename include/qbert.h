@@ -162,7 +162,7 @@ qb_status qb_quantize_pack_weights_batch(const qb_weight_desc* descs /*host*/, i
  * receives tensors but no allocator, code running while its memory pool is frozen, a serving loop in
  * which cudaMalloc is banned because it stalls the whole device.  For them the per-group min/max
  * scratch that normally sits in the caller's workspace is a fixed array inside the library, held on
- * every GPU that loads it until the process ends (256 + 12 * QB_NOALLOC_MAX_GROUPS bytes).  The call
+ * every GPU that loads it until the process ends (256 + 40 * QB_NOALLOC_MAX_GROUPS bytes).  The call
  * itself allocates and frees nothing.
  *
  *  - Arguments and results are those of qb_quantize_pack_weights, minus the workspace.  `groups` may

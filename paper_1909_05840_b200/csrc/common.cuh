@@ -19,7 +19,7 @@ namespace qb {
 // [40]  uint32 arrived           blocks of the running launch that have published      } calls
 // [44]  uint32 round             counts the launches whose blocks waited for one another
 // [256] uint32 range_hi_enc[G], uint32 range_lo_inv[G]   ordered encodings of per-group max / min
-//       uint32 arrived[G]        CTAs whose part of the group's range is in (weight_ring_kernel)
+//       or, weight_ring_kernel: uint64 [groups][CTAs], encoded max << 32 | inverted encoded min
 constexpr size_t kWsStatusOff = 0;
 constexpr size_t kWsDetailOff = 4;
 constexpr size_t kWsActMaxOff = 16;
@@ -38,14 +38,19 @@ struct WsHeader {
   uint32_t round;
 };
 
-// What a call on G groups must get, and what qb_workspace_bytes tells callers to give: with four more bytes per
-// group the weight quantizer reads W once where groups are too large for a cluster's registers.
-inline size_t ws_bytes_of(int groups, size_t per_group) {
-  size_t b = kWsRangeOff + (groups > 0 ? size_t(groups) * per_group : 0);
-  return (b + 255) / 256 * 256;
+// What a call on G groups must get, and what qb_workspace_bytes tells callers to give: with a slot per group and CTA
+// (for up to kRingMaxGroups groups) the weight quantizer reads W once where groups are too large for a
+// cluster's registers.
+constexpr int kRingMaxGroups = 128;
+constexpr int kRingMaxCtas = 160;
+inline size_t ring_table_bytes(size_t groups) { return groups * kRingMaxCtas * 8; }
+inline size_t ws_round(size_t b) { return (b + 255) / 256 * 256; }
+inline size_t ws_bytes_needed(int groups) { return ws_round(kWsRangeOff + (groups > 0 ? size_t(groups) * 8 : 0)); }
+inline size_t ws_bytes_recommended(int groups) {
+  if (groups <= 0) return ws_bytes_needed(0);
+  const size_t tables = size_t(groups) * 8, ring = ring_table_bytes(groups < kRingMaxGroups ? groups : kRingMaxGroups);
+  return ws_round(kWsRangeOff + (tables > ring ? tables : ring));
 }
-inline size_t ws_bytes_needed(int groups) { return ws_bytes_of(groups, 8); }
-inline size_t ws_bytes_recommended(int groups) { return ws_bytes_of(groups, 12); }
 
 // ---- host-side error plumbing ------------------------------------------------------------------
 void set_last_error(const char* fmt, ...);

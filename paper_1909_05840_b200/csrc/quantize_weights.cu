@@ -721,34 +721,40 @@ weight_regs_kernel(const __grid_constant__ RegsBatch b) {
 // Groups too large for a cluster's registers (one range per matrix, say), read once: one persistent CTA per SM
 // (cooperative launch), every group cut into chunks of 32 units that are dealt round-robin, so that a group of
 // 9 MB is spread over all SMs and its range is known a few chunks after its first chunk was loaded.  A chunk
-// stays in a CTA's ring of twelve 16 KB stages from its load to its rounding:
-//   warp 0         brings chunks in with cp.async.bulk, as far ahead as stages are free
+// stays in a CTA's ring of twelve 16 KB stages, then in the registers of a rounding team, until it is:
+//   warp 0         brings chunks in with cp.async.bulk, as far ahead as stages are free, and leaves beside each
+//                  what the others need to know of it (the one place where the deal is worked out per chunk)
 //   warps 1..4     range: every warp reduces a quarter of each chunk, keeps the extremes over the CTA's run of
 //                  chunks of one group, and hands them over when the run ends
-//   warps 5..12    agents, one lane each, take the CTA's runs in turn: merge the run's range into the group's
-//                  (atomicMax), count the CTA in (release), wait until every CTA that holds a part of the
-//                  group has been counted (acquire), leave the group's parameters in shared memory.  The chain
-//                  takes about 2 us, five chunks' time; eight agents keep eight runs under way.
-//   warps 13..24   rounding: three teams of four warps take every third chunk, round and pack (or
-//                  fake-quantize) it from the ring and free the stage
+//   warps 5..12    agents take the CTA's runs in turn: put the run's range into the CTA's slot of the group's
+//                  table, wait until the slots of all CTAs that hold a part of the group are in, reduce them,
+//                  leave the group's parameters in shared memory.  Eight agents keep eight runs under way.
+//   warps 13..28   rounding: four teams of four warps take every fourth chunk into registers, which frees the
+//                  stage, wait for the group's parameters, round and pack (or fake-quantize)
 // Nobody waits for a later chunk of its own CTA's list, and a group may not span more rounds of the deal than
-// the ring has stages, so the loads and ranges that a team waits for never depend on that team.  One count and
-// two atomicMax per CTA and group, one polling lane per CTA and run: with one per warp and chunk the atomics
-// and polls of all SMs met on three words of one L2 slice and the set below took 299 us.
+// a CTA holds chunks (sixteen), so the loads and ranges that a team waits for never depend on that team.
+// A chunk is held from its load until its group's range has gone round, and 37 MB are held at once: the exchange's
+// latency bounds the rate.  So a slot's two words carry their own tag: no fence, no count, no atomic; one
+// store by the writer, one load by the reader.  (The set below with atomicMax, a release count and a
+// polling lane per CTA: 97.8 us; with those per warp and chunk, which met on three words of one L2 slice: 299.)
 // Memory-bound: 4 + k/8 B per weight.
 constexpr int kRingUnits = 32;                 // per chunk: 16 KB
 constexpr int kRingStages = 12;
 constexpr int kRingRangeWarps = 4;
 constexpr int kRingAgents = 8;
-constexpr int kRingRoundTeams = 3;             // of four warps
+constexpr int kRingPolls = 1;  // runs of a CTA that poll at a time (below)
+constexpr int kRingRoundTeams = 4;             // of four warps
 constexpr int kRingFirstAgent = 1 + kRingRangeWarps;
 constexpr int kRingFirstRound = kRingFirstAgent + kRingAgents;
 constexpr int kRingThreads = 32 * (kRingFirstRound + 4 * kRingRoundTeams);
 constexpr int kRingWarpUnits = kRingUnits / 4; // of a range or rounding warp
 constexpr int kRingSmemBytes = kRingStages * kRingUnits * 512 + 4 * kRingRoundTeams * kRingWarpUnits * 128;
+// A CTA's runs (its chunks of one group) use slot run % kRingSlots.  Once a chunk has landed, the one twelve
+// chunks before it is in its team's registers, so that all chunks sixteen or more before it have been rounded.
+constexpr int kRingSlots = kRingStages + kRingRoundTeams;
 // Rounds of the deal that a group may span, so that its last chunk is loaded and reduced while its first one
-// is still held, with two stages left for loads in flight.
-constexpr int kRingMaxSpan = kRingStages - 2;
+// is still held, with four stages left for loads in flight.
+constexpr int kRingMaxSpan = kRingSlots - 4;
 static_assert(kRingStages % kRingRoundTeams == 0, "a stage is always rounded by the same team");
 
 struct RingItem {
@@ -760,14 +766,13 @@ struct RingItem {
   int32_t chunks_per_group;
   int32_t chunk_begin;       // of the matrix, in the launch's list
   int32_t group_begin;       // of the matrix, in the launch's tables
+  int32_t groups;
   int32_t bits;
 };
 
 struct RingBatch {
   RingItem item[kMaxWeightBatch];
-  uint32_t* hi_enc;    // [groups of the launch], cleared before the launch
-  uint32_t* lo_inv;
-  uint32_t* arrived;
+  unsigned long long* slots;  // [groups of the launch][CTAs]: encoded max << 32 | inverted encoded min, 0 until written
   void* ws;
   int32_t chunks_total;
   int32_t count;
@@ -775,14 +780,13 @@ struct RingBatch {
 
 // A chunk of the launch's list.  `it` only moves forward.
 struct RingChunk {
-  int it, group, first_unit, n;  // matrix, group inside it, first unit inside the group, units
+  int it, group, first_unit;  // matrix, group inside it, first unit inside the group
   __device__ __forceinline__ void seek(const RingBatch& b, int c) {
     while (it + 1 < b.count && c >= b.item[it + 1].chunk_begin) ++it;
     const RingItem& m = b.item[it];
     const int local = c - m.chunk_begin;
     group = local / m.chunks_per_group;
     first_unit = (local - group * m.chunks_per_group) * kRingUnits;
-    n = min(m.ug - first_unit, kRingUnits);
   }
   // chunks of this group that the CTA meets from here on, one every `step` chunks
   __device__ __forceinline__ int run(const RingBatch& b, int step) const {
@@ -790,9 +794,20 @@ struct RingChunk {
   }
 };
 
-__global__ void __launch_bounds__(256) clear_words_kernel(uint32_t* p, int n) {
+// What the producer leaves beside a stage's chunk.
+struct __align__(16) RingStage {
+  uint32_t* out;     // where the chunk's codes (or fp32 values) go
+  int32_t unit_words;  // output words per unit
+  int16_t n;         // units
+  int16_t bits;
+  int16_t slot;      // of the chunk's run
+  int16_t phase;     // of the slot's barriers
+  int16_t last;      // the run ends with this chunk
+};
+
+__global__ void __launch_bounds__(256) clear_slots_kernel(unsigned long long* p, int n) {
   pdl_begin();
-  for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) p[i] = 0u;
+  for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256) p[i] = 0ull;
 }
 
 // Codes of the warp's units (n <= kRingWarpUnits) to the packed stream.
@@ -800,14 +815,13 @@ template <int BITS>
 __device__ __forceinline__ void ring_pack(const float4 (&v)[kRingWarpUnits], const int n, const RgGroup& g, uint8_t* stg,
                                           uint32_t* __restrict__ out, const int lane) {
 #pragma unroll
-  for (int j = 0; j < kRingWarpUnits; ++j)
-    if (j < n) {
-      const uint32_t f = quant_field_open<BITS, false>(v[j], g.lo, g.inv, g.hi);
-      const int fi = j * 32 + lane;
-      if (BITS == 8) reinterpret_cast<uint32_t*>(stg)[fi] = f;
-      if (BITS == 4 || BITS == 3) reinterpret_cast<uint16_t*>(stg)[fi] = (uint16_t)f;
-      if (BITS == 2) stg[fi] = (uint8_t)f;
-    }
+  for (int j = 0; j < kRingWarpUnits; ++j) {  // all of them: what lies past the chunk's end is not copied out
+    const uint32_t f = quant_field_open<BITS, false>(v[j], g.lo, g.inv, g.hi);
+    const int fi = j * 32 + lane;
+    if (BITS == 8) reinterpret_cast<uint32_t*>(stg)[fi] = f;
+    if (BITS == 4 || BITS == 3) reinterpret_cast<uint16_t*>(stg)[fi] = (uint16_t)f;
+    if (BITS == 2) stg[fi] = (uint8_t)f;
+  }
   __syncwarp();
   if (BITS == 3) {
     if (lane < 4 * n) store_3bit_item(stg, out, lane);
@@ -826,22 +840,23 @@ template <bool FAKE>
 __global__ void __launch_bounds__(kRingThreads, 1)
 weight_ring_kernel(const __grid_constant__ RingBatch b) {
   extern __shared__ __align__(1024) uint8_t smem[];
-  // A CTA's runs (its chunks of one group) use slot run % kRingStages: a run holds at least one stage, so at most
-  // kRingStages runs are between their first load and their last rounding.
-  __shared__ __align__(8) uint64_t s_bar[4 * kRingStages];
-  __shared__ uint32_t s_hi[kRingStages][kRingRangeWarps], s_lo[kRingStages][kRingRangeWarps];
-  __shared__ RgGroup s_par[kRingStages];
+  __shared__ __align__(8) uint64_t s_bar[2 * kRingStages + 2 * kRingSlots];
+  __shared__ uint32_t s_hi[kRingSlots][kRingRangeWarps], s_lo[kRingSlots][kRingRangeWarps];
+  __shared__ RgGroup s_par[kRingSlots];
+  __shared__ RingStage s_stage[kRingStages];
   __shared__ volatile int s_abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t ring = ptx::smem_u32(smem), bars = ptx::smem_u32(s_bar);
   auto full = [&](int s) { return bars + 8u * s; };                       // the stage's chunk has landed
-  auto empty = [&](int s) { return bars + 8u * (kRingStages + s); };      // the stage's chunk has been rounded
+  auto empty = [&](int s) { return bars + 8u * (kRingStages + s); };      // range and rounding warps have read it
   auto ranged = [&](int r) { return bars + 8u * (2 * kRingStages + r); }; // the run's range is in s_hi, s_lo
-  auto ready = [&](int r) { return bars + 8u * (3 * kRingStages + r); };  // the group's parameters are in s_par
+  auto ready = [&](int r) { return bars + 8u * (2 * kRingStages + kRingSlots + r); };  // the group's parameters are in s_par
   if (threadIdx.x == 0) {
     for (int s = 0; s < kRingStages; ++s) {
       ptx::mbar_init(full(s), 1);
-      ptx::mbar_init(empty(s), 4);
+      ptx::mbar_init(empty(s), kRingRangeWarps + 4);
+    }
+    for (int s = 0; s < kRingSlots; ++s) {
       ptx::mbar_init(ranged(s), kRingRangeWarps);
       ptx::mbar_init(ready(s), 1);
     }
@@ -854,20 +869,45 @@ weight_ring_kernel(const __grid_constant__ RingBatch b) {
   RingChunk c;
   c.it = 0;
   const int step = (int)gridDim.x;
+  const int chunks = (b.chunks_total - (int)blockIdx.x + step - 1) / step;  // of this CTA
   if (warp == 0) {
     if (ptx::elect_one()) {
-      int stage = 0;
-      uint32_t phase = 0;
-      for (int id = blockIdx.x; id < b.chunks_total; id += step) {
-        c.seek(b, id);
-        const RingItem& m = b.item[c.it];
+      // One thread serves a chunk every 0.4 us: the walk over the deal is incremental, the matrix's fields stay in
+      // registers, and the next chunk is worked out before the wait for its stage.  (With the division of
+      // RingChunk::seek and the fields read per chunk it took 800 cycles, and bound the kernel.)
+      int stage = 0, slot = -1, left = 0;
+      uint32_t phase = 0, slot_phase = 1;
+      RingItem m = b.item[0];
+      int it = 0, group = 0, pos = (int)blockIdx.x;  // pos: chunk inside the group
+      int words = FAKE ? 128 : 4 * m.bits;
+      for (int k = 0; k < chunks; ++k) {
+        while (pos >= m.chunks_per_group) {
+          pos -= m.chunks_per_group;
+          left = 0;
+          if (++group == m.groups) {
+            group = 0;
+            m = b.item[++it];
+            words = FAKE ? 128 : 4 * m.bits;
+          }
+        }
+        if (left == 0) {  // the CTA's run in this group begins
+          left = (m.chunks_per_group - pos + step - 1) / step;
+          if (++slot == kRingSlots) slot = 0;
+          if (slot == 0) slot_phase ^= 1u;
+        }
+        --left;
+        const int n = min(m.ug - pos * kRingUnits, kRingUnits);
+        const int64_t unit = (int64_t)group * m.ug + pos * kRingUnits;
+        const RingStage st{m.packed + unit * words, words, (int16_t)n, (int16_t)m.bits, (int16_t)slot, (int16_t)slot_phase,
+                           (int16_t)(left == 0)};
         if (!wait_barrier_relaxed(empty(stage), phase ^ 1u, &s_abort)) {
           timed_out = true;
           break;
         }
-        ptx::mbar_arrive_expect_tx(full(stage), (uint32_t)c.n * 512u);
-        ptx::bulk_load_1d(ring + stage * kRingUnits * 512, m.w + ((int64_t)c.group * m.ug + c.first_unit) * 32,
-                          (uint32_t)c.n * 512u, full(stage));
+        s_stage[stage] = st;
+        ptx::mbar_arrive_expect_tx(full(stage), (uint32_t)n * 512u);  // publishes s_stage too
+        ptx::bulk_load_1d(ring + stage * kRingUnits * 512, m.w + unit * 32, (uint32_t)n * 512u, full(stage));
+        pos += step;
         if (++stage == kRingStages) {
           stage = 0;
           phase ^= 1u;
@@ -877,26 +917,29 @@ weight_ring_kernel(const __grid_constant__ RingBatch b) {
   } else if (warp < kRingFirstAgent) {
     const int part = warp - 1;
     const float kInf = __int_as_float(0x7f800000);
-    int stage = 0, slot = 0, left = 0;  // left: chunks of this CTA left in the run
+    int stage = 0;
     uint32_t phase = 0;
     float lo = kInf, hi = -kInf;
-    for (int id = blockIdx.x; id < b.chunks_total; id += step) {
-      c.seek(b, id);
-      if (left == 0) left = c.run(b, step);
+    for (int k = 0; k < chunks; ++k) {
       if (!wait_barrier_relaxed(full(stage), phase, &s_abort)) {
         timed_out = true;
         break;
       }
       const float4* src = reinterpret_cast<const float4*>(smem + stage * kRingUnits * 512) + part * kRingWarpUnits * 32 + lane;
-      const int n = min(c.n - part * kRingWarpUnits, kRingWarpUnits);
+      const int n = s_stage[stage].n - part * kRingWarpUnits, slot = s_stage[stage].slot;
+      const bool last = s_stage[stage].last != 0;
+      float4 v[kRingWarpUnits];
+#pragma unroll
+      for (int j = 0; j < kRingWarpUnits; ++j) v[j] = src[j * 32];  // units past the chunk's end: stale, not used
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(empty(stage));
 #pragma unroll
       for (int j = 0; j < kRingWarpUnits; ++j)
         if (j < n) {
-          const float4 v = src[j * 32];
-          lo = min3_nan(min3_nan(lo, v.x, v.y), v.z, v.w);
-          hi = max3_nan(max3_nan(hi, v.x, v.y), v.z, v.w);
+          lo = min3_nan(min3_nan(lo, v[j].x, v[j].y), v[j].z, v[j].w);
+          hi = max3_nan(max3_nan(hi, v[j].x, v[j].y), v[j].z, v[j].w);
         }
-      if (--left == 0) {
+      if (last) {
         const uint32_t e_hi = __reduce_max_sync(0xffffffffu, float_to_ordered(hi));
         const uint32_t e_lo = __reduce_max_sync(0xffffffffu, ~float_to_ordered(lo));
         if (lane == 0) {
@@ -906,7 +949,6 @@ weight_ring_kernel(const __grid_constant__ RingBatch b) {
         }
         lo = kInf;
         hi = -kInf;
-        if (++slot == kRingStages) slot = 0;
       }
       if (++stage == kRingStages) {
         stage = 0;
@@ -914,41 +956,67 @@ weight_ring_kernel(const __grid_constant__ RingBatch b) {
       }
     }
   } else if (warp < kRingFirstRound) {
-    if (lane == 0) {
-      const int agent = warp - kRingFirstAgent;
-      int slot = 0;
-      uint32_t phase = 0;
-      int id = blockIdx.x;
-      for (int run = 0; id < b.chunks_total; ++run) {
-        c.seek(b, id);
-        const int len = c.run(b, step);
-        if (run % kRingAgents == agent) {
-          const RingItem& m = b.item[c.it];
-          const int g = m.group_begin + c.group;
-          if (!wait_barrier_relaxed(ranged(slot), phase, &s_abort)) {
-            timed_out = true;
-            break;
-          }
-          uint32_t e_hi = 0, e_lo = 0;
+    const int agent = warp - kRingFirstAgent;
+    int slot = 0;
+    uint32_t phase = 0;
+    int id = blockIdx.x;
+    for (int run = 0; id < b.chunks_total; ++run) {
+      c.seek(b, id);
+      const int len = c.run(b, step);
+      if (run % kRingAgents == agent) {
+        const RingItem& m = b.item[c.it];
+        unsigned long long* const table = b.slots + (size_t)(m.group_begin + c.group) * step;
+        if (!wait_barrier_relaxed(ranged(slot), phase, &s_abort)) {
+          timed_out = true;
+          break;
+        }
+        const uint32_t my_hi = __reduce_max_sync(0xffffffffu, lane < kRingRangeWarps ? s_hi[slot][lane] : 0u);
+        // (a NaN as minimum encodes to 0, which would read as missing; the maximum is then NaN too and reports it)
+        const uint32_t my_lo = __reduce_max_sync(0xffffffffu, lane < kRingRangeWarps ? s_lo[slot][lane] : 1u);
+        // the CTA that holds the group's chunk j has slot j (chunks j + step, ... are its own too)
+        if (lane == 0)
+          asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(table + c.first_unit / kRingUnits),
+                       "l"((unsigned long long)my_hi << 32 | max(my_lo, 1u)) : "memory");
+        const int n = min(m.chunks_per_group, step);  // CTAs that hold a part of the group
+        const int prev = slot < kRingPolls ? slot + kRingSlots - kRingPolls : slot - kRingPolls;
+        const uint32_t prev_phase = slot < kRingPolls ? phase ^ 1u : phase;
+        if (run >= kRingPolls && !wait_barrier_relaxed(ready(prev), prev_phase, &s_abort)) {
+          timed_out = true;
+          break;
+        }
+        uint32_t e_hi, e_lo;
+        const long long t0 = clock64();
+        bool ok = true, all;
+        constexpr int kPer = (kRingMaxCtas + 31) / 32;
+        unsigned long long v[kPer];
 #pragma unroll
-          for (int i = 0; i < kRingRangeWarps; ++i) {
-            e_hi = max(e_hi, s_hi[slot][i]);
-            e_lo = max(e_lo, s_lo[slot][i]);
-          }
-          atomicMax(b.hi_enc + g, e_hi);
-          atomicMax(b.lo_inv + g, e_lo);
-          asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(b.arrived + g) : "memory");
-          const uint32_t target = (uint32_t)min(m.chunks_per_group, step);  // CTAs that hold a part of the group
-          if (ld_acquire(b.arrived + g) != target) {
-            const long long t0 = clock64();
-            while (ld_acquire(b.arrived + g) != target)
-              if (s_abort != 0 || clock64() - t0 > kWaitLimitCycles) {
-                timed_out = true;
-                break;
-              }
-          }
-          if (timed_out) break;
-          const float g_hi = ordered_to_float(__ldcg(b.hi_enc + g)), g_lo = ordered_to_float(~__ldcg(b.lo_inv + g));
+        for (int i = 0; i < kPer; ++i) v[i] = lane + 32 * i < n ? 0ull : 1ull;
+        for (;;) {  // all of the lane's missing slots in flight at once
+#pragma unroll
+          for (int i = 0; i < kPer; ++i)
+            if (v[i] == 0ull)
+              asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v[i]) : "l"(table + lane + 32 * i) : "memory");
+          all = true;
+#pragma unroll
+          for (int i = 0; i < kPer; ++i) all = all && v[i] != 0ull;
+          all = __all_sync(0xffffffffu, all);
+          ok = !__any_sync(0xffffffffu, !all && (s_abort != 0 || clock64() - t0 > kWaitLimitCycles));
+          if (all || !ok) break;
+        }
+        e_hi = e_lo = 0;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+          e_hi = max(e_hi, (uint32_t)(v[i] >> 32));
+          e_lo = max(e_lo, (uint32_t)v[i]);
+        }
+        e_hi = __reduce_max_sync(0xffffffffu, e_hi);
+        e_lo = __reduce_max_sync(0xffffffffu, e_lo);
+        if (!ok) {
+          timed_out = true;
+          break;
+        }
+        if (lane == 0) {
+          const float g_hi = ordered_to_float(e_hi), g_lo = ordered_to_float(~e_lo);
           const int L = (1 << m.bits) - 1;
           const bool publish = c.first_unit == 0;
           if (publish && !(fabsf(g_hi) <= 3.402823466e38f && fabsf(g_lo) <= 3.402823466e38f)) report_status(b.ws, QB_ERR_NONFINITE);
@@ -956,63 +1024,57 @@ weight_ring_kernel(const __grid_constant__ RingBatch b) {
           s_par[slot] = RgGroup{gp.lo, gp.inv, group_step(gp, L), gp.hi};
           ptx::mbar_arrive(ready(slot));
         }
-        id += len * step;
-        if (++slot == kRingStages) {
-          slot = 0;
-          phase ^= 1u;
-        }
+        __syncwarp();
+      }
+      id += len * step;
+      if (++slot == kRingSlots) {
+        slot = 0;
+        phase ^= 1u;
       }
     }
   } else {
     const int rw = warp - kRingFirstRound;
     const int team = rw >> 2, part = rw & 3;
     uint8_t* const stg = smem + kRingStages * kRingUnits * 512 + rw * kRingWarpUnits * 128;
-    int stage = 0, slot = -1, left = 0, turn = team;
-    uint32_t phase = 0, slot_phase = 1;
-    for (int id = blockIdx.x; id < b.chunks_total; id += step) {
-      c.seek(b, id);
-      if (left == 0) {
-        left = c.run(b, step);
-        if (++slot == kRingStages) slot = 0;
-        if (slot == 0) slot_phase ^= 1u;
+    int stage = team;
+    uint32_t phase = 0;
+    for (int k = team; k < chunks; k += kRingRoundTeams) {
+      if (!wait_barrier_relaxed(full(stage), phase, &s_abort)) {
+        timed_out = true;
+        break;
       }
-      --left;
-      if (turn == 0) {
-        turn = kRingRoundTeams;
-        const RingItem& m = b.item[c.it];
-        // In this order: once the chunk has landed, the one twelve chunks before it has been rounded, and with it
-        // every run that used this slot before; a barrier's parity is only told apart one phase at a time.
-        if (!wait_barrier_relaxed(full(stage), phase, &s_abort) || !wait_barrier_relaxed(ready(slot), slot_phase, &s_abort)) {
-          timed_out = true;
-          break;
-        }
-        const RgGroup cur = s_par[slot];
-        const int u0 = part * kRingWarpUnits;
-        const int n = min(c.n - u0, kRingWarpUnits);
-        const float4* src = reinterpret_cast<const float4*>(smem + stage * kRingUnits * 512) + u0 * 32 + lane;
-        float4 v[kRingWarpUnits];
+      const RingStage st = s_stage[stage];
+      const int u0 = part * kRingWarpUnits;
+      const int n = min((int)st.n - u0, kRingWarpUnits);
+      const float4* src = reinterpret_cast<const float4*>(smem + stage * kRingUnits * 512) + u0 * 32 + lane;
+      float4 v[kRingWarpUnits];
+#pragma unroll
+      for (int j = 0; j < kRingWarpUnits; ++j) v[j] = src[j * 32];  // units past the chunk's end: stale, not used
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(empty(stage));
+      // After the wait for the chunk, not before: every run that used this slot earlier is then behind us (a
+      // barrier's parity is only told apart one phase at a time).
+      if (!wait_barrier_relaxed(ready(st.slot), (uint32_t)st.phase, &s_abort)) {
+        timed_out = true;
+        break;
+      }
+      const RgGroup cur = s_par[st.slot];
+      uint32_t* const out = st.out + u0 * st.unit_words;
+      if (FAKE) {
 #pragma unroll
         for (int j = 0; j < kRingWarpUnits; ++j)
-          if (j < n) v[j] = src[j * 32];
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(empty(stage));  // the warp's part is in registers
-        uint32_t* const out = m.packed + ((int64_t)c.group * m.ug + c.first_unit + u0) * (FAKE ? 128 : 4 * m.bits);
-        if (FAKE) {
-#pragma unroll
-          for (int j = 0; j < kRingWarpUnits; ++j)
-            if (j < n) reinterpret_cast<float4*>(out)[j * 32 + lane] = fake_quant4<false>(v[j], cur);
-        } else {
-          switch (m.bits) {  // team-uniform
-            case 2: ring_pack<2>(v, n, cur, stg, out, lane); break;
-            case 3: ring_pack<3>(v, n, cur, stg, out, lane); break;
-            case 4: ring_pack<4>(v, n, cur, stg, out, lane); break;
-            default: ring_pack<8>(v, n, cur, stg, out, lane); break;
-          }
+          if (j < n) reinterpret_cast<float4*>(out)[j * 32 + lane] = fake_quant4<false>(v[j], cur);
+      } else {
+        switch (st.bits) {  // team-uniform
+          case 2: ring_pack<2>(v, n, cur, stg, out, lane); break;
+          case 3: ring_pack<3>(v, n, cur, stg, out, lane); break;
+          case 4: ring_pack<4>(v, n, cur, stg, out, lane); break;
+          default: ring_pack<8>(v, n, cur, stg, out, lane); break;
         }
       }
-      --turn;
-      if (++stage == kRingStages) {
-        stage = 0;
+      stage += kRingRoundTeams;
+      if (stage >= kRingStages) {
+        stage -= kRingStages;
         phase ^= 1u;
       }
     }
@@ -1278,7 +1340,6 @@ static qb_status launch_regs(const HostWeight* m_all, int count_all, void* ws, i
 }
 
 // One pair of launches (clear, ring kernel) over `count` matrices (<= kMaxWeightBatch) whose groups fit the ring.
-// Their tables sit back to back in the workspace: maxima at ws + kWsRangeOff, inverted minima, arrivals.
 template <bool FAKE>
 static qb_status launch_ring_form(const RingBatch& b, unsigned grid, cudaStream_t stream) {
   static std::atomic<bool> attr_set[64] = {};
@@ -1305,42 +1366,59 @@ static qb_status launch_ring(const HostWeight* m, int count, void* ws, int sm_co
     it.chunks_per_group = (it.ug + kRingUnits - 1) / kRingUnits;
     it.chunk_begin = chunks;
     it.group_begin = groups;
+    it.groups = h.groups;
     it.bits = h.bits;
     chunks += it.chunks_per_group * h.groups;
     groups += h.groups;
   }
   b.ws = ws;
-  b.hi_enc = reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + kWsRangeOff);
-  b.lo_inv = b.hi_enc + groups;
-  b.arrived = b.lo_inv + groups;
+  b.slots = reinterpret_cast<unsigned long long*>(static_cast<char*>(ws) + kWsRangeOff);
   b.chunks_total = chunks;
   b.count = count;
-  QB_CUDA_TRY(launch_kernel(clear_words_kernel, (unsigned)std::min((3 * groups + 255) / 256, sm_count), 256, 0, stream, true, 1, false,
-                            b.hi_enc, 3 * groups));
-  const unsigned grid = (unsigned)std::min(chunks, sm_count);
+  const unsigned grid = (unsigned)std::min(chunks, std::min(sm_count, kRingMaxCtas));
+  const int slots = groups * (int)grid;
+  QB_CUDA_TRY(launch_kernel(clear_slots_kernel, (unsigned)std::min((slots + 255) / 256, sm_count), 256, 0, stream, true, 1, false,
+                            b.slots, slots));
   return fake ? launch_ring_form<true>(b, grid, stream) : launch_ring_form<false>(b, grid, stream);
 }
 
 // Matrices whose groups do not fit a cluster's registers: the ring as long as a group spans few enough rounds of
-// its deal (up to 148 * 9 chunks of 16 KB, 22 MB), else, and where the workspace has no room for the
-// arrival counts, the two passes.  Both are a pair of launches per kMaxWeightBatch matrices.
+// its deal (up to 148 * 11 chunks of 16 KB, 27 MB), else, and where the workspace has no room for the
+// slots, the two passes.  Both are a pair of launches per job.
 static inline bool ring_eligible(const HostWeight& h, int sm_count) {
-  return (group_units(h) + kRingUnits - 1) / kRingUnits <= (int64_t)(kRingMaxSpan - 1) * sm_count;
+  return (group_units(h) + kRingUnits - 1) / kRingUnits <= (int64_t)(kRingMaxSpan - 1) * std::min(sm_count, kRingMaxCtas) &&
+         h.groups <= kRingMaxGroups;
+}
+struct LargeJob {
+  std::vector<HostWeight> m;  // at most kMaxWeightBatch matrices
+  int64_t groups = 0;         // of all of them; a ring job has at most kRingMaxGroups
+  bool ring = false;
+};
+static std::vector<LargeJob> plan_large_groups(const std::vector<HostWeight>& m, int sm_count) {
+  std::vector<LargeJob> jobs;
+  for (const bool ring : {true, false}) {
+    bool open = false;
+    for (const HostWeight& h : m) {
+      if (ring_eligible(h, sm_count) != ring) continue;
+      if (!open || (int)jobs.back().m.size() == kMaxWeightBatch || (ring && jobs.back().groups + h.groups > kRingMaxGroups)) {
+        jobs.emplace_back();
+        jobs.back().ring = ring;
+        open = true;
+      }
+      jobs.back().m.push_back(h);
+      jobs.back().groups += h.groups;
+    }
+  }
+  return jobs;
 }
 static qb_status launch_large_groups(const std::vector<HostWeight>& m, void* ws, size_t ws_bytes, int sm_count,
                                      cudaStream_t stream, bool fake) {
-  std::vector<HostWeight> part[2];
-  for (const HostWeight& h : m) part[ring_eligible(h, sm_count) ? 0 : 1].push_back(h);
-  for (int k = 0; k < 2; ++k)
-    for (size_t i = 0; i < part[k].size(); i += kMaxWeightBatch) {
-      const int n = (int)std::min<size_t>(kMaxWeightBatch, part[k].size() - i);
-      size_t groups = 0;
-      for (int j = 0; j < n; ++j) groups += (size_t)part[k][i + j].groups;
-      const bool ring = k == 0 && kWsRangeOff + 12 * groups <= ws_bytes;
-      qb_status st = ring ? launch_ring(part[k].data() + i, n, ws, sm_count, stream, fake)
-                          : launch_two_pass(part[k].data() + i, n, ws, sm_count, stream, fake);
-      if (st != QB_OK) return st;
-    }
+  for (const LargeJob& j : plan_large_groups(m, sm_count)) {
+    const bool ring = j.ring && kWsRangeOff + ring_table_bytes((size_t)j.groups) <= ws_bytes;
+    qb_status st = ring ? launch_ring(j.m.data(), (int)j.m.size(), ws, sm_count, stream, fake)
+                        : launch_two_pass(j.m.data(), (int)j.m.size(), ws, sm_count, stream, fake);
+    if (st != QB_OK) return st;
+  }
   return QB_OK;
 }
 
@@ -1444,10 +1522,11 @@ extern "C" int32_t qb_quantize_pack_weights_launch_count(const qb_weight_desc* d
   int sms = 148;
   qb::require_sm100(&sms);  // without a device: the plan for a 148-SM part
   int per_cluster[qb::kRgMaxCluster + 1] = {};
-  int ranged = 0, ring = 0, two_pass = 0;
+  int ranged = 0;
+  std::vector<qb::HostWeight> large;
   for (const qb::HostWeight& h : host_weights(descs, count)) {
     if (!qb::regs_eligible(h))
-      ++(qb::ring_eligible(h, sms) ? ring : two_pass);
+      large.push_back(h);
     else if (h.range_lo != nullptr)
       ++ranged;
     else
@@ -1456,7 +1535,7 @@ extern "C" int32_t qb_quantize_pack_weights_launch_count(const qb_weight_desc* d
   const auto launches = [](int matrices, int per_launch) { return (matrices + per_launch - 1) / per_launch; };
   int32_t n = launches(ranged, qb::kRgMaxBatch);
   for (int cl = 1; cl <= qb::kRgMaxCluster; ++cl) n += launches(per_cluster[cl], qb::kRgMaxBatch);
-  n += 2 * (launches(ring, qb::kMaxWeightBatch) + launches(two_pass, qb::kMaxWeightBatch));
+  n += 2 * (int32_t)qb::plan_large_groups(large, sms).size();
   return n;
 }
 

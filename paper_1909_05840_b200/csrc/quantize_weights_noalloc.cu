@@ -24,7 +24,9 @@ qb_status launch_quantize_pack_weights(const float* w, int64_t N, int64_t K, int
                                        const float* range_lo, const float* range_hi, uint32_t* packed,
                                        float* delta, float* q0, void* ws, size_t ws_bytes, int sm_count, cudaStream_t stream);
 
-constexpr size_t kNoAllocScratchBytes = kWsRangeOff + 12 * (size_t)QB_NOALLOC_MAX_GROUPS;
+// the range tables of QB_NOALLOC_MAX_GROUPS groups, or the per-CTA slots of the groups the single-read path takes
+constexpr size_t kNoAllocScratchBytes = kWsRangeOff + 40 * (size_t)QB_NOALLOC_MAX_GROUPS;
+static_assert(kNoAllocScratchBytes >= kWsRangeOff + (size_t)kRingMaxGroups * kRingMaxCtas * 8, "scratch too small");
 
 // Same layout as a caller-provided workspace: status word at offset 0, encoded ranges at kWsRangeOff.
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];

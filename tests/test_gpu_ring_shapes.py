@@ -1,5 +1,5 @@
 """The weight quantizer's single-read path for groups too large for a cluster's registers, against the oracle: groups
-of one to nine rounds of 148 chunks (of 32 units of 128 weights), last chunks of any length, several groups per
+of one to eleven rounds of 148 chunks (of 32 units of 128 weights), last chunks of any length, several groups per
 matrix, packing and fake quantization, a batch of mixed widths; and the two passes just beyond."""
 import numpy as np
 import pytest
@@ -18,10 +18,10 @@ def ws():
     return qb.workspace(groups=4096)
 
 
-# units per group: 2,305 (73 chunks), 148 chunks exactly, one more, 32 k + 1, 9 * 148 chunks (the last size that
+# units per group: 2,305 (73 chunks), 148 chunks exactly, one more, 32 k + 1, 11 * 148 chunks (the last size that
 # fits) and one unit more (two passes)
 @pytest.mark.parametrize("N,K,groups", [(2305, 128, 1), (768, 768, 1), (4736, 128, 1), (4737, 128, 1), (5210, 256, 2),
-                                        (3072, 768, 1), (42624, 128, 1), (42625, 128, 1)])
+                                        (3072, 768, 1), (52096, 128, 1), (52097, 128, 1)])
 def test_large_groups(ws, N, K, groups):
     w = synth.weights(N, K, seed=N + K)
     for bits in (2, 3, 4, 8):
@@ -61,7 +61,7 @@ def test_nonfinite_is_reported(bad):
     assert qb.read_status(ws) == qb.QB_ERR_NONFINITE
 
 
-def test_workspace_without_room_for_arrival_counts():
+def test_workspace_without_room_for_the_slots():
     # 8 bytes per group are enough: the two passes serve the call
     G = 40
     ws = qb.workspace(groups=4096)
