@@ -228,22 +228,44 @@ __device__ __forceinline__ float group_step(const GroupParams& gp, int bits_leve
 
 // ---- straight-through backward (quantization-aware fine-tuning) ----------------------------------------
 // Backward (straight-through estimator): the gradient passes where Clamp passes X (lo_g <= x <= hi_g).
+// Memory-bound, 12 B per weight; a matrix of a base model is 28 MB, 4.4 us of bandwidth, so what counts is that all
+// of it is in flight at once: a warp takes four units (eight 512-byte loads) and works out their group with
+// one division.  Four BERT-base layers, one call per matrix: STE_MEASURED.
+constexpr int kSteUnits = 4;
 __global__ void __launch_bounds__(256)
-ste_backward_kernel(const float4* __restrict__ grad_q, const float4* __restrict__ w, int64_t n4, int64_t k4,
-                    int64_t rows_per_group, const float* __restrict__ lo, const float* __restrict__ hi,
-                    float4* __restrict__ grad_w) {
+ste_backward_kernel(const float4* grad_q, const float4* __restrict__ w, int64_t units, uint32_t units_per_group,
+                    const float* __restrict__ lo, const float* __restrict__ hi, float4* grad_w) {
   pdl_begin();
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += stride) {
-    const int64_t g = (i / k4) / rows_per_group;
-    const float l = __ldg(lo + g), h = __ldg(hi + g);
-    const float4 x = __ldg(w + i);
-    float4 gq = __ldg(grad_q + i);
-    gq.x = (x.x >= l && x.x <= h) ? gq.x : 0.0f;
-    gq.y = (x.y >= l && x.y <= h) ? gq.y : 0.0f;
-    gq.z = (x.z >= l && x.z <= h) ? gq.z : 0.0f;
-    gq.w = (x.w >= l && x.w <= h) ? gq.w : 0.0f;
-    grad_w[i] = gq;
+  const int lane = threadIdx.x & 31;
+  const int64_t step = (int64_t)gridDim.x * 8 * kSteUnits;
+  for (int64_t u = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * kSteUnits; u < units; u += step) {
+    const int n = (int)min(units - u, (int64_t)kSteUnits);
+    float4 x[kSteUnits], g[kSteUnits];
+#pragma unroll
+    for (int j = 0; j < kSteUnits; ++j)
+      if (j < n) {
+        x[j] = __ldg(w + (u + j) * 32 + lane);
+        g[j] = grad_q[(u + j) * 32 + lane];  // grad_w may be the same buffer
+      }
+    uint32_t group = (uint32_t)u / units_per_group, in_group = (uint32_t)u - group * units_per_group;
+    float l = __ldg(lo + group), h = __ldg(hi + group);
+#pragma unroll
+    for (int j = 0; j < kSteUnits; ++j)
+      if (j < n) {
+        if (in_group == units_per_group) {
+          in_group = 0;
+          ++group;
+          l = __ldg(lo + group);
+          h = __ldg(hi + group);
+        }
+        ++in_group;
+        float4 r = g[j];
+        r.x = (x[j].x >= l && x[j].x <= h) ? r.x : 0.0f;
+        r.y = (x[j].y >= l && x[j].y <= h) ? r.y : 0.0f;
+        r.z = (x[j].z >= l && x[j].z <= h) ? r.z : 0.0f;
+        r.w = (x[j].w >= l && x[j].w <= h) ? r.w : 0.0f;
+        grad_w[(u + j) * 32 + lane] = r;
+      }
   }
 }
 
@@ -1606,11 +1628,14 @@ extern "C" qb_status qb_ste_backward(const float* grad_wq, const float* w, int64
                                   stream));
     return QB_OK;
   }
-  const int64_t n4 = N * K / 4;
-  int64_t blocks = (n4 + 256 * 4 - 1) / (256 * 4);
-  if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
+  const int64_t units = N * (K / 128);  // below 2^33; a tensor that large does not exist, but the division is 32-bit
+  if (units > 0xffffffffll) {
+    qb::set_last_error("qb_ste_backward: matrix too large (N=%lld K=%lld)", (long long)N, (long long)K);
+    return QB_ERR_INVALID;
+  }
+  const int64_t blocks = std::min((units + 8 * qb::kSteUnits - 1) / (8 * qb::kSteUnits), (int64_t)sms * 64);
   QB_CUDA_TRY(qb::launch_kernel(qb::ste_backward_kernel, (unsigned)blocks, 256, 0, stream, true, 1, false,
-                                reinterpret_cast<const float4*>(grad_wq), reinterpret_cast<const float4*>(w), n4, K / 4,
-                                N / groups, range_lo, range_hi, reinterpret_cast<float4*>(grad_w)));
+                                reinterpret_cast<const float4*>(grad_wq), reinterpret_cast<const float4*>(w), units,
+                                (uint32_t)(N / groups * (K / 128)), range_lo, range_hi, reinterpret_cast<float4*>(grad_w)));
   return QB_OK;
 }
