@@ -352,8 +352,8 @@ qb_status qb_fake_quantize_weights_batch(const qb_weight_desc* descs /*host*/, i
  *   packed   dev uint32 [V][D*bits/32], 16-byte aligned           (written)
  *   delta,q0 dev fp32 [G]                                         (written)
  * D must be a multiple of 128, at most 4096, and divisible by G.  The workspace must hold
- * qb_workspace_bytes(0, 0, 0, 0, D) bytes (8 per column).  Two kernels: per-column min/max into the
- * workspace, then round/clamp/pack.
+ * qb_workspace_bytes(0, 0, 0, 0, D) bytes.  Two kernels: per-group min/max into the workspace, then
+ * round/clamp/pack.
  *
  * qb_embedding_lookup gathers and dequantizes: out[t][d] = Delta_g * code[ids[t]][d] + q0_g (one fused
  * multiply-add), g = d / (D / G); with accumulate != 0 that value is added to what `out` holds (one
