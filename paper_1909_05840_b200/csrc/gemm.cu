@@ -135,7 +135,7 @@ struct GemmCfg {
   static constexpr int kXBytes = kXRows * kBlockK;
   static constexpr int kStageBytes = kWBytes + kXBytes;
   static constexpr int kStages = (kStageBytes == 48 * 1024) ? 3 : 5;
-  static constexpr int kTmemCols = 2 * BT;
+  static constexpr int kTmemCols = BT == 192 ? 512 : 2 * BT;  // a power of two
   static constexpr int kBarBytes = 256 + 2 * 256 * 4;  // barriers + two row-sum tiles
   static constexpr int kOutStageBytes = kEpilogueWarps * 2 * 32 * 32 * 4;  // per epilogue warp: two buffers of 32 tokens x 32 neurons fp32
   static constexpr int kSmemBytes = kStages * kStageBytes + kOutStageBytes + kBarBytes;
@@ -1008,9 +1008,10 @@ static qb_status launch_group_bits(int bits, const GP& gp, int grid, cudaStream_
 }
 
 // Token-tile width for a launch: 256 tokens unless every problem has at most 128 or the launch is too
-// small to give every SM a 256-token tile.  The 128-wide instruction takes as long as the 256-wide one
-// (measured with qb_probe_i8_mma: 498 vs 512 cycles per K block), so narrow tiles halve the tensor rate
-// and double the weight expansion per token; they pay only when SMs would otherwise idle.
+// small to give every SM a 256-token tile.  Narrow tiles double the weight expansion per token; they pay only
+// when SMs would otherwise idle.  (The instruction itself takes half as long at half the width: 256 cycles per K block
+// at 128 tokens, 384 at 192, 512 at 256, when the issuing thread is elected, so that its operands stay in
+// uniform registers; issued from an ordinary thread every width takes about 500.)
 // `cg_out`: CTAs per tile.  A launch with at least one 256 x 256 tile per pair of SMs runs as CTA pairs: each
 // CTA then stages half of the token tile (half the L2 and shared-memory traffic per MMA) and the ring is
 // five K blocks deep instead of three.
@@ -1025,7 +1026,29 @@ static int choose_token_tile(const qb_linear_desc* d, const int* idx, int count,
   *cg_out = 1;
   if (wide && sm_count >= 2 && tiles_pair >= sm_count / 2 && g_pair_mode != 0) {
     *cg_out = 2;
-    return 256;
+    // 192 tokens per tile when that leaves the pairs less idle at the end.  Measured per tile (12 and 16 full rounds of
+    // all pairs, 4 bits, hundredths of a microsecond): 283 + 37 per K block at 256 tokens, 222 + 31 at 192, that
+    // is 8-10 % more per token; 6144 x 4096 x 1024 (5.2 rounds of 256-token tiles) 41.2 -> 38.9 us,
+    // 6144 x 1024 x 4096 (1.3 rounds) 33.8 -> 29.5 us.
+    const int pairs = sm_count / 2;
+    int64_t est[2];
+    for (int w = 0; w < 2; ++w) {
+      const int bt = w ? 192 : 256;
+      int64_t sum = 0, longest = 0, tiles = 0;
+      bool uniform = true;
+      for (int i = 0; i < count; ++i) {
+        const qb_linear_desc& q = d[idx[i]];
+        const int64_t n = ((q.N + 2 * kTileN - 1) / (2 * kTileN)) * ((q.M + bt - 1) / bt);
+        const int64_t cost = w ? 222 + 31 * (q.K / kBlockK) : 283 + 37 * (q.K / kBlockK);
+        tiles += n;
+        sum += n * cost;
+        longest = std::max(longest, cost);
+        uniform = uniform && q.K == d[idx[0]].K;
+      }
+      // tiles of one length: whole rounds; of several: the balanced lists end about half a long tile apart
+      est[w] = uniform ? (tiles + pairs - 1) / pairs * longest : sum / pairs + longest / 2;
+    }
+    return est[1] < est[0] ? 192 : 256;
   }
   // a launch that cannot give every SM a 256-token tile uses 128-token tiles: twice the CTAs at work,
   // half the epilogue per tile
@@ -1113,7 +1136,9 @@ template <int OUT, class GP>
 static qb_status launch_group_out(int bits, int bt, int cg, const GP& gp, int grid, cudaStream_t stream) {
   if constexpr (GP::kProblems > 1)
     if (bits == 0) return launch_group_inst<128, 0, OUT, 1>(gp, grid, stream);
-  if (cg == 2) return launch_group_bits<256, OUT, 2>(bits, gp, 2 * grid, stream);
+  if (cg == 2)
+    return bt == 256 ? launch_group_bits<256, OUT, 2>(bits, gp, 2 * grid, stream)
+                     : launch_group_bits<192, OUT, 2>(bits, gp, 2 * grid, stream);
   return bt == 256 ? launch_group_bits<256, OUT, 1>(bits, gp, grid, stream)
                    : launch_group_bits<128, OUT, 1>(bits, gp, grid, stream);
 }
