@@ -84,7 +84,9 @@ qb_status qb_read_status(const void* ws /*dev*/, void* cuda_stream);
  *   xq        dev, int8 [M][K], 16-byte aligned          (written)
  *   act_scale dev, fp32 [1]                              (written)
  *   rowsum    dev, int32 [M]                             (written)
- * Two kernels: a grid-wide max-abs reduction into the workspace, then round/clamp/store.
+ * One kernel for tensors of up to 32 segments (of up to 1,024 elements of a row) per SM, which stay in registers
+ * while the blocks agree on the maximum; else two: a grid-wide max-abs reduction into the workspace, then
+ * round/store.
  */
 qb_status qb_quantize_act(const float* x, int64_t M, int64_t K, int8_t* xq, float* act_scale,
                           int32_t* rowsum, void* ws, size_t ws_bytes, void* cuda_stream);
@@ -106,8 +108,10 @@ qb_status qb_quantize_act(const float* x, int64_t M, int64_t K, int8_t* xq, floa
  * One kernel (the weights are read once and stay in registers between the range and the rounding)
  * when the range is the group's own and the groups have at most 294,912 weights each (groups above
  * 36,864 weights are held by a thread-block cluster), and always with caller-supplied ranges
- * (nothing is reduced then); otherwise two kernels: per-group min/max reduction into the workspace,
- * then round/clamp/pack.
+ * (nothing is reduced then).  Otherwise two: for groups of up to about 27 MB one that clears slots in the
+ * workspace and one that reads the weights once, held on the chip between the range and the rounding (with
+ * qb_workspace_bytes() bytes of workspace); beyond, a per-group min/max reduction into the workspace, then
+ * round/clamp/pack.
  */
 qb_status qb_quantize_pack_weights(const float* w, int64_t N, int64_t K, int bits, int groups,
                                    const float* range_lo, const float* range_hi, uint32_t* packed,
@@ -145,7 +149,7 @@ typedef struct {
  * all matrices that take the single-kernel path of qb_quantize_pack_weights go into one launch per 96
  * matrices, whatever their widths (a mixed-precision stack is one launch), separately for groups that
  * fit one thread block, for each cluster size, and for caller-supplied ranges.  The others get a pair
- * of launches per bit width and 32 matrices.  Everything is enqueued on `cuda_stream`; the call
+ * of launches per 96 matrices (and 128 groups).  Everything is enqueued on `cuda_stream`; the call
  * creates no host or device object.
  * Workspace: qb_workspace_bytes(0, 0, 0, 0, G) bytes with G = max(32, sum of `groups` over the batch).
  */
