@@ -104,6 +104,19 @@ __device__ __forceinline__ uint32_t quant_word(const float4& v, float inv) {
   return __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
 }
 
+// The tensor of the batch that holds unit / segment `x`: the last one that begins at or before it.  (Walking a batch of 48
+// from its start cost every block and warp some 50 cycles per tensor.)
+template <int P, int64_t ActItem::*BEGIN>
+__device__ __forceinline__ int find_item(const ActBatch<P>& b, int64_t x) {
+  int lo = 0, hi = b.count - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (b.item[mid].*BEGIN <= x) lo = mid;
+    else hi = mid - 1;
+  }
+  return lo;
+}
+
 template <int P>
 __global__ void __launch_bounds__(kActThreads, kActBlocksPerSm)
 act_absmax_kernel(const __grid_constant__ ActBatch<P> b) {
@@ -117,14 +130,15 @@ act_absmax_kernel(const __grid_constant__ ActBatch<P> b) {
   const int64_t u0 = (int64_t)blockIdx.x * b.units_per_block;
   const int64_t u1 = min(u0 + b.units_per_block, b.units_total);
   bool cleared = warp != 0;
-  for (int it = 0; it < b.count; ++it) {
+  const int first = find_item<P, &ActItem::unit_begin>(b, u0);
+  int it = first;
+  for (; it < b.count && b.item[it].unit_begin < u1; ++it) {
     const ActItem& t = b.item[it];
-    const int64_t units = t.M * t.units_per_row;
-    const int64_t lo = max(u0 - t.unit_begin, (int64_t)0), hi = min(u1 - t.unit_begin, units);
-    if (t.segs_per_row > 1)  // row sums that several warps will add to
-      for (int64_t m = (int64_t)blockIdx.x * kActThreads + threadIdx.x; m < t.M; m += (int64_t)gridDim.x * kActThreads)
-        t.rowsum[m] = 0;
-    if (lo >= hi) continue;
+    const int64_t lo = max(u0 - t.unit_begin, (int64_t)0), hi = min(u1 - t.unit_begin, t.M * t.units_per_row);
+    if (t.segs_per_row > 1) {  // row sums that several warps will add to: of the rows that begin in this share
+      const int64_t m0 = (lo + t.units_per_row - 1) / t.units_per_row, m1 = (hi + t.units_per_row - 1) / t.units_per_row;
+      for (int64_t m = m0 + threadIdx.x; m < m1; m += kActThreads) t.rowsum[m] = 0;
+    }
     const float4* __restrict__ x = reinterpret_cast<const float4*>(t.x) + lane;
     Extremes ex;
     for (int64_t u = lo + warp * kSegUnits; u < hi; u += kActWarps * kSegUnits) {
@@ -147,7 +161,7 @@ act_absmax_kernel(const __grid_constant__ ActBatch<P> b) {
   __syncthreads();
   if (threadIdx.x == 0 && !poll_word<true>(&h->cleared, 1u)) report_status(b.ws, QB_ERR_TIMEOUT);
   __syncthreads();
-  for (int i = threadIdx.x; i < b.count; i += kActThreads)
+  for (int i = first + threadIdx.x; i < it; i += kActThreads)
     if (s_max[i] != 0u) atomicMax(b.absmax_bits + i, s_max[i]);
 }
 
@@ -182,9 +196,10 @@ act_quantize_kernel(const __grid_constant__ ActBatch<P> b) {
   }
   const int64_t warps = (int64_t)gridDim.x * kActWarps;
   const uint64_t pol = policy_evict_first();
-  int it = 0, cur = -1;
+  const int64_t s0 = (int64_t)blockIdx.x * kActWarps + (threadIdx.x >> 5);
+  int it = find_item<P, &ActItem::seg_begin>(b, s0), cur = -1;
   float inv = 0.0f;
-  for (int64_t s = (int64_t)blockIdx.x * kActWarps + (threadIdx.x >> 5); s < b.segs_total; s += warps) {
+  for (int64_t s = s0; s < b.segs_total; s += warps) {
     while (it + 1 < b.count && s >= b.item[it + 1].seg_begin) ++it;
     const ActItem& t = b.item[it];
     const uint32_t local = (uint32_t)(s - t.seg_begin);  // below 2^24 rows x 64 segments
