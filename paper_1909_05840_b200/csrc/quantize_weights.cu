@@ -555,9 +555,6 @@ __device__ __forceinline__ uint32_t cluster_size() {
   asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
   return r;
 }
-__device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v) {
-  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
-}
 
 // CLUSTER = false: the kernel described above.  CLUSTER = true: groups of 289 to 2,304 units; a thread-block
 // cluster of 2 to 8 CTAs (the launch's cluster size) holds one group, every CTA reduces its 16 slices,
@@ -592,6 +589,7 @@ weight_regs_kernel(const __grid_constant__ RegsBatch b) {
   const int id0 = (int)blockIdx.x / csize, stride = (int)gridDim.x / csize;  // items go to clusters
   int it = 0, prev_it = 0;
   float4 v[kRgUnits];
+  if (CLUSTER) ptx::cluster_sync_all();  // every CTA has started: its shared memory may be written to
   pdl_begin();
   RegsSlice s = regs_slice<CLUSTER>(b, id0, it, warp, lane, crank);
 #pragma unroll
@@ -693,8 +691,8 @@ weight_regs_kernel(const __grid_constant__ RegsBatch b) {
         e_hi = __reduce_max_sync(0xffffffffu, lane < kRgWarps ? s_hi[flip][lane] : 0u);
         e_lo = __reduce_max_sync(0xffffffffu, lane < kRgWarps ? s_lo[flip][lane] : 0u);
         if (warp == 0 && lane < csize) {  // this CTA's range into slot `crank` of CTA `lane`
-          st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&x_hi[flip][crank]), (uint32_t)lane), e_hi);
-          st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&x_lo[flip][crank]), (uint32_t)lane), e_lo);
+          ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&x_hi[flip][crank]), (uint32_t)lane), e_hi);
+          ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&x_lo[flip][crank]), (uint32_t)lane), e_lo);
         }
         ptx::cluster_sync_all();
         e_hi = __reduce_max_sync(0xffffffffu, lane < csize ? x_hi[flip][lane] : 0u);
