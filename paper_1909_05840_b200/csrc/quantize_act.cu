@@ -12,8 +12,8 @@
 //                        store, row sum by dp4a and a warp reduction (rows of several segments: atomicAdd on
 //                        row sums that the first kernel cleared).
 //   act_fused_kernel     both for one tensor whose segments each find a warp on the device: the segment
-//                        stays in registers while the blocks agree on a, x is read once and there is one
-//                        launch instead of two.
+//                        stays in registers while the blocks agree on a (up to 256 segments: as one cluster,
+//                        in distributed shared memory), x is read once and there is one launch instead of two.
 //
 // Both passes are memory-bound (4 B read per element, then 4 B read, from L2 as far as it holds the
 // tensors, and 1 B written).  What bounds them below L2's size is the bytes in flight and the instructions per
@@ -25,12 +25,15 @@
 
 #include "common.cuh"
 #include "mbar_wait.cuh"
+#include "ptx.cuh"
 
 namespace qb {
 
 constexpr int kActThreads = 256;
 constexpr int kActWarps = kActThreads / 32;
 constexpr int kActBlocksPerSm = 4;
+constexpr int kActMaxCluster = 8;     // act_fused_kernel: CTAs of a cluster (the portable size)
+constexpr int kActMaxThreads = 1024;  // and threads of such a CTA
 constexpr int kSegUnits = 8;      // float4 per lane and segment
 constexpr int kMaxActBatch = 64;  // tensors per launch (descriptors travel as kernel parameters, 4 KB)
 
@@ -224,28 +227,36 @@ act_quantize_kernel(const __grid_constant__ ActBatch<P> b) {
   }
 }
 
-// One tensor, one segment per warp, every block resident (cooperative launch).
-__global__ void __launch_bounds__(kActThreads, kActBlocksPerSm)
+// One tensor, one segment per warp.  CLUSTER: the blocks, of 8 to 32 warps, are the CTAs of one thread-block cluster
+// and agree on the maximum through distributed shared memory.  Otherwise they agree through the workspace, and every
+// block is resident (cooperative launch).  The agreement bounds both: five round trips to L2 and a cooperative launch,
+// or one barrier of the cluster (M = 32 x 768 with its GEMM: 12.3 -> 9.3 us).
+template <bool CLUSTER>
+__global__ void __launch_bounds__(CLUSTER ? kActMaxThreads : kActThreads, CLUSTER ? 1 : kActBlocksPerSm)
 act_fused_kernel(const __grid_constant__ ActBatch<1> b) {
-  __shared__ uint32_t s_max;
+  __shared__ uint32_t s_max, s_peer[kActMaxCluster];
   __shared__ int s_ok;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   WsHeader* const h = reinterpret_cast<WsHeader*>(b.ws);
   const ActItem& t = b.item[0];
-  const uint32_t local = blockIdx.x * kActWarps + warp;
+  const uint32_t local = blockIdx.x * (blockDim.x >> 5) + warp;
   const bool mine = local < (uint32_t)b.segs_total;
   const uint32_t row = local / (uint32_t)t.segs_per_row;
   const int seg = (int)(local - row * t.segs_per_row);
   const int n = mine ? min(t.seg_units, t.units_per_row - seg * t.seg_units) : 0;
   const float4* src = reinterpret_cast<const float4*>(t.x) + ((int64_t)row * t.units_per_row + seg * t.seg_units) * 32 + lane;
   if (threadIdx.x == 0) s_max = 0u;
+  if constexpr (CLUSTER) ptx::cluster_arrive();  // "this CTA has started": waited for before the first remote store
   pdl_begin();
   float4 v[kSegUnits];
 #pragma unroll
   for (int j = 0; j < kSegUnits; ++j)
     if (j < n) v[j] = __ldg(src + j * 32);
-  const uint32_t round = ld_acquire(&h->round);  // only the block that arrives last changes it
-  if (warp == 0) clear_slots(b.absmax_bits, 1, h, lane);
+  uint32_t round = 0;
+  if constexpr (!CLUSTER) {
+    round = ld_acquire(&h->round);  // only the block that arrives last changes it
+    if (warp == 0) clear_slots(b.absmax_bits, 1, h, lane);
+  }
   if (mine && t.segs_per_row > 1 && seg == 0 && lane == 0) t.rowsum[row] = 0;  // published by the barrier below
   __syncthreads();
   Extremes ex;
@@ -255,31 +266,43 @@ act_fused_kernel(const __grid_constant__ ActBatch<1> b) {
   const uint32_t m = ex.warp_bits();
   if (lane == 0 && m != 0u) atomicMax(&s_max, m);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    // publish this block's maximum, then wait for all blocks: the last one to arrive lets the others go
-    bool ok = poll_word<true>(&h->cleared, 1u);
-    if (ok) {
-      if (s_max != 0u) atomicMax(b.absmax_bits, s_max);
-      __threadfence();
-      if (atomicAdd(&h->arrived, 1u) == gridDim.x - 1u) {
-        h->ticket = 0u;
-        h->cleared = 0u;
-        h->arrived = 0u;
+  uint32_t absmax;
+  if constexpr (CLUSTER) {
+    ptx::cluster_wait();
+    if (threadIdx.x < gridDim.x)  // this CTA's maximum into its slot of CTA threadIdx.x
+      ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&s_peer[blockIdx.x]), threadIdx.x), s_max);
+    __syncwarp();
+    ptx::cluster_sync_all();  // publishes the row sums set to zero, too
+    absmax = 0u;
+    for (int i = 0; i < (int)gridDim.x; ++i) absmax = max(absmax, s_peer[i]);
+  } else {
+    if (threadIdx.x == 0) {
+      // publish this block's maximum, then wait for all blocks: the last one to arrive lets the others go
+      bool ok = poll_word<true>(&h->cleared, 1u);
+      if (ok) {
+        if (s_max != 0u) atomicMax(b.absmax_bits, s_max);
         __threadfence();
-        st_release(&h->round, round + 1u);
-      } else {
-        ok = poll_word<false>(&h->round, round);
+        if (atomicAdd(&h->arrived, 1u) == gridDim.x - 1u) {
+          h->ticket = 0u;
+          h->cleared = 0u;
+          h->arrived = 0u;
+          __threadfence();
+          st_release(&h->round, round + 1u);
+        } else {
+          ok = poll_word<false>(&h->round, round);
+        }
+        __threadfence();
+        s_max = __ldcg(b.absmax_bits);
       }
-      __threadfence();
-      s_max = __ldcg(b.absmax_bits);
+      if (!ok) report_status(b.ws, QB_ERR_TIMEOUT);
+      s_ok = ok ? 1 : 0;
     }
-    if (!ok) report_status(b.ws, QB_ERR_TIMEOUT);
-    s_ok = ok ? 1 : 0;
+    __syncthreads();
+    if (!s_ok) return;
+    absmax = s_max;
   }
-  __syncthreads();
-  if (!s_ok) return;
   float scale, inv;
-  const bool finite = act_scales(s_max, &scale, &inv);
+  const bool finite = act_scales(absmax, &scale, &inv);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *t.act_scale = scale;
     if (!finite) report_status(b.ws, QB_ERR_NONFINITE);
@@ -329,10 +352,20 @@ static qb_status launch_act_batch(const qb_act_desc* d, int count, void* ws, uin
   b.keep_fraction = l2_keep_fraction(512.0 * (double)units);
   const int64_t seg_blocks = (segs + kActWarps - 1) / kActWarps;
   if constexpr (P == 1) {
+    b.units_per_block = 0;
+    // A segment for every warp of one cluster of 8 CTAs (the portable size): up to 256 segments, 32 x 768 has 32.
+    // With the GEMM behind it, one cluster against all blocks resident: M = 1 x 768 9.3 us, 12.7; 128 x 768 9.4, 14.3;
+    // 256 x 768 10.2, 14.3; 77 x 3,072 (231 segments) 15.5, 20.5.  CTAs of at least 1, 4 or 16 warps take as
+    // long as those of 8, to 0.3 us.
+    if (segs <= kActMaxCluster * (kActMaxThreads / 32)) {
+      const unsigned warps = (unsigned)std::max<int64_t>((segs + kActMaxCluster - 1) / kActMaxCluster, kActWarps);
+      const unsigned ctas = (unsigned)((segs + warps - 1) / warps);
+      QB_CUDA_TRY(launch_kernel(act_fused_kernel<true>, ctas, warps * 32, 0, stream, true, ctas, false, b));
+      return QB_OK;
+    }
     // A segment for every resident warp (4,736 of them; 1,024 x 768 needs 1,024): one launch.
     if (seg_blocks <= cap) {
-      b.units_per_block = 0;
-      QB_CUDA_TRY(launch_kernel(act_fused_kernel, (unsigned)seg_blocks, kActThreads, 0, stream, true, 1, true, b));
+      QB_CUDA_TRY(launch_kernel(act_fused_kernel<false>, (unsigned)seg_blocks, kActThreads, 0, stream, true, 1, true, b));
       return QB_OK;
     }
   }

@@ -33,6 +33,22 @@ def test_quantize_act_shapes(ws, M, K):
     assert qb.read_status(ws) == qb.QB_OK
 
 
+# one cluster: 1 to 8 CTAs of 8 to 32 warps, the largest with 256 segments; 257 segments are beyond it
+@pytest.mark.parametrize("M,K", [(8, 256), (9, 256), (17, 1024), (12, 2304), (5, 8192), (63, 768), (65, 768), (127, 640),
+                                 (51, 5120), (256, 1024), (257, 1024)])
+def test_one_cluster(ws, M, K):
+    for seed in (1, 2):
+        x = synth.activations(M, K, seed=M + K + seed)
+        x[M - 1 if seed == 1 else 0, K - 1] = 300.0  # the maximum in the last CTA or in the first
+        xq, sc, rs = gu.gpu_quantize_act(x, ws)
+        _, o_xq, o_s, o_rs = oracle.quantize_act(x)
+        assert sc.item() == o_s
+        assert np.array_equal(xq.cpu().numpy(), o_xq) and np.array_equal(rs.cpu().numpy(), o_rs)
+    x[M // 2, 1] = np.nan
+    gu.gpu_quantize_act(x, ws2 := qb.workspace(groups=64))
+    assert qb.read_status(ws2) == qb.QB_ERR_NONFINITE and qb.read_status(ws) == qb.QB_OK
+
+
 def test_fused_call_between_batches(ws):
     # batches (two passes) and single calls (one launch) share the words that count blocks
     for rep in range(3):
