@@ -13,11 +13,11 @@ namespace qb {
 // ---- workspace layout (device memory owned by the caller) ------------------------------------
 // [0]   int32  status   first device-side error, never cleared by a kernel
 // [4]   int32  detail   where a bounded wait gave up (role << 16 | stage), diagnostics only
-// [16]  uint32 act_absmax_bits   bit pattern of max|x| of the last qb_quantize_act
-// [32]  uint32 ticket            blocks of the running launch that have started        } zero
-// [36]  uint32 cleared           1 once the running launch's reduction slots are clear } between
-// [40]  uint32 arrived           blocks of the running launch that have published      } calls
-// [44]  uint32 round             counts the launches whose blocks waited for one another
+// [16]  uint32 act_absmax_bits   reduction slot of act_absmax_kernel for a single tensor
+// [32]  uint32 ticket            blocks of the running launch that have started        } zero between
+// [36]  uint32 cleared           1 once the running launch's reduction slots are clear } calls
+// [40]  uint32 round             counts the launches whose clusters waited for one another
+// [64]  uint64 cluster_max[24]   round << 32 | bit pattern of a cluster's max|x|, all of the last such launch
 // [256] uint32 range_hi_enc[G], uint32 range_lo_inv[G]   ordered encodings of per-group max / min
 //       or, weight_ring_kernel: uint64 [groups][CTAs], encoded max << 32 | inverted encoded min
 constexpr size_t kWsStatusOff = 0;
@@ -25,6 +25,7 @@ constexpr size_t kWsDetailOff = 4;
 constexpr size_t kWsActMaxOff = 16;
 constexpr size_t kWsRangeOff = 256;
 constexpr size_t kWsMinBytes = 256;
+constexpr int kWsClusters = 24;
 
 struct WsHeader {
   int32_t status;
@@ -34,9 +35,11 @@ struct WsHeader {
   uint32_t pad2[3];
   uint32_t ticket;
   uint32_t cleared;
-  uint32_t arrived;
   uint32_t round;
+  uint32_t pad3[5];
+  unsigned long long cluster_max[kWsClusters];
 };
+static_assert(sizeof(WsHeader) == kWsRangeOff, "the tables follow the header");
 
 // What a call on G groups must get, and what qb_workspace_bytes tells callers to give: with a slot per group and CTA
 // (for up to kRingMaxGroups groups) the weight quantizer reads W once where groups are too large for a
@@ -147,6 +150,14 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
   uint32_t v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
   return v;
+}
+__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_release(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 __device__ __forceinline__ void st_release(uint32_t* p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");

@@ -77,7 +77,7 @@ emb_range_kernel(const float4* __restrict__ e, int64_t V, int d4, int slots, int
     mine[4 * q + i] = float_to_ordered(hi[i]);
     mine[D + 4 * q + i] = ~float_to_ordered(lo[i]);
   }
-  if (threadIdx.x == 0 && !poll_word<true>(&h->cleared, 1u)) report_status(ws, QB_ERR_TIMEOUT);
+  if (threadIdx.x == 0 && !poll_word(&h->cleared, 1u)) report_status(ws, QB_ERR_TIMEOUT);
   __syncthreads();
   // groups of few columns: a thread each; of many: a warp each
   const bool by_warp = cols_per_group >= 16;

@@ -54,12 +54,11 @@ __device__ __forceinline__ bool wait_barrier_warp(uint32_t bar, uint32_t parity,
   return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
-// One thread polls a global word until it equals / differs from v (acquire); false when the bound ran out.
-template <bool EQUAL>
+// One thread polls a global word until it equals v (acquire); false when the bound ran out.
 __device__ __forceinline__ bool poll_word(const uint32_t* p, uint32_t v, long long limit = kWaitLimitCycles) {
-  if ((ld_acquire(p) == v) == EQUAL) return true;
+  if (ld_acquire(p) == v) return true;
   const long long t0 = clock64();
-  while ((ld_acquire(p) == v) != EQUAL)
+  while (ld_acquire(p) != v)
     if (clock64() - t0 > limit) return false;
   return true;
 }

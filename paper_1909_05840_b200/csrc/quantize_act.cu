@@ -11,15 +11,15 @@
 //   act_quantize_kernel  one warp per segment: x * (127/a), round half to even, four codes per 32-bit
 //                        store, row sum by dp4a and a warp reduction (rows of several segments: atomicAdd on
 //                        row sums that the first kernel cleared).
-//   act_fused_kernel     both for one tensor whose segments each find a warp on the device: the segment
-//                        stays in registers while the blocks agree on a (up to 256 segments: as one cluster,
-//                        in distributed shared memory), x is read once and there is one launch instead of two.
+//   act_fused_kernel     both for one tensor of up to 2,368 segments, each of which finds a warp on the device: the
+//                        segment stays in registers while the blocks agree on a, within a cluster in
+//                        distributed shared memory; x is read once and there is one launch instead of two.
 //
 // Both passes are memory-bound (4 B read per element, then 4 B read, from L2 as far as it holds the
 // tensors, and 1 B written).  What bounds them below L2's size is the bytes in flight and the instructions per
 // element: 128 KB of loads per SM and about nine instructions per float4 (packed fp32x2, no clamp) instead of
 // 64 KB and thirty.  Quantizer and GEMMs of one BERT-base layer at M = 4096 (88 MB of input): 86.9 -> 81.1 us;
-// int8 chain at M = 6144 98.0 -> 91.5; query projection at M = 1024 (fused) 20.1 -> 17.4.
+// int8 chain at M = 6144 98.0 -> 91.5; query projection at M = 1024 (fused) 20.1 -> 17.4 -> 12.6.
 #include <algorithm>
 #include <cstring>
 
@@ -162,7 +162,7 @@ act_absmax_kernel(const __grid_constant__ ActBatch<P> b) {
     if (lane == 0 && m != 0u) atomicMax(&s_max[it], m);
   }
   __syncthreads();
-  if (threadIdx.x == 0 && !poll_word<true>(&h->cleared, 1u)) report_status(b.ws, QB_ERR_TIMEOUT);
+  if (threadIdx.x == 0 && !poll_word(&h->cleared, 1u)) report_status(b.ws, QB_ERR_TIMEOUT);
   __syncthreads();
   for (int i = first + threadIdx.x; i < it; i += kActThreads)
     if (s_max[i] != 0u) atomicMax(b.absmax_bits + i, s_max[i]);
@@ -227,12 +227,15 @@ act_quantize_kernel(const __grid_constant__ ActBatch<P> b) {
   }
 }
 
-// One tensor, one segment per warp.  CLUSTER: the blocks, of 8 to 32 warps, are the CTAs of one thread-block cluster
-// and agree on the maximum through distributed shared memory.  Otherwise they agree through the workspace, and every
-// block is resident (cooperative launch).  The agreement bounds both: five round trips to L2 and a cooperative launch,
-// or one barrier of the cluster (M = 32 x 768 with its GEMM: 12.3 -> 9.3 us).
-template <bool CLUSTER>
-__global__ void __launch_bounds__(CLUSTER ? kActMaxThreads : kActThreads, CLUSTER ? 1 : kActBlocksPerSm)
+// One tensor, one segment per warp; the segment stays in registers while the warps agree on the maximum, which is what
+// bounds the kernel.  The blocks of a cluster (of 8 to 32 warps) agree through distributed shared memory: one barrier of
+// the cluster.  MANY: the maxima of several clusters, all resident (cooperative launch), meet in the workspace: each
+// is stored with the launch's number, and every block polls for all of them, one release and one acquire in all;
+// no word has to be cleared first.  All blocks resident that met in one word (clear, maximum, count, go-ahead,
+// read: five trips to L2) took, with the GEMM, 12.7 us at M = 32 x 768 (now, one cluster: 9.3), 14.3 at
+// 1,024 x 768 (now, 16 clusters: 12.4).
+template <bool MANY>
+__global__ void __launch_bounds__(kActMaxThreads, 1)
 act_fused_kernel(const __grid_constant__ ActBatch<1> b) {
   __shared__ uint32_t s_max, s_peer[kActMaxCluster];
   __shared__ int s_ok;
@@ -246,17 +249,15 @@ act_fused_kernel(const __grid_constant__ ActBatch<1> b) {
   const int n = mine ? min(t.seg_units, t.units_per_row - seg * t.seg_units) : 0;
   const float4* src = reinterpret_cast<const float4*>(t.x) + ((int64_t)row * t.units_per_row + seg * t.seg_units) * 32 + lane;
   if (threadIdx.x == 0) s_max = 0u;
-  if constexpr (CLUSTER) ptx::cluster_arrive();  // "this CTA has started": waited for before the first remote store
+  const uint32_t rank = ptx::cluster_ctarank(), ctas = MANY ? kActMaxCluster : gridDim.x;
+  ptx::cluster_arrive();  // "this CTA has started": waited for before the first remote store
   pdl_begin();
   float4 v[kSegUnits];
 #pragma unroll
   for (int j = 0; j < kSegUnits; ++j)
     if (j < n) v[j] = __ldg(src + j * 32);
-  uint32_t round = 0;
-  if constexpr (!CLUSTER) {
-    round = ld_acquire(&h->round);  // only the block that arrives last changes it
-    if (warp == 0) clear_slots(b.absmax_bits, 1, h, lane);
-  }
+  uint32_t tag = 0u;
+  if (MANY && warp == 0) tag = ld_acquire(&h->round) + 1u;  // every CTA reads it before its cluster publishes
   if (mine && t.segs_per_row > 1 && seg == 0 && lane == 0) t.rowsum[row] = 0;  // published by the barrier below
   __syncthreads();
   Extremes ex;
@@ -266,36 +267,40 @@ act_fused_kernel(const __grid_constant__ ActBatch<1> b) {
   const uint32_t m = ex.warp_bits();
   if (lane == 0 && m != 0u) atomicMax(&s_max, m);
   __syncthreads();
-  uint32_t absmax;
-  if constexpr (CLUSTER) {
-    ptx::cluster_wait();
-    if (threadIdx.x < gridDim.x)  // this CTA's maximum into its slot of CTA threadIdx.x
-      ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&s_peer[blockIdx.x]), threadIdx.x), s_max);
-    __syncwarp();
-    ptx::cluster_sync_all();  // publishes the row sums set to zero, too
-    absmax = 0u;
-    for (int i = 0; i < (int)gridDim.x; ++i) absmax = max(absmax, s_peer[i]);
-  } else {
-    if (threadIdx.x == 0) {
-      // publish this block's maximum, then wait for all blocks: the last one to arrive lets the others go
-      bool ok = poll_word<true>(&h->cleared, 1u);
-      if (ok) {
-        if (s_max != 0u) atomicMax(b.absmax_bits, s_max);
-        __threadfence();
-        if (atomicAdd(&h->arrived, 1u) == gridDim.x - 1u) {
-          h->ticket = 0u;
-          h->cleared = 0u;
-          h->arrived = 0u;
-          __threadfence();
-          st_release(&h->round, round + 1u);
-        } else {
-          ok = poll_word<false>(&h->round, round);
+  ptx::cluster_wait();
+  if (threadIdx.x < ctas)  // this CTA's maximum into its slot of CTA threadIdx.x
+    ptx::st_cluster_u32(ptx::map_to_cta(ptx::smem_u32(&s_peer[rank]), threadIdx.x), s_max);
+  __syncwarp();
+  ptx::cluster_sync_all();  // publishes the row sums set to zero, too
+  uint32_t absmax = 0u;
+  for (uint32_t i = 0; i < ctas; ++i) absmax = max(absmax, s_peer[i]);
+  if constexpr (MANY) {
+    if (warp == 0) {
+      const uint32_t cluster = blockIdx.x / kActMaxCluster, clusters = gridDim.x / kActMaxCluster;
+      if (rank == 0 && lane == 0) st_release(&h->cluster_max[cluster], (unsigned long long)tag << 32 | absmax);
+      bool ok = true;
+      uint32_t m = 0u;
+      if (lane < (int)clusters) {
+        unsigned long long w = ld_acquire(&h->cluster_max[lane]);
+        if ((uint32_t)(w >> 32) != tag) {
+          const long long t0 = clock64();
+          do {
+            w = ld_acquire(&h->cluster_max[lane]);
+            ok = clock64() - t0 <= kWaitLimitCycles;
+          } while ((uint32_t)(w >> 32) != tag && ok);
         }
-        __threadfence();
-        s_max = __ldcg(b.absmax_bits);
+        m = (uint32_t)w;
+      } else if (blockIdx.x == 0 && lane < kWsClusters) {  // no slot keeps the number of an older launch
+        h->cluster_max[lane] = (unsigned long long)tag << 32;
       }
-      if (!ok) report_status(b.ws, QB_ERR_TIMEOUT);
-      s_ok = ok ? 1 : 0;
+      ok = __all_sync(0xffffffffu, ok);
+      m = __reduce_max_sync(0xffffffffu, m);
+      if (lane == 0) {
+        s_max = m;
+        s_ok = ok ? 1 : 0;
+        if (!ok) report_status(b.ws, QB_ERR_TIMEOUT);
+        if (blockIdx.x == 0) h->round = tag;
+      }
     }
     __syncthreads();
     if (!s_ok) return;
@@ -353,19 +358,24 @@ static qb_status launch_act_batch(const qb_act_desc* d, int count, void* ws, uin
   const int64_t seg_blocks = (segs + kActWarps - 1) / kActWarps;
   if constexpr (P == 1) {
     b.units_per_block = 0;
-    // A segment for every warp of one cluster of 8 CTAs (the portable size): up to 256 segments, 32 x 768 has 32.
-    // With the GEMM behind it, one cluster against all blocks resident: M = 1 x 768 9.3 us, 12.7; 128 x 768 9.4, 14.3;
-    // 256 x 768 10.2, 14.3; 77 x 3,072 (231 segments) 15.5, 20.5.  CTAs of at least 1, 4 or 16 warps take as
+    // With the GEMM behind it, one cluster of up to 8 CTAs (the portable size; 256 segments) against all blocks
+    // resident and one word: M = 128 x 768 9.4 us, 14.3; 256 x 768 10.2, 14.3.  CTAs of at least 1, 4 or 16 warps take as
     // long as those of 8, to 0.3 us.
     if (segs <= kActMaxCluster * (kActMaxThreads / 32)) {
       const unsigned warps = (unsigned)std::max<int64_t>((segs + kActMaxCluster - 1) / kActMaxCluster, kActWarps);
       const unsigned ctas = (unsigned)((segs + warps - 1) / warps);
-      QB_CUDA_TRY(launch_kernel(act_fused_kernel<true>, ctas, warps * 32, 0, stream, true, ctas, false, b));
+      QB_CUDA_TRY(launch_kernel(act_fused_kernel<false>, ctas, warps * 32, 0, stream, true, ctas, false, b));
       return QB_OK;
     }
-    // A segment for every resident warp (4,736 of them; 1,024 x 768 needs 1,024): one launch.
-    if (seg_blocks <= cap) {
-      QB_CUDA_TRY(launch_kernel(act_fused_kernel<false>, (unsigned)seg_blocks, kActThreads, 0, stream, true, 1, true, b));
+    // Several clusters while they need no more than half of the warps that the device holds, so that clusters of CTAs
+    // of 8 or 16 warps find their place: 1,024 x 768 12.4 us, 14.3 as two launches; 1,500 x 1,024 14.0, 15.0;
+    // 2,368 x 1,024 14.4, 15.2.  A segment per warp for all the warps there are (one CTA a cluster, cooperative) is the
+    // slower one: 4,500 x 768 18.4, 16.4 as two launches; 1,000 x 4,096 26.4, 24.6.
+    if (segs <= (int64_t)sm_count * (kActBlocksPerSm * kActWarps / 2) && segs <= kWsClusters * kActMaxCluster * 2 * kActWarps) {
+      const int64_t warps = segs <= kWsClusters * kActMaxCluster * kActWarps ? kActWarps : 2 * kActWarps;
+      const unsigned clusters = (unsigned)((segs + warps * kActMaxCluster - 1) / (warps * kActMaxCluster));
+      QB_CUDA_TRY(launch_kernel(act_fused_kernel<true>, clusters * kActMaxCluster, (unsigned)warps * 32, 0, stream, true,
+                                kActMaxCluster, true, b));
       return QB_OK;
     }
   }

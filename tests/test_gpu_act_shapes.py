@@ -1,5 +1,5 @@
-"""The activation quantizer's launch shapes against the oracle: one launch with the tensor in registers (up to one
-segment of 1,024 elements per resident warp) and two passes beyond; rows of one and of several segments, rows
+"""The activation quantizer's launch shapes against the oracle: one launch with the tensor in registers (a segment of
+up to 1,024 elements per warp: one cluster, then several) and two passes beyond; rows of one and of several segments, rows
 whose last segment is shorter, and calls that follow one another on the same workspace."""
 import numpy as np
 import pytest
@@ -18,7 +18,7 @@ def ws():
     return qb.workspace(groups=64)
 
 
-# 148 SMs x 4 blocks x 8 warps = 4,736 segments in one launch
+# 148 SMs x 16 warps = 2,368 segments in one launch, 4,736 in one wave of the second pass
 @pytest.mark.parametrize("M,K", [(1, 128), (1, 65536), (7, 1024), (9, 1152), (33, 4224), (4736, 128), (4737, 128),
                                  (2368, 1152), (2369, 1152), (73, 65536), (75, 65536)])
 def test_quantize_act_shapes(ws, M, K):
@@ -35,11 +35,30 @@ def test_quantize_act_shapes(ws, M, K):
 
 # one cluster: 1 to 8 CTAs of 8 to 32 warps, the largest with 256 segments; 257 segments are beyond it
 @pytest.mark.parametrize("M,K", [(8, 256), (9, 256), (17, 1024), (12, 2304), (5, 8192), (63, 768), (65, 768), (127, 640),
-                                 (51, 5120), (256, 1024), (257, 1024)])
+                                 (51, 5120), (256, 1024)])
 def test_one_cluster(ws, M, K):
     for seed in (1, 2):
         x = synth.activations(M, K, seed=M + K + seed)
         x[M - 1 if seed == 1 else 0, K - 1] = 300.0  # the maximum in the last CTA or in the first
+        xq, sc, rs = gu.gpu_quantize_act(x, ws)
+        _, o_xq, o_s, o_rs = oracle.quantize_act(x)
+        assert sc.item() == o_s
+        assert np.array_equal(xq.cpu().numpy(), o_xq) and np.array_equal(rs.cpu().numpy(), o_rs)
+    x[M // 2, 1] = np.nan
+    gu.gpu_quantize_act(x, ws2 := qb.workspace(groups=64))
+    assert qb.read_status(ws2) == qb.QB_ERR_NONFINITE and qb.read_status(ws) == qb.QB_OK
+
+
+# several clusters of 8 CTAs: 8 warps each up to 24 x 64 segments, then 16 warps, up to 2,368; 5 and 24 clusters after
+# one another, so that slots of earlier calls would show
+@pytest.mark.parametrize("M,K", [(257, 1024), (320, 1024), (321, 768), (150, 2304), (1536, 128), (1537, 128), (37, 65536),
+                                 (592, 4096), (2368, 256), (2369, 256), (257, 128)])
+def test_several_clusters(ws, M, K):
+    for seed in (1, 2, 3):
+        x = synth.activations(M, K, seed=M + K + seed)
+        if seed != 2:
+            x *= np.float32(0.01)
+        x[M - 1 if seed == 1 else 0, K - 1] = 3.0 * seed  # the maximum in the last cluster or in the first
         xq, sc, rs = gu.gpu_quantize_act(x, ws)
         _, o_xq, o_s, o_rs = oracle.quantize_act(x)
         assert sc.item() == o_s
