@@ -111,6 +111,10 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned b
 // kernel before this one on the stream has completed and its results are visible, and only then lets the
 // next kernel's blocks be set up.  In this order every kernel that runs has all kernels but its direct
 // predecessor behind it when it is set up.
+// The predecessor still writes when this kernel begins, so nothing that it may have written is read-only for this kernel's
+// lifetime: such data (inputs included, which another call of the library may have made) is read with ordinary loads.
+// A non-coherent one (__ldg, or a const __restrict__ argument that the compiler turns into one) counts as invariant
+// and may be moved above the wait.
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -180,7 +184,7 @@ __device__ __forceinline__ void clear_slots(uint32_t* slots, int count, WsHeader
 // the second pass marks its reads as the first to go.
 __device__ __forceinline__ float4 ldg_policy(const float4* p, uint64_t policy) {
   float4 v;
-  asm volatile("ld.global.nc.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
+  asm volatile("ld.global.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
                : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                : "l"(p), "l"(policy));
   return v;

@@ -38,8 +38,8 @@ constexpr int kEmbRangeRows = 8, kEmbRows = 4;  // in flight per thread, range p
 __device__ __forceinline__ bool finite_f(float x) { return fabsf(x) <= 3.402823466e38f; }
 
 __global__ void __launch_bounds__(1024)
-emb_range_kernel(const float4* __restrict__ e, int64_t V, int d4, int slots, int cols_per_group, int groups, float keep_fraction,
-                 uint32_t* __restrict__ g_hi, uint32_t* __restrict__ g_lo_inv, void* ws) {
+emb_range_kernel(const float4* e, int64_t V, int d4, int slots, int cols_per_group, int groups, float keep_fraction,
+                 uint32_t* g_hi, uint32_t* g_lo_inv, void* ws) {
   extern __shared__ uint32_t emb_smem[];  // [slots][2][4 * d4] encoded maxima / inverted minima
   pdl_begin();
   const uint64_t pol = policy_evict_last(keep_fraction);
@@ -105,7 +105,7 @@ emb_range_kernel(const float4* __restrict__ e, int64_t V, int d4, int slots, int
 }
 
 // Range of group g -> q0, 1/Delta, Delta; `report`: the one thread that says that the table is not finite.
-__device__ __forceinline__ void embed_group(int g, int levels, const uint32_t* __restrict__ g_hi, const uint32_t* __restrict__ g_lo_inv,
+__device__ __forceinline__ void embed_group(int g, int levels, const uint32_t* g_hi, const uint32_t* g_lo_inv,
                                             float* lo, float* inv, float* d, bool report, void* ws) {
   float l = ordered_to_float(~g_lo_inv[g]), h = ordered_to_float(g_hi[g]);
   if (!(finite_f(l) && finite_f(h))) {
@@ -153,9 +153,8 @@ __device__ __forceinline__ uint32_t quant_columns(const float4& v, const float (
 
 template <int BITS>
 __global__ void __launch_bounds__(1024)
-emb_pack_kernel(const float4* __restrict__ e, int64_t V, int d4, int slots, int cols_per_group,
-                const uint32_t* __restrict__ g_hi, const uint32_t* __restrict__ g_lo_inv, uint32_t* __restrict__ packed,
-                float* __restrict__ delta, float* __restrict__ q0, void* ws) {
+emb_pack_kernel(const float4* e, int64_t V, int d4, int slots, int cols_per_group,
+                const uint32_t* g_hi, const uint32_t* g_lo_inv, uint32_t* packed, float* delta, float* q0, void* ws) {
   constexpr int L = (1 << BITS) - 1;
   pdl_begin();
   if (blockIdx.x == 0 && threadIdx.x == 0) {  // for the next call; nothing of this launch reads them
@@ -210,8 +209,8 @@ emb_pack_kernel(const float4* __restrict__ e, int64_t V, int d4, int slots, int 
 
 template <int BITS, bool ADD>
 __global__ void __launch_bounds__(1024)
-emb_lookup_kernel(const int32_t* __restrict__ ids, int64_t T, const uint32_t* __restrict__ packed, int64_t V, int d4, int slots,
-                  int cols_per_group, const float* __restrict__ delta, const float* __restrict__ q0, float4* __restrict__ out,
+emb_lookup_kernel(const int32_t* ids, int64_t T, const uint32_t* packed, int64_t V, int d4, int slots,
+                  int cols_per_group, const float* delta, const float* q0, float4* out,
                   void* ws) {
   constexpr uint32_t cm = (1u << BITS) - 1u;
   pdl_begin();
@@ -224,20 +223,20 @@ emb_lookup_kernel(const int32_t* __restrict__ ids, int64_t T, const uint32_t* __
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int g = (4 * q + k) / cols_per_group;
-    d[k] = __ldg(delta + g);
-    z[k] = __ldg(q0 + g);
+    d[k] = delta[g];
+    z[k] = q0[g];
   }
   for (int64_t i = (int64_t)blockIdx.x * slots + slot; i < T; i += step) {
     const int64_t t = ADD ? T - 1 - i : i;
-    const int id = __ldg(ids + t);
+    const int id = ids[t];
     float4* const o = out + t * d4 + q;
     float4 a;
     if (ADD) a = *o;
     float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
     if (id >= 0 && id < V) {
       const uint32_t* row = packed + (int64_t)id * words_per_row + wi;
-      uint32_t f = __ldg(row);
-      if (BITS == 3 && sh + 12 > 32) f = __funnelshift_r(f, __ldg(row + 1), sh);
+      uint32_t f = row[0];
+      if (BITS == 3 && sh + 12 > 32) f = __funnelshift_r(f, row[1], sh);
       else f >>= sh;
       r.x = __fmaf_rn(d[0], (float)(f & cm), z[0]);
       r.y = __fmaf_rn(d[1], (float)((f >> BITS) & cm), z[1]);

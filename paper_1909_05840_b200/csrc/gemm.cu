@@ -212,20 +212,20 @@ __device__ __forceinline__ void expand_item(const uint32_t* in, uint32_t (&out)[
 
 // Load one item (32 codes = BITS words, 4*BITS bytes) with the widest aligned access.
 template <int BITS>
-__device__ __forceinline__ void load_item(const uint32_t* __restrict__ src, uint32_t* dst) {
+__device__ __forceinline__ void load_item(const uint32_t* src, uint32_t* dst) {
   if constexpr (BITS == 8) {
-    const uint4 a = __ldg(reinterpret_cast<const uint4*>(src));
-    const uint4 b = __ldg(reinterpret_cast<const uint4*>(src) + 1);
+    const uint4 a = reinterpret_cast<const uint4*>(src)[0];
+    const uint4 b = reinterpret_cast<const uint4*>(src)[1];
     dst[0] = a.x; dst[1] = a.y; dst[2] = a.z; dst[3] = a.w;
     dst[4] = b.x; dst[5] = b.y; dst[6] = b.z; dst[7] = b.w;
   } else if constexpr (BITS == 4) {
-    const uint4 a = __ldg(reinterpret_cast<const uint4*>(src));
+    const uint4 a = reinterpret_cast<const uint4*>(src)[0];
     dst[0] = a.x; dst[1] = a.y; dst[2] = a.z; dst[3] = a.w;
   } else if constexpr (BITS == 2) {
-    const uint2 a = __ldg(reinterpret_cast<const uint2*>(src));
+    const uint2 a = reinterpret_cast<const uint2*>(src)[0];
     dst[0] = a.x; dst[1] = a.y;
   } else {
-    dst[0] = __ldg(src); dst[1] = __ldg(src + 1); dst[2] = __ldg(src + 2);
+    dst[0] = src[0]; dst[1] = src[1]; dst[2] = src[2];
   }
 }
 
@@ -720,13 +720,13 @@ qb_gemm_kernel(const __grid_constant__ GP gp) {
       const int n = tv.n_base + r;
       tv.s_a = tv.dlt = tv.z = tv.b = 0.f;  // neurons past N: alpha = beta = b = 0, never stored
       if (n < pr.N) {
-        tv.s_a = __ldg(pr.act_scale);
+        tv.s_a = *pr.act_scale;
         const int g = n / pr.rows_per_group;
-        tv.dlt = __ldg(pr.delta + g);
-        tv.z = __ldg(pr.q0 + g);
-        tv.b = pr.bias ? __ldg(pr.bias + n) : 0.0f;
+        tv.dlt = pr.delta[g];
+        tv.z = pr.q0[g];
+        tv.b = pr.bias ? pr.bias[n] : 0.0f;
       }
-      tv.rs_i = (e < BT && tv.m0 + e < pr.M) ? __ldg(pr.rowsum + tv.m0 + e) : 0;
+      tv.rs_i = (e < BT && tv.m0 + e < pr.M) ? pr.rowsum[tv.m0 + e] : 0;
     };
 
     TileCursor c;
@@ -755,7 +755,7 @@ qb_gemm_kernel(const __grid_constant__ GP gp) {
       uint16_t* const y16_ptr = reinterpret_cast<uint16_t*>(pr.y);
       int8_t* const y8_ptr = reinterpret_cast<int8_t*>(pr.y);
       float out_inv = 0.0f;
-      if constexpr (OUT == kOutI8) out_inv = __fdiv_rn(1.0f, __ldg(pr.out_scale));
+      if constexpr (OUT == kOutI8) out_inv = __fdiv_rn(1.0f, *pr.out_scale);
       int32_t* const acc_ptr = pr.acc_out;
 
       // one warp polls the accumulator's barrier; the others are parked at the named barrier below (a
@@ -1346,15 +1346,15 @@ extern "C" qb_status qb_gemm_i8(const int8_t* xq, const float* act_scale, const 
 
 namespace qb {
 // one warp per row, 16 codes per lane and load
-__global__ void __launch_bounds__(256) rowsum_i8_kernel(const int4* __restrict__ xq, int64_t M, int64_t k16,
-                                                        int32_t* __restrict__ rowsum) {
+__global__ void __launch_bounds__(256) rowsum_i8_kernel(const int4* xq, int64_t M, int64_t k16,
+                                                        int32_t* rowsum) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * 8;
   pdl_begin();
   for (int64_t m = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5); m < M; m += warps) {
     int s = 0;
     for (int64_t c = lane; c < k16; c += 32) {
-      const int4 v = __ldg(xq + m * k16 + c);
+      const int4 v = xq[m * k16 + c];
       s = __dp4a(v.x, 0x01010101, s);
       s = __dp4a(v.y, 0x01010101, s);
       s = __dp4a(v.z, 0x01010101, s);

@@ -142,7 +142,7 @@ act_absmax_kernel(const __grid_constant__ ActBatch<P> b) {
       const int64_t m0 = (lo + t.units_per_row - 1) / t.units_per_row, m1 = (hi + t.units_per_row - 1) / t.units_per_row;
       for (int64_t m = m0 + threadIdx.x; m < m1; m += kActThreads) t.rowsum[m] = 0;
     }
-    const float4* __restrict__ x = reinterpret_cast<const float4*>(t.x) + lane;
+    const float4* x = reinterpret_cast<const float4*>(t.x) + lane;
     Extremes ex;
     for (int64_t u = lo + warp * kSegUnits; u < hi; u += kActWarps * kSegUnits) {
       const int n = (int)min(hi - u, (int64_t)kSegUnits);
@@ -255,7 +255,7 @@ act_fused_kernel(const __grid_constant__ ActBatch<1> b) {
   float4 v[kSegUnits];
 #pragma unroll
   for (int j = 0; j < kSegUnits; ++j)
-    if (j < n) v[j] = __ldg(src + j * 32);
+    if (j < n) v[j] = src[j * 32];
   uint32_t tag = 0u;
   if (MANY && warp == 0) tag = ld_acquire(&h->round) + 1u;  // every CTA reads it before its cluster publishes
   if (mine && t.segs_per_row > 1 && seg == 0 && lane == 0) t.rowsum[row] = 0;  // published by the barrier below

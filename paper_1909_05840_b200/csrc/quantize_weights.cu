@@ -234,8 +234,8 @@ __device__ __forceinline__ float group_step(const GroupParams& gp, int bits_leve
 // (113 MB of weights fake-quantized in one call, then one backward call per matrix): 144.2 -> 119.3 us.
 constexpr int kSteUnits = 4;
 __global__ void __launch_bounds__(256)
-ste_backward_kernel(const float4* grad_q, const float4* __restrict__ w, int64_t units, uint32_t units_per_group,
-                    const float* __restrict__ lo, const float* __restrict__ hi, float4* grad_w) {
+ste_backward_kernel(const float4* grad_q, const float4* w, int64_t units, uint32_t units_per_group,
+                    const float* lo, const float* hi, float4* grad_w) {
   pdl_begin();
   const int lane = threadIdx.x & 31;
   const int64_t step = (int64_t)gridDim.x * 8 * kSteUnits;
@@ -245,19 +245,19 @@ ste_backward_kernel(const float4* grad_q, const float4* __restrict__ w, int64_t 
 #pragma unroll
     for (int j = 0; j < kSteUnits; ++j)
       if (j < n) {
-        x[j] = __ldg(w + (u + j) * 32 + lane);
+        x[j] = w[(u + j) * 32 + lane];
         g[j] = grad_q[(u + j) * 32 + lane];  // grad_w may be the same buffer
       }
     uint32_t group = (uint32_t)u / units_per_group, in_group = (uint32_t)u - group * units_per_group;
-    float l = __ldg(lo + group), h = __ldg(hi + group);
+    float l = lo[group], h = hi[group];
 #pragma unroll
     for (int j = 0; j < kSteUnits; ++j)
       if (j < n) {
         if (in_group == units_per_group) {
           in_group = 0;
           ++group;
-          l = __ldg(lo + group);
-          h = __ldg(hi + group);
+          l = lo[group];
+          h = hi[group];
         }
         ++in_group;
         float4 r = g[j];
@@ -392,7 +392,7 @@ template <int BITS, int BLK, bool MULTI, bool CLAMP>
 __device__ __forceinline__ void regs_pack_block(float4 (&v)[kRgUnits], const int n, RgGroup& cur, const RgGroup& mine,
                                                 int& gi, int& next_start, const int ug, uint8_t* stg,
                                                 uint32_t* __restrict__ out, const int lane,
-                                                const float4* __restrict__ next_src, const int next_n) {
+                                                const float4* next_src, const int next_n) {
 #pragma unroll
   for (int jj = 0; jj < kRgBlock; ++jj) {
     const int j = BLK * kRgBlock + jj;
@@ -411,7 +411,7 @@ __device__ __forceinline__ void regs_pack_block(float4 (&v)[kRgUnits], const int
 #pragma unroll
   for (int jj = 0; jj < kRgBlock; ++jj) {
     const int j = BLK * kRgBlock + jj;
-    if (j < next_n) v[j] = __ldg(next_src + j * 32);
+    if (j < next_n) v[j] = next_src[j * 32];
   }
   __syncwarp();
   const int nu = min(kRgBlock, n - BLK * kRgBlock);
@@ -462,7 +462,7 @@ __device__ __forceinline__ float4 fake_quant4(float4 v, const RgGroup& g) {
 template <int BLK, bool MULTI, bool CLAMP>
 __device__ __forceinline__ void regs_fake_block(float4 (&v)[kRgUnits], const int n, RgGroup& cur, const RgGroup& mine,
                                                 int& gi, int& next_start, const int ug, float4* __restrict__ out,
-                                                const float4* __restrict__ next_src, const int next_n) {
+                                                const float4* next_src, const int next_n) {
 #pragma unroll
   for (int jj = 0; jj < kRgBlock; ++jj) {
     const int j = BLK * kRgBlock + jj;
@@ -472,7 +472,7 @@ __device__ __forceinline__ void regs_fake_block(float4 (&v)[kRgUnits], const int
       }
       out[j * 32] = fake_quant4<CLAMP>(v[j], cur);
     }
-    if (j < next_n) v[j] = __ldg(next_src + j * 32);
+    if (j < next_n) v[j] = next_src[j * 32];
   }
 }
 
@@ -480,12 +480,12 @@ template <int BLK, bool MULTI, bool FAKE, bool CLAMP>
 __device__ __forceinline__ void regs_pack_block_any(const int bits, float4 (&v)[kRgUnits], const int n, RgGroup& cur,
                                                     const RgGroup& mine, int& gi, int& next_start, const int ug,
                                                     uint8_t* stg, uint32_t* __restrict__ out, const int lane,
-                                                    const float4* __restrict__ next_src, const int next_n) {
+                                                    const float4* next_src, const int next_n) {
   if (BLK * kRgBlock >= n) {  // nothing of this slice here: only the next slice's loads
 #pragma unroll
     for (int jj = 0; jj < kRgBlock; ++jj) {
       const int j = BLK * kRgBlock + jj;
-      if (j < next_n) v[j] = __ldg(next_src + j * 32);
+      if (j < next_n) v[j] = next_src[j * 32];
     }
     return;
   }
@@ -564,11 +564,11 @@ __device__ __forceinline__ uint32_t cluster_size() {
 // Supplied range of group g: the caller's floats, or the encodings the range pass of the two-pass path left.
 __device__ __forceinline__ GroupParams supplied_group(const RegsItem& m, int g, int L, bool publish, void* ws) {
   if (m.encoded) {
-    const float lo = ordered_to_float(~__ldg(reinterpret_cast<const uint32_t*>(m.range_lo) + g));
-    const float hi = ordered_to_float(__ldg(reinterpret_cast<const uint32_t*>(m.range_hi) + g));
+    const float lo = ordered_to_float(~reinterpret_cast<const uint32_t*>(m.range_lo)[g]);
+    const float hi = ordered_to_float(reinterpret_cast<const uint32_t*>(m.range_hi)[g]);
     return finish_group(lo, hi, false, L, g, m.delta, m.q0, publish, ws);
   }
-  return finish_group(__ldg(m.range_lo + g), __ldg(m.range_hi + g), true, L, g, m.delta, m.q0, publish, ws);
+  return finish_group(m.range_lo[g], m.range_hi[g], true, L, g, m.delta, m.q0, publish, ws);
 }
 
 // FAKE: the fp32 fake-quantized matrix is written instead of packed words (`packed` of the item points to it).
@@ -594,7 +594,7 @@ weight_regs_kernel(const __grid_constant__ RegsBatch b) {
   RegsSlice s = regs_slice<CLUSTER>(b, id0, it, warp, lane, crank);
 #pragma unroll
   for (int j = 0; j < kRgUnits; ++j)
-    if (j < s.n) v[j] = __ldg(s.src + j * 32);
+    if (j < s.n) v[j] = s.src[j * 32];
   for (int id = id0, round = 0; id < b.total_items; id += stride, ++round) {
     const RegsItem& m = b.item[s.it];
     // The exchange buffers below are double-buffered per run of items with the same teams; when the
@@ -731,7 +731,7 @@ weight_regs_kernel(const __grid_constant__ RegsBatch b) {
       // nothing of this item here (a last item with fewer groups than teams): only the next slice's loads
 #pragma unroll
       for (int j = 0; j < kRgUnits; ++j)
-        if (j < nx.n) v[j] = __ldg(nx.src + j * 32);
+        if (j < nx.n) v[j] = nx.src[j * 32];
     }
     s = nx;
   }
