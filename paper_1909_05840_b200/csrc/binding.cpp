@@ -4,7 +4,9 @@
 // torch.empty and torch.cuda.current_stream the same two calls took the host more than thirty (an output
 // allocated from Python 2.5 us each, the stream 3.2 us, seventeen converted arguments 1.5 us).  Here the
 // tensors are read, the outputs allocated and the stream looked up in C++, so that a call costs the host
-// little more than its launches.  Marshalling only: no arithmetic, no state, no fallback.
+// little more than its launches.  Marshalling only: no arithmetic, no state, no fallback.  The interpreter's lock is
+// released while outputs are allocated and the library runs: both can block (a full launch queue, an allocation that has to
+// free first), and other threads go on meanwhile.
 //
 // Every function takes its arguments by position (the wrappers in __init__.py give them names and
 // defaults) and raises what the wrapper's own checks would: AssertionError for a tensor of the wrong kind,
@@ -59,25 +61,52 @@ int64_t integer(PyObject* o) {
 }
 void* stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
-// An output: the caller's tensor, or a new one of this shape.  `get` hands over a new reference.
+// Other Python threads run while one of these lives; no Python object may be touched.
+struct Unlocked {
+  PyThreadState* const state = PyEval_SaveThread();
+  Unlocked() = default;
+  Unlocked(const Unlocked&) = delete;
+  ~Unlocked() { PyEval_RestoreThread(state); }
+};
+
+// An output: the caller's tensor, or a new one that `make` allocates (a caller's tensor stays).  `get` hands over a new
+// reference.
 struct Out {
-  PyObject* obj;
-  void* data;
-  Out(PyObject* given, at::IntArrayRef shape, at::ScalarType type, const at::Tensor& like) {
-    if (given != Py_None) {
-      data = tensor(given).data_ptr();
-      obj = Py_NewRef(given);
-    } else {
-      at::Tensor t(at::detail::empty_cuda(shape, type, like.device(), std::nullopt));
-      data = t.data_ptr();
-      obj = THPVariable_Wrap(std::move(t));
-      if (!obj) throw Failed{};
-    }
+  PyObject* obj = nullptr;
+  void* data = nullptr;
+  at::Tensor made;
+  explicit Out(PyObject* given) {
+    if (given == Py_None) return;
+    data = tensor(given).data_ptr();
+    obj = Py_NewRef(given);
   }
   Out(const Out&) = delete;
   ~Out() { Py_XDECREF(obj); }
-  PyObject* get() { return std::exchange(obj, nullptr); }
+  void make(at::IntArrayRef shape, at::ScalarType type, at::Device device) {
+    if (obj) return;
+    made = at::Tensor(at::detail::empty_cuda(shape, type, device, std::nullopt));
+    data = made.data_ptr();
+  }
+  void wrap() {
+    if (!obj) obj = THPVariable_Wrap(std::move(made));
+    if (!obj) throw Failed{};
+  }
+  PyObject* get() {
+    wrap();
+    return std::exchange(obj, nullptr);
+  }
 };
+PyObject* triple(Out& a, Out& b, Out& c) {
+  a.wrap();
+  b.wrap();
+  c.wrap();
+  PyObject* r = PyTuple_New(3);
+  if (!r) throw Failed{};
+  PyTuple_SET_ITEM(r, 0, a.get());
+  PyTuple_SET_ITEM(r, 1, b.get());
+  PyTuple_SET_ITEM(r, 2, c.get());
+  return r;
+}
 
 struct Workspace {
   void* data;
@@ -111,17 +140,21 @@ PyObject* quantize_act(Args a) {
   const at::Tensor& x = input(a[0], at::kFloat, "x: a contiguous fp32 CUDA tensor of two dimensions");
   need(x.dim() == 2, "x: a contiguous fp32 CUDA tensor of two dimensions");
   const int64_t M = x.size(0), K = x.size(1);
+  const at::Device device = x.device();
+  const float* const x_data = x.const_data_ptr<float>();
   const Workspace ws(a[1]);
-  Out xq(a[2], {M, K}, at::kChar, x), scale(a[3], {1}, at::kFloat, x), rowsum(a[4], {M}, at::kInt, x);
-  check(qb_quantize_act(x.const_data_ptr<float>(), M, K, static_cast<int8_t*>(xq.data), static_cast<float*>(scale.data),
-                        static_cast<int32_t*>(rowsum.data), ws.data, ws.bytes, stream()),
-        "qb_quantize_act");
-  PyObject* r = PyTuple_New(3);
-  if (!r) throw Failed{};
-  PyTuple_SET_ITEM(r, 0, xq.get());
-  PyTuple_SET_ITEM(r, 1, scale.get());
-  PyTuple_SET_ITEM(r, 2, rowsum.get());
-  return r;
+  Out xq(a[2]), scale(a[3]), rowsum(a[4]);
+  qb_status st;
+  {
+    const Unlocked unlocked;
+    xq.make({M, K}, at::kChar, device);
+    scale.make({1}, at::kFloat, device);
+    rowsum.make({M}, at::kInt, device);
+    st = qb_quantize_act(x_data, M, K, static_cast<int8_t*>(xq.data), static_cast<float*>(scale.data),
+                         static_cast<int32_t*>(rowsum.data), ws.data, ws.bytes, stream());
+  }
+  check(st, "qb_quantize_act");
+  return triple(xq, scale, rowsum);
 }
 
 // gemm(kind, xq, act_scale, rowsum, packed, delta, q0, bias, N, bits, groups, ws, y, acc_out | out_scale)
@@ -131,12 +164,13 @@ PyObject* gemm(Args a) {
   const at::Tensor& xq = input(a[1], at::kChar, "xq: a contiguous int8 CUDA tensor");
   need(xq.dim() == 2, "xq: two dimensions");
   const int64_t M = xq.size(0), K = xq.size(1), N = integer(a[8]);
+  const at::Device device = xq.device();
   const int bits = (int)integer(a[9]), groups = (int)integer(a[10]);
   const Workspace ws(a[11]);
-  const at::ScalarType type = kind == 0 ? at::kFloat : (kind == 1 ? at::kBFloat16 : at::kChar);
   if (kind == 1 && a[12] != Py_None)
     need(tensor(a[12]).scalar_type() == at::kBFloat16 && tensor(a[12]).is_contiguous(), "y: a contiguous bfloat16 tensor");
-  Out y(a[12], {M, N}, type, xq);
+  if (kind == 2) need(tensor(a[13]).is_cuda() && tensor(a[13]).scalar_type() == at::kFloat, "out_scale: an fp32 CUDA tensor");
+  Out y(a[12]);
   const int8_t* x = xq.const_data_ptr<int8_t>();
   const float* scale = static_cast<const float*>(ptr(a[2]));
   const int32_t* rowsum = static_cast<const int32_t*>(ptr(a[3]));
@@ -144,21 +178,22 @@ PyObject* gemm(Args a) {
   const float* delta = static_cast<const float*>(ptr(a[5]));
   const float* q0 = static_cast<const float*>(ptr(a[6]));
   const float* bias = static_cast<const float*>(ptr(a[7]));
-  if (kind == 0) {
-    check(qb_gemm(x, scale, rowsum, packed, delta, q0, bias, M, N, K, bits, groups, static_cast<float*>(y.data),
-                  static_cast<int32_t*>(ptr(a[13])), ws.data, ws.bytes, stream()),
-          "qb_gemm");
-  } else if (kind == 1) {
-    check(qb_gemm_bf16(x, scale, rowsum, packed, delta, q0, bias, M, N, K, bits, groups, static_cast<uint16_t*>(y.data),
-                       ws.data, ws.bytes, stream()),
-          "qb_gemm_bf16");
-  } else {
-    const at::Tensor& s = tensor(a[13]);
-    need(s.is_cuda() && s.scalar_type() == at::kFloat, "out_scale: an fp32 CUDA tensor");
-    check(qb_gemm_i8(x, scale, rowsum, packed, delta, q0, bias, M, N, K, bits, groups, s.const_data_ptr<float>(),
-                     static_cast<int8_t*>(y.data), ws.data, ws.bytes, stream()),
-          "qb_gemm_i8");
+  void* const last = ptr(a[13]);
+  qb_status st;
+  {
+    const Unlocked unlocked;
+    y.make({M, N}, kind == 0 ? at::kFloat : (kind == 1 ? at::kBFloat16 : at::kChar), device);
+    if (kind == 0)
+      st = qb_gemm(x, scale, rowsum, packed, delta, q0, bias, M, N, K, bits, groups, static_cast<float*>(y.data),
+                   static_cast<int32_t*>(last), ws.data, ws.bytes, stream());
+    else if (kind == 1)
+      st = qb_gemm_bf16(x, scale, rowsum, packed, delta, q0, bias, M, N, K, bits, groups, static_cast<uint16_t*>(y.data),
+                        ws.data, ws.bytes, stream());
+    else
+      st = qb_gemm_i8(x, scale, rowsum, packed, delta, q0, bias, M, N, K, bits, groups, static_cast<const float*>(last),
+                      static_cast<int8_t*>(y.data), ws.data, ws.bytes, stream());
   }
+  check(st, kind == 0 ? "qb_gemm" : (kind == 1 ? "qb_gemm_bf16" : "qb_gemm_i8"));
   return y.get();
 }
 
@@ -166,9 +201,17 @@ PyObject* gemm(Args a) {
 PyObject* rowsum_i8(Args a) {
   const at::Tensor& xq = input(a[0], at::kChar, "xq: a contiguous int8 CUDA tensor of two dimensions");
   need(xq.dim() == 2, "xq: a contiguous int8 CUDA tensor of two dimensions");
-  Out rowsum(a[1], {xq.size(0)}, at::kInt, xq);
-  check(qb_rowsum_i8(xq.const_data_ptr<int8_t>(), xq.size(0), xq.size(1), static_cast<int32_t*>(rowsum.data), stream()),
-        "qb_rowsum_i8");
+  const int64_t M = xq.size(0), K = xq.size(1);
+  const at::Device device = xq.device();
+  const int8_t* const x = xq.const_data_ptr<int8_t>();
+  Out rowsum(a[1]);
+  qb_status st;
+  {
+    const Unlocked unlocked;
+    rowsum.make({M}, at::kInt, device);
+    st = qb_rowsum_i8(x, M, K, static_cast<int32_t*>(rowsum.data), stream());
+  }
+  check(st, "qb_rowsum_i8");
   return rowsum.get();
 }
 
@@ -177,20 +220,23 @@ PyObject* quantize_pack_weights(Args a) {
   const at::Tensor& w = input(a[0], at::kFloat, "w: a contiguous fp32 CUDA tensor of two dimensions");
   need(w.dim() == 2, "w: a contiguous fp32 CUDA tensor of two dimensions");
   const int64_t N = w.size(0), K = w.size(1), bits = integer(a[1]), groups = integer(a[2]);
+  const at::Device device = w.device();
+  const float* const w_data = w.const_data_ptr<float>();
   const Workspace ws(a[3]);
-  Out packed(a[6], {N, std::max<int64_t>(1, K * bits / 32)}, at::kInt, w);
-  Out delta(a[7], {std::max<int64_t>(groups, 1)}, at::kFloat, w), q0(a[8], {std::max<int64_t>(groups, 1)}, at::kFloat, w);
-  check(qb_quantize_pack_weights(w.const_data_ptr<float>(), N, K, (int)bits, (int)groups,
-                                 static_cast<const float*>(ptr(a[4])), static_cast<const float*>(ptr(a[5])),
-                                 static_cast<uint32_t*>(packed.data), static_cast<float*>(delta.data),
-                                 static_cast<float*>(q0.data), ws.data, ws.bytes, stream()),
-        "qb_quantize_pack_weights");
-  PyObject* r = PyTuple_New(3);
-  if (!r) throw Failed{};
-  PyTuple_SET_ITEM(r, 0, packed.get());
-  PyTuple_SET_ITEM(r, 1, delta.get());
-  PyTuple_SET_ITEM(r, 2, q0.get());
-  return r;
+  const float* const lo = static_cast<const float*>(ptr(a[4]));
+  const float* const hi = static_cast<const float*>(ptr(a[5]));
+  Out packed(a[6]), delta(a[7]), q0(a[8]);
+  qb_status st;
+  {
+    const Unlocked unlocked;
+    packed.make({N, std::max<int64_t>(1, K * bits / 32)}, at::kInt, device);
+    delta.make({std::max<int64_t>(groups, 1)}, at::kFloat, device);
+    q0.make({std::max<int64_t>(groups, 1)}, at::kFloat, device);
+    st = qb_quantize_pack_weights(w_data, N, K, (int)bits, (int)groups, lo, hi, static_cast<uint32_t*>(packed.data),
+                                  static_cast<float*>(delta.data), static_cast<float*>(q0.data), ws.data, ws.bytes, stream());
+  }
+  check(st, "qb_quantize_pack_weights");
+  return triple(packed, delta, q0);
 }
 
 // fake_quantize_weights(w, bits, groups, ws, range_lo, range_hi, wq) -> (wq, delta, q0)
@@ -198,20 +244,23 @@ PyObject* fake_quantize_weights(Args a) {
   const at::Tensor& w = input(a[0], at::kFloat, "w: a contiguous fp32 CUDA tensor of two dimensions");
   need(w.dim() == 2, "w: a contiguous fp32 CUDA tensor of two dimensions");
   const int64_t N = w.size(0), K = w.size(1), bits = integer(a[1]), groups = integer(a[2]);
+  const at::Device device = w.device();
+  const float* const w_data = w.const_data_ptr<float>();
   const Workspace ws(a[3]);
-  Out wq(a[6], {N, K}, at::kFloat, w);
-  Out delta(Py_None, {std::max<int64_t>(groups, 0)}, at::kFloat, w), q0(Py_None, {std::max<int64_t>(groups, 0)}, at::kFloat, w);
-  check(qb_fake_quantize_weights(w.const_data_ptr<float>(), N, K, (int)bits, (int)groups,
-                                 static_cast<const float*>(ptr(a[4])), static_cast<const float*>(ptr(a[5])),
-                                 static_cast<float*>(wq.data), static_cast<float*>(delta.data),
-                                 static_cast<float*>(q0.data), ws.data, ws.bytes, stream()),
-        "qb_fake_quantize_weights");
-  PyObject* r = PyTuple_New(3);
-  if (!r) throw Failed{};
-  PyTuple_SET_ITEM(r, 0, wq.get());
-  PyTuple_SET_ITEM(r, 1, delta.get());
-  PyTuple_SET_ITEM(r, 2, q0.get());
-  return r;
+  const float* const lo = static_cast<const float*>(ptr(a[4]));
+  const float* const hi = static_cast<const float*>(ptr(a[5]));
+  Out wq(a[6]), delta(Py_None), q0(Py_None);
+  qb_status st;
+  {
+    const Unlocked unlocked;
+    wq.make({N, K}, at::kFloat, device);
+    delta.make({std::max<int64_t>(groups, 0)}, at::kFloat, device);
+    q0.make({std::max<int64_t>(groups, 0)}, at::kFloat, device);
+    st = qb_fake_quantize_weights(w_data, N, K, (int)bits, (int)groups, lo, hi, static_cast<float*>(wq.data),
+                                  static_cast<float*>(delta.data), static_cast<float*>(q0.data), ws.data, ws.bytes, stream());
+  }
+  check(st, "qb_fake_quantize_weights");
+  return triple(wq, delta, q0);
 }
 
 // ste_backward(grad_wq, w, groups, range_lo, range_hi, grad_w) -> grad_w
@@ -219,11 +268,20 @@ PyObject* ste_backward(Args a) {
   const at::Tensor& g = input(a[0], at::kFloat, "grad_wq: a contiguous fp32 CUDA tensor of the shape of w");
   const at::Tensor& w = tensor(a[1]);
   need(g.dim() == 2 && g.sizes() == w.sizes(), "grad_wq: a contiguous fp32 CUDA tensor of the shape of w");
-  Out grad_w(a[5], w.sizes(), at::kFloat, w);
-  check(qb_ste_backward(g.const_data_ptr<float>(), static_cast<const float*>(w.const_data_ptr()), w.size(0), w.size(1),
-                        (int)integer(a[2]), static_cast<const float*>(ptr(a[3])), static_cast<const float*>(ptr(a[4])),
-                        static_cast<float*>(grad_w.data), stream()),
-        "qb_ste_backward");
+  const int64_t N = w.size(0), K = w.size(1), groups = integer(a[2]);
+  const at::Device device = w.device();
+  const float* const g_data = g.const_data_ptr<float>();
+  const float* const w_data = static_cast<const float*>(w.const_data_ptr());
+  const float* const lo = static_cast<const float*>(ptr(a[3]));
+  const float* const hi = static_cast<const float*>(ptr(a[4]));
+  Out grad_w(a[5]);
+  qb_status st;
+  {
+    const Unlocked unlocked;
+    grad_w.make({N, K}, at::kFloat, device);
+    st = qb_ste_backward(g_data, w_data, N, K, (int)groups, lo, hi, static_cast<float*>(grad_w.data), stream());
+  }
+  check(st, "qb_ste_backward");
   return grad_w.get();
 }
 
@@ -232,34 +290,45 @@ PyObject* quantize_embedding(Args a) {
   const at::Tensor& t = input(a[0], at::kFloat, "table: a contiguous fp32 CUDA tensor of two dimensions");
   need(t.dim() == 2, "table: a contiguous fp32 CUDA tensor of two dimensions");
   const int64_t V = t.size(0), D = t.size(1), bits = integer(a[1]), groups = integer(a[2]);
+  const at::Device device = t.device();
+  const float* const table = t.const_data_ptr<float>();
   const Workspace ws(a[3]);
-  Out packed(a[4], {V, D * bits / 32}, at::kInt, t);
-  Out delta(Py_None, {std::max<int64_t>(groups, 0)}, at::kFloat, t), q0(Py_None, {std::max<int64_t>(groups, 0)}, at::kFloat, t);
-  check(qb_quantize_embedding(t.const_data_ptr<float>(), V, D, (int)bits, (int)groups, static_cast<uint32_t*>(packed.data),
-                              static_cast<float*>(delta.data), static_cast<float*>(q0.data), ws.data, ws.bytes, stream()),
-        "qb_quantize_embedding");
-  PyObject* r = PyTuple_New(3);
-  if (!r) throw Failed{};
-  PyTuple_SET_ITEM(r, 0, packed.get());
-  PyTuple_SET_ITEM(r, 1, delta.get());
-  PyTuple_SET_ITEM(r, 2, q0.get());
-  return r;
+  Out packed(a[4]), delta(Py_None), q0(Py_None);
+  qb_status st;
+  {
+    const Unlocked unlocked;
+    packed.make({V, D * bits / 32}, at::kInt, device);
+    delta.make({std::max<int64_t>(groups, 0)}, at::kFloat, device);
+    q0.make({std::max<int64_t>(groups, 0)}, at::kFloat, device);
+    st = qb_quantize_embedding(table, V, D, (int)bits, (int)groups, static_cast<uint32_t*>(packed.data),
+                               static_cast<float*>(delta.data), static_cast<float*>(q0.data), ws.data, ws.bytes, stream());
+  }
+  check(st, "qb_quantize_embedding");
+  return triple(packed, delta, q0);
 }
 
 // embedding_lookup(ids, packed, delta, q0, D, bits, groups, ws, out, accumulate) -> out
 PyObject* embedding_lookup(Args a) {
   const at::Tensor& ids = input(a[0], at::kInt, "ids: a contiguous int32 CUDA tensor");
   const at::Tensor& packed = tensor(a[1]);
-  const int64_t T = ids.numel(), V = packed.size(0), D = integer(a[4]);
+  const int64_t T = ids.numel(), V = packed.size(0), D = integer(a[4]), bits = integer(a[5]), groups = integer(a[6]);
+  const at::Device device = ids.device();
+  const int32_t* const id_data = ids.const_data_ptr<int32_t>();
+  const uint32_t* const codes = static_cast<const uint32_t*>(packed.const_data_ptr());
+  const float* const delta = static_cast<const float*>(ptr(a[2]));
+  const float* const q0 = static_cast<const float*>(ptr(a[3]));
   const Workspace ws(a[7]);
   const int accumulate = PyObject_IsTrue(a[9]);
   if (a[8] == Py_None) need(!accumulate, "accumulate needs `out`");
-  Out out(a[8], {T, D}, at::kFloat, ids);
-  check(qb_embedding_lookup(ids.const_data_ptr<int32_t>(), T, static_cast<const uint32_t*>(packed.const_data_ptr()),
-                            static_cast<const float*>(ptr(a[2])), static_cast<const float*>(ptr(a[3])), V, D,
-                            (int)integer(a[5]), (int)integer(a[6]), accumulate ? 1 : 0, static_cast<float*>(out.data),
-                            ws.data, ws.bytes, stream()),
-        "qb_embedding_lookup");
+  Out out(a[8]);
+  qb_status st;
+  {
+    const Unlocked unlocked;
+    out.make({T, D}, at::kFloat, device);
+    st = qb_embedding_lookup(id_data, T, codes, delta, q0, V, D, (int)bits, (int)groups, accumulate ? 1 : 0,
+                             static_cast<float*>(out.data), ws.data, ws.bytes, stream());
+  }
+  check(st, "qb_embedding_lookup");
   return out.get();
 }
 
@@ -270,7 +339,12 @@ PyObject* over_descs(Args a, const char* what) {
   const Workspace ws(a[1]);
   int32_t count = 0;
   const T* p = d.as<T>(&count);
-  check(F(p, count, ws.data, ws.bytes, stream()), what);
+  qb_status st;
+  {
+    const Unlocked unlocked;
+    st = F(p, count, ws.data, ws.bytes, stream());
+  }
+  check(st, what);
   Py_RETURN_NONE;
 }
 PyObject* quantize_act_batch(Args a) { return over_descs<qb_act_desc, qb_quantize_act_batch>(a, "qb_quantize_act_batch"); }
