@@ -229,7 +229,7 @@ def fake_quantize_weights(w: torch.Tensor, bits: int, groups: int, ws: torch.Ten
 def fake_quantize_weights_batch(items, ws: torch.Tensor) -> None:
     """``qb_fake_quantize_weights_batch`` over ``(w, bits, groups, wq, delta, q0)`` tuples (or a C array whose
     ``packed`` fields point to the fp32 outputs)."""
-    arr = items if isinstance(items, ctypes.Array) else make_weight_desc_array(items)
+    arr = _descs(items, WeightDescC, make_weight_desc_array)
     (_native or _ext()).fake_quantize_weights_batch(arr, ws)
 
 
@@ -252,6 +252,16 @@ def embedding_lookup(ids: torch.Tensor, packed: torch.Tensor, delta: torch.Tenso
     return (_native or _ext()).embedding_lookup(ids, packed, delta, q0, D, bits, groups, ws, out, accumulate)
 
 
+def _descs(items, kind, make):
+    """``items`` as a C array of ``kind``; an array of other elements is refused, as ctypes refuses it for a typed pointer
+    (``_qbert.so`` sees bytes)."""
+    if not isinstance(items, ctypes.Array):
+        return make(items)
+    if not issubclass(items._type_, kind):
+        raise ctypes.ArgumentError(f"expected an array of {kind.__name__}, got one of {items._type_.__name__}")
+    return items
+
+
 def make_act_desc_array(items):
     """``items``: sequence of ``(x, xq, act_scale, rowsum)`` tensors -> C array of ``qb_act_desc``."""
     arr = (ActDescC * len(items))()
@@ -263,7 +273,7 @@ def make_act_desc_array(items):
 
 def quantize_act_batch(items, ws: torch.Tensor) -> None:
     """``qb_quantize_act_batch`` over ``(x, xq, act_scale, rowsum)`` tuples (or a prepared C array)."""
-    arr = items if isinstance(items, ctypes.Array) else make_act_desc_array(items)
+    arr = _descs(items, ActDescC, make_act_desc_array)
     (_native or _ext()).quantize_act_batch(arr, ws)
 
 
@@ -279,7 +289,7 @@ def make_weight_desc_array(items):
 
 def quantize_pack_weights_batch(items, ws: torch.Tensor) -> None:
     """``qb_quantize_pack_weights_batch`` over ``(w, bits, groups, packed, delta, q0)`` tuples (or a C array)."""
-    arr = items if isinstance(items, ctypes.Array) else make_weight_desc_array(items)
+    arr = _descs(items, WeightDescC, make_weight_desc_array)
     (_native or _ext()).quantize_pack_weights_batch(arr, ws)
 
 
@@ -389,7 +399,7 @@ def make_desc_array(descs: Sequence[LinearDesc]):
 
 def layer_linears(descs, ws: torch.Tensor) -> None:
     """``qb_layer_linears`` over a list of ``LinearDesc`` (or an array from ``make_desc_array``)."""
-    arr = descs if isinstance(descs, ctypes.Array) else make_desc_array(descs)
+    arr = _descs(descs, LinearDescC, make_desc_array)
     (_native or _ext()).layer_linears(arr, ws)
 
 
@@ -422,5 +432,5 @@ def layer_linears_bf16(descs, ws: torch.Tensor) -> None:
     """``qb_layer_linears_bf16``: as ``layer_linears``, every ``y`` a bfloat16 [M,N] tensor."""
     if not isinstance(descs, ctypes.Array):
         assert all(d.y.dtype == torch.bfloat16 for d in descs)
-        descs = make_desc_array(descs)
-    (_native or _ext()).layer_linears_bf16(descs, ws)
+    arr = _descs(descs, LinearDescC, make_desc_array)
+    (_native or _ext()).layer_linears_bf16(arr, ws)
