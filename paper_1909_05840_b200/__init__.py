@@ -3,8 +3,8 @@
 Every step of the path (activation quantizer, group-wise weight quantizer and packer, integer
 GEMM with dequantizing epilogue, encoder-layer linear stack) runs in the CUDA kernels behind the C
 ABI declared in ``include/qbert.h``.  torch is used for device buffers and the current stream.  The calls
-that a model makes on every pass go through ``_qbert.so`` (tensors read, outputs allocated and the stream
-looked up in C++), the others through ctypes.  There is no CPU fallback: if the libraries have not been
+that a model makes on every pass go through the extension module ``_qbert`` (tensors read, outputs allocated and the
+stream looked up in C++), the others through ctypes.  There is no CPU fallback: if the libraries have not been
 built, importing works but the first call raises ``QbertError``.
 """
 from __future__ import annotations
@@ -12,6 +12,7 @@ from __future__ import annotations
 import ctypes
 import importlib.machinery
 import importlib.util
+import sysconfig
 from dataclasses import dataclass
 from pathlib import Path
 from typing import Optional, Sequence
@@ -20,7 +21,9 @@ import torch
 
 _PKG = Path(__file__).resolve().parent
 LIB_PATH = _PKG / "libqbert.so"
-EXT_PATH = _PKG / "_qbert.so"  # the calls made on every pass, marshalled in C++ (csrc/binding.cpp)
+# The calls made on every pass, marshalled in C++ (csrc/binding.cpp).  The module uses torch's and Python's C++ interfaces,
+# which change between versions: it carries both in its name, so that one built for others is never loaded.
+EXT_PATH = _PKG / f"_qbert.torch-{torch.__version__}.{sysconfig.get_config_var('SOABI')}.so"
 
 QB_OK = 0
 QB_ERR_INVALID = -1
@@ -152,11 +155,11 @@ _native = None
 
 
 def _ext():
-    """Load ``_qbert.so`` on the first call that needs it."""
+    """Load the extension module on the first call that needs it."""
     global _native
     lib()
     if not EXT_PATH.exists():
-        raise QbertError(QB_ERR_CUDA, f"{EXT_PATH} is missing: build it with "
+        raise QbertError(QB_ERR_CUDA, f"{EXT_PATH} is missing (not built for this torch and Python): build it with "
                                       "`python -m paper_1909_05840_b200.build`; there is no CPU fallback")
     loader = importlib.machinery.ExtensionFileLoader("_qbert", str(EXT_PATH))
     mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("_qbert", loader))
@@ -254,7 +257,7 @@ def embedding_lookup(ids: torch.Tensor, packed: torch.Tensor, delta: torch.Tenso
 
 def _descs(items, kind, make):
     """``items`` as a C array of ``kind``; an array of other elements is refused, as ctypes refuses it for a typed pointer
-    (``_qbert.so`` sees bytes)."""
+    (``_qbert`` sees bytes)."""
     if not isinstance(items, ctypes.Array):
         return make(items)
     if not issubclass(items._type_, kind):

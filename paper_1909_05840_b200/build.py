@@ -1,4 +1,4 @@
-"""Build libqbert.so in-tree with nvcc for sm_100a, and the Python entry to it, _qbert.so, with the host compiler (no
+"""Build libqbert.so in-tree with nvcc for sm_100a, and the Python entry to it, _qbert, with the host compiler (no
 JIT cache: the built libraries travel with the tree)."""
 from __future__ import annotations
 
@@ -8,11 +8,12 @@ import sys
 import sysconfig
 from pathlib import Path
 
+from . import EXT_PATH as EXT
+
 PKG = Path(__file__).resolve().parent
 CSRC = PKG / "csrc"
 INCLUDE = PKG.parent / "include"
 LIB = PKG / "libqbert.so"
-EXT = PKG / "_qbert.so"
 SOURCES = ["api.cu", "quantize_act.cu", "quantize_weights.cu", "quantize_weights_noalloc.cu", "gemm.cu", "probe.cu", "embedding.cu", "sensitivity.cu"]
 
 
@@ -21,12 +22,24 @@ def _nvcc() -> str:
     return cand if Path(cand).exists() else "nvcc"
 
 
-def needs_build() -> bool:
-    if not LIB.exists() or not EXT.exists():
+def _stale(target: Path, *patterns: str) -> bool:
+    if not target.exists():
         return True
-    t = min(LIB.stat().st_mtime, EXT.stat().st_mtime)
-    deps = [d for pattern in ("*.cu", "*.cuh", "*.cpp") for d in CSRC.glob(pattern)] + list(INCLUDE.glob("*.h"))
+    t = target.stat().st_mtime
+    deps = [d for pattern in patterns for d in CSRC.glob(pattern)] + list(INCLUDE.glob("*.h"))
     return any(d.stat().st_mtime > t for d in deps)
+
+
+def _lib_stale() -> bool:
+    return _stale(LIB, "*.cu", "*.cuh")
+
+
+def _ext_stale() -> bool:
+    return _stale(EXT, "*.cpp")
+
+
+def needs_build() -> bool:
+    return _lib_stale() or _ext_stale()
 
 
 def _binding_command(out: str) -> list[str]:
@@ -42,8 +55,16 @@ def _binding_command(out: str) -> list[str]:
 
 def build(force: bool = False, verbose: bool = False) -> Path:
     """Compile every CUDA source of the library for sm_100a into one shared object, then the Python entry to it."""
-    if not force and not needs_build():
-        return LIB
+    if force or _lib_stale():
+        _build_lib(verbose)
+    if force or _ext_stale():
+        tmp = str(EXT) + ".tmp"
+        subprocess.run(_binding_command(tmp), check=True)
+        os.replace(tmp, EXT)
+    return LIB
+
+
+def _build_lib(verbose: bool) -> None:
     objs = []
     build_dir = PKG / "_build"
     build_dir.mkdir(exist_ok=True)
@@ -68,10 +89,6 @@ def build(force: bool = False, verbose: bool = False) -> Path:
     tmp = str(LIB) + ".tmp"
     subprocess.run([_nvcc(), "-shared", "-Wno-deprecated-gpu-targets", "-o", tmp, *objs, "-cudart", "static"], check=True)
     os.replace(tmp, LIB)
-    tmp = str(EXT) + ".tmp"
-    subprocess.run(_binding_command(tmp), check=True)
-    os.replace(tmp, EXT)
-    return LIB
 
 
 if __name__ == "__main__":
