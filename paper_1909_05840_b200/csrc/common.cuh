@@ -105,6 +105,15 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned b
   return cudaLaunchKernelEx(&cfg, kernel, std::decay_t<P>(args)...);
 }
 
+// Was a launch refused because its blocks (of a cooperative launch, of a cluster) cannot be resident together?  The
+// grids are made for the whole device; a green context or an MPS client may have fewer SMs.  The forms that need
+// residency have one beside them that does not, which such a launch falls back to.
+inline bool residency_refused(cudaError_t e) {
+  if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorInvalidClusterSize) return false;
+  cudaGetLastError();  // not an error of the call
+  return true;
+}
+
 // ---- device-side helpers -----------------------------------------------------------------------
 #ifdef __CUDACC__
 // Called by every thread of a kernel started by launch_kernel before it touches global memory: waits until the

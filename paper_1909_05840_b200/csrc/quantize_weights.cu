@@ -1362,7 +1362,7 @@ static qb_status launch_regs(const HostWeight* m_all, int count_all, void* ws, i
 
 // One pair of launches (clear, ring kernel) over `count` matrices (<= kMaxWeightBatch) whose groups fit the ring.
 template <bool FAKE>
-static qb_status launch_ring_form(const RingBatch& b, unsigned grid, cudaStream_t stream) {
+static qb_status launch_ring_form(const RingBatch& b, unsigned grid, cudaStream_t stream, bool* refused) {
   static std::atomic<bool> attr_set[64] = {};
   int dev = 0;
   QB_CUDA_TRY(cudaGetDevice(&dev));
@@ -1370,10 +1370,14 @@ static qb_status launch_ring_form(const RingBatch& b, unsigned grid, cudaStream_
     QB_CUDA_TRY(cudaFuncSetAttribute(weight_ring_kernel<FAKE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingSmemBytes));
     if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_release);
   }
-  QB_CUDA_TRY(launch_kernel(weight_ring_kernel<FAKE>, grid, kRingThreads, kRingSmemBytes, stream, true, 1, true, b));
+  const cudaError_t e = launch_kernel(weight_ring_kernel<FAKE>, grid, kRingThreads, kRingSmemBytes, stream, true, 1, true, b);
+  *refused = residency_refused(e);
+  if (!*refused) QB_CUDA_TRY(e);
   return QB_OK;
 }
-static qb_status launch_ring(const HostWeight* m, int count, void* ws, int sm_count, cudaStream_t stream, bool fake) {
+// `refused`: nothing was rounded, the blocks cannot all be resident.
+static qb_status launch_ring(const HostWeight* m, int count, void* ws, int sm_count, cudaStream_t stream, bool fake,
+                             bool* refused) {
   RingBatch b;
   int groups = 0, chunks = 0;
   for (int i = 0; i < count; ++i) {
@@ -1400,7 +1404,7 @@ static qb_status launch_ring(const HostWeight* m, int count, void* ws, int sm_co
   const int slots = groups * (int)grid;
   QB_CUDA_TRY(launch_kernel(clear_slots_kernel, (unsigned)std::min((slots + 255) / 256, sm_count), 256, 0, stream, true, 1, false,
                             b.slots, slots));
-  return fake ? launch_ring_form<true>(b, grid, stream) : launch_ring_form<false>(b, grid, stream);
+  return fake ? launch_ring_form<true>(b, grid, stream, refused) : launch_ring_form<false>(b, grid, stream, refused);
 }
 
 // Matrices whose groups do not fit a cluster's registers: the ring as long as a group spans few enough rounds of
@@ -1435,9 +1439,10 @@ static std::vector<LargeJob> plan_large_groups(const std::vector<HostWeight>& m,
 static qb_status launch_large_groups(const std::vector<HostWeight>& m, void* ws, size_t ws_bytes, int sm_count,
                                      cudaStream_t stream, bool fake) {
   for (const LargeJob& j : plan_large_groups(m, sm_count)) {
-    const bool ring = j.ring && kWsRangeOff + ring_table_bytes((size_t)j.groups) <= ws_bytes;
-    qb_status st = ring ? launch_ring(j.m.data(), (int)j.m.size(), ws, sm_count, stream, fake)
-                        : launch_two_pass(j.m.data(), (int)j.m.size(), ws, sm_count, stream, fake);
+    bool two_pass = !j.ring || kWsRangeOff + ring_table_bytes((size_t)j.groups) > ws_bytes;
+    qb_status st = QB_OK;
+    if (!two_pass) st = launch_ring(j.m.data(), (int)j.m.size(), ws, sm_count, stream, fake, &two_pass);
+    if (st == QB_OK && two_pass) st = launch_two_pass(j.m.data(), (int)j.m.size(), ws, sm_count, stream, fake);
     if (st != QB_OK) return st;
   }
   return QB_OK;
