@@ -14,9 +14,9 @@ namespace qb {
 // [0]   int32  status   first device-side error, never cleared by a kernel
 // [4]   int32  detail   where a bounded wait gave up (role << 16 | stage), diagnostics only
 // [16]  uint32 act_absmax_bits   reduction slot of act_absmax_kernel for a single tensor
-// [32]  uint32 ticket            blocks of the running launch that have started        } zero between
-// [36]  uint32 cleared           1 once the running launch's reduction slots are clear } calls
-// [40]  uint32 round             counts the launches whose clusters waited for one another
+// [32]  uint64 ticket            launches that cleared slots << 32 | blocks of the running one that have started
+// [40]  uint32 cleared           number of the last such launch whose reduction slots are clear
+// [44]  uint32 round             counts the launches whose clusters waited for one another
 // [64]  uint64 cluster_max[24]   round << 32 | bit pattern of a cluster's max|x|, all of the last such launch
 // [256] uint32 range_hi_enc[G], uint32 range_lo_inv[G]   ordered encodings of per-group max / min
 //       or, weight_ring_kernel: uint64 [groups][CTAs], encoded max << 32 | inverted encoded min
@@ -33,10 +33,10 @@ struct WsHeader {
   uint32_t pad[2];
   uint32_t act_absmax_bits;
   uint32_t pad2[3];
-  uint32_t ticket;
+  unsigned long long ticket;
   uint32_t cleared;
   uint32_t round;
-  uint32_t pad3[5];
+  uint32_t pad3[4];
   unsigned long long cluster_max[kWsClusters];
 };
 static_assert(sizeof(WsHeader) == kWsRangeOff, "the tables follow the header");
@@ -177,16 +177,25 @@ __device__ __forceinline__ void st_release(uint32_t* p, uint32_t v) {
 }
 // Called by one warp of every block: the block that comes first clears the launch's reduction slots and says so
 // (whichever block it is, it is running, so nobody waits for a block that has not started).  The others
-// look (h->cleared) before they publish; by then they have read their share of the input and the wait is
-// over before it begins.  The next launch on the stream sets ticket and cleared back to zero.
-__device__ __forceinline__ void clear_slots(uint32_t* slots, int count, WsHeader* h, int lane) {
-  uint32_t ticket = 0;
-  if (lane == 0) ticket = atomicAdd(&h->ticket, 1u);
-  if (__shfl_sync(0xffffffffu, ticket, 0) != 0u) return;
-  for (int i = lane; i < count; i += 32) slots[i] = 0u;
-  __threadfence();
-  __syncwarp();
-  if (lane == 0) st_release(&h->cleared, 1u);
+// look before they publish (h->cleared shows the number returned here); by then they have read their share of the
+// input and the wait is over before it begins.  The block that comes last opens the next launch's count, so that nothing
+// is left for a later kernel to put back: one that is never launched would leave the next call with slots that
+// count as clear.
+__device__ __forceinline__ uint32_t clear_slots(uint32_t* slots, int count, WsHeader* h, int lane) {
+  unsigned long long t = 0;
+  if (lane == 0) {
+    t = atomicAdd(&h->ticket, 1ull);
+    if ((uint32_t)t == gridDim.x - 1) atomicAdd(&h->ticket, (1ull << 32) - gridDim.x);
+  }
+  t = __shfl_sync(0xffffffffu, t, 0);
+  const uint32_t launch = (uint32_t)(t >> 32) + 1u;
+  if ((uint32_t)t == 0u) {
+    for (int i = lane; i < count; i += 32) slots[i] = 0u;
+    __threadfence();
+    __syncwarp();
+    if (lane == 0) st_release(&h->cleared, launch);
+  }
+  return launch;
 }
 // 16-byte load with an L2 eviction-priority policy (createpolicy).  The two-pass quantizers use it: the
 // first pass asks L2 to keep a fraction of what it reads (the second pass reads the same tensor next),

@@ -49,6 +49,7 @@ emb_range_kernel(const float4* e, int64_t V, int d4, int slots, int cols_per_gro
   float lo[4] = {kInf, kInf, kInf, kInf}, hi[4] = {-kInf, -kInf, -kInf, -kInf};
   const int64_t step = (int64_t)gridDim.x * slots;
   bool cleared = threadIdx.x >= 32;
+  uint32_t launch = 0;
   for (int64_t r = (int64_t)blockIdx.x * slots + slot; r < V; r += kEmbRangeRows * step) {
     float4 v[kEmbRangeRows];
 #pragma unroll
@@ -56,7 +57,7 @@ emb_range_kernel(const float4* e, int64_t V, int d4, int slots, int cols_per_gro
       v[j] = ldg_policy(e + (r + j * step < V ? r + j * step : r) * d4 + q, pol);
     if (!cleared) {  // the block's first warp (its first row exists), while its first loads are on their way
       cleared = true;
-      clear_slots(g_hi, 2 * groups, h, threadIdx.x);
+      launch = clear_slots(g_hi, 2 * groups, h, threadIdx.x);
     }
 #pragma unroll
     for (int j = 0; j < kEmbRangeRows; j += 2) {
@@ -77,7 +78,7 @@ emb_range_kernel(const float4* e, int64_t V, int d4, int slots, int cols_per_gro
     mine[4 * q + i] = float_to_ordered(hi[i]);
     mine[D + 4 * q + i] = ~float_to_ordered(lo[i]);
   }
-  if (threadIdx.x == 0 && !poll_word(&h->cleared, 1u)) report_status(ws, QB_ERR_TIMEOUT);
+  if (threadIdx.x == 0 && !poll_word(&h->cleared, launch)) report_status(ws, QB_ERR_TIMEOUT);
   __syncthreads();
   // groups of few columns: a thread each; of many: a warp each
   const bool by_warp = cols_per_group >= 16;
@@ -157,11 +158,6 @@ emb_pack_kernel(const float4* e, int64_t V, int d4, int slots, int cols_per_grou
                 const uint32_t* g_hi, const uint32_t* g_lo_inv, uint32_t* packed, float* delta, float* q0, void* ws) {
   constexpr int L = (1 << BITS) - 1;
   pdl_begin();
-  if (blockIdx.x == 0 && threadIdx.x == 0) {  // for the next call; nothing of this launch reads them
-    WsHeader* const h = reinterpret_cast<WsHeader*>(ws);
-    h->ticket = 0u;
-    h->cleared = 0u;
-  }
   const int q = threadIdx.x % d4, slot = threadIdx.x / d4, lane = threadIdx.x & 31;
   const uint64_t pol = policy_evict_first();
   const int64_t step = (int64_t)gridDim.x * slots;

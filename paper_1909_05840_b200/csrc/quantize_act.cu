@@ -133,6 +133,7 @@ act_absmax_kernel(const __grid_constant__ ActBatch<P> b) {
   const int64_t u0 = (int64_t)blockIdx.x * b.units_per_block;
   const int64_t u1 = min(u0 + b.units_per_block, b.units_total);
   bool cleared = warp != 0;
+  uint32_t launch = 0;
   const int first = find_item<P, &ActItem::unit_begin>(b, u0);
   int it = first;
   for (; it < b.count && b.item[it].unit_begin < u1; ++it) {
@@ -152,7 +153,7 @@ act_absmax_kernel(const __grid_constant__ ActBatch<P> b) {
         if (j < n) v[j] = ldg_policy(x + (u + j) * 32, pol);
       if (!cleared) {  // warp 0, while its first loads are on their way (every block has at least one unit)
         cleared = true;
-        clear_slots(b.absmax_bits, b.count, h, lane);
+        launch = clear_slots(b.absmax_bits, b.count, h, lane);
       }
 #pragma unroll
       for (int j = 0; j < kSegUnits; ++j)
@@ -162,7 +163,7 @@ act_absmax_kernel(const __grid_constant__ ActBatch<P> b) {
     if (lane == 0 && m != 0u) atomicMax(&s_max[it], m);
   }
   __syncthreads();
-  if (threadIdx.x == 0 && !poll_word(&h->cleared, 1u)) report_status(b.ws, QB_ERR_TIMEOUT);
+  if (threadIdx.x == 0 && !poll_word(&h->cleared, launch)) report_status(b.ws, QB_ERR_TIMEOUT);
   __syncthreads();
   for (int i = first + threadIdx.x; i < it; i += kActThreads)
     if (s_max[i] != 0u) atomicMax(b.absmax_bits + i, s_max[i]);
@@ -191,12 +192,7 @@ template <int P>
 __global__ void __launch_bounds__(kActThreads, kActBlocksPerSm)
 act_quantize_kernel(const __grid_constant__ ActBatch<P> b) {
   const int lane = threadIdx.x & 31;
-  WsHeader* const h = reinterpret_cast<WsHeader*>(b.ws);
   pdl_begin();
-  if (blockIdx.x == 0 && threadIdx.x == 0) {  // for the next call; nothing of this launch reads them
-    h->ticket = 0u;
-    h->cleared = 0u;
-  }
   const int64_t warps = (int64_t)gridDim.x * kActWarps;
   const uint64_t pol = policy_evict_first();
   const int64_t s0 = (int64_t)blockIdx.x * kActWarps + (threadIdx.x >> 5);
