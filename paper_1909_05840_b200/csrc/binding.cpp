@@ -319,6 +319,7 @@ PyObject* embedding_lookup(Args a) {
   const float* const q0 = static_cast<const float*>(ptr(a[3]));
   const Workspace ws(a[7]);
   const int accumulate = PyObject_IsTrue(a[9]);
+  if (accumulate < 0) throw Failed{};
   if (a[8] == Py_None) need(!accumulate, "accumulate needs `out`");
   Out out(a[8]);
   qb_status st;

@@ -22,3 +22,19 @@ def test_descriptor_arrays_are_typed(call, kind):
     assert qb._descs((kind * 3)(), kind, None)._length_ == 3
     derived = type("Derived", (kind,), {})
     assert qb._descs((derived * 2)(), kind, None)._length_ == 2
+
+
+@pytest.mark.gpu
+def test_truth_value_that_raises():
+    ws = qb.workspace(groups=256)
+    packed, delta, q0 = qb.quantize_embedding(torch.rand((8, 128), device="cuda"), 4, 8, ws)
+    ids = torch.zeros(3, dtype=torch.int32, device="cuda")
+
+    class NoTruth:
+        def __bool__(self):
+            raise ValueError("no truth value")
+
+    out = torch.zeros((3, 128), device="cuda")
+    with pytest.raises(ValueError, match="no truth value"):
+        qb.embedding_lookup(ids, packed, delta, q0, 128, 4, 8, ws, out=out, accumulate=NoTruth())
+    assert not out.any()
