@@ -261,6 +261,13 @@ int32_t qb_quantize_pack_weights_launch_count(const qb_weight_desc* descs /*host
 int32_t qb_layer_linears_launch_count(const qb_linear_desc* descs /*host*/, int32_t count);
 
 /*
+ * Tokens per tile (128, 192 or 256) of launch number `launch` of such a stack; `out` 0: fp32 outputs, 1: bfloat16,
+ * 2: int8.  Host arithmetic as above (a single linear is a stack of one).  (No counterpart in the paper; it
+ * lets a test see which kernel a shape is served by.)  Returns 0 for a null or empty stack or a launch it does not have.
+ */
+int32_t qb_layer_linears_tile_tokens(const qb_linear_desc* descs /*host*/, int32_t count, int32_t out, int32_t launch);
+
+/*
  * Narrow-output forms of qb_gemm and qb_layer_linears.  The paper keeps the activations between
  * layers at 8 bits (Table 1 caption: every quantized model uses 8-bit activations), so the fp32
  * result of a linear is an intermediate that the next operation narrows again; writing it as

@@ -39,7 +39,7 @@ EXPORTS = (
     "qb_layer_linears", "qb_quantize_pack_weights_noalloc", "qb_probe_i8_mma", "qb_quantize_act_batch",
     "qb_quantize_pack_weights_batch", "qb_gemm_bf16", "qb_layer_linears_bf16",
     "qb_fake_quantize_weights", "qb_fake_quantize_weights_batch", "qb_ste_backward", "qb_quantize_embedding", "qb_embedding_lookup",
-    "qb_gemm_i8", "qb_rowsum_i8", "qb_layer_linears_i8", "qb_sensitivity_bits", "qb_probe_wait_limit", "qb_layer_linears_launch_count", "qb_quantize_pack_weights_launch_count", "qb_quantize_act_launch_count",
+    "qb_gemm_i8", "qb_rowsum_i8", "qb_layer_linears_i8", "qb_sensitivity_bits", "qb_probe_wait_limit", "qb_layer_linears_launch_count", "qb_layer_linears_tile_tokens", "qb_quantize_pack_weights_launch_count", "qb_quantize_act_launch_count",
 )
 NOALLOC_MAX_GROUPS = 4096
 
@@ -110,6 +110,8 @@ def lib() -> ctypes.CDLL:
     L.qb_probe_i8_mma.restype = i32
     L.qb_layer_linears_launch_count.argtypes = [ctypes.POINTER(LinearDescC), i32]
     L.qb_layer_linears_launch_count.restype = i32
+    L.qb_layer_linears_tile_tokens.argtypes = [ctypes.POINTER(LinearDescC), i32, i32, i32]
+    L.qb_layer_linears_tile_tokens.restype = i32
     L.qb_quantize_pack_weights_launch_count.argtypes = [ctypes.POINTER(WeightDescC), i32]
     L.qb_quantize_pack_weights_launch_count.restype = i32
     L.qb_quantize_act_launch_count.argtypes = [i32]
@@ -421,6 +423,12 @@ def layer_linears_launch_count(descs) -> int:
     """``qb_layer_linears_launch_count``: GEMM kernel launches ``layer_linears`` issues for this stack."""
     arr = descs if isinstance(descs, ctypes.Array) else make_desc_array(descs)
     return int(lib().qb_layer_linears_launch_count(arr, len(arr)))
+
+
+def layer_linears_tile_tokens(descs, out: torch.dtype = torch.float32, launch: int = 0) -> int:
+    """``qb_layer_linears_tile_tokens``: tokens per tile of one launch of this stack (a single linear is a stack of one)."""
+    arr = descs if isinstance(descs, ctypes.Array) else make_desc_array(descs)
+    return int(lib().qb_layer_linears_tile_tokens(arr, len(arr), (torch.float32, torch.bfloat16, torch.int8).index(out), launch))
 
 
 def layer_linears_i8(descs: Sequence[LinearDesc], out_scales: Sequence[torch.Tensor], ws: torch.Tensor) -> None:

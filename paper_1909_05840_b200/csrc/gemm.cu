@@ -1018,7 +1018,12 @@ static qb_status launch_group_bits(int bits, const GP& gp, int grid, cudaStream_
 // `cg_out`: CTAs per tile.  A launch with at least one 256 x 256 tile per pair of SMs runs as CTA pairs: each
 // CTA then stages half of the token tile (half the L2 and shared-memory traffic per MMA) and the ring is
 // five K blocks deep instead of three.
-static int choose_token_tile(const qb_linear_desc* d, const int* idx, int count, int sm_count, int* cg_out) {
+static int choose_token_tile(const qb_linear_desc* d, const int* idx, int count, int sm_count, int out, int* cg_out) {
+  for (int i = 1; i < count; ++i)
+    if (d[idx[i]].bits != d[idx[0]].bits) {  // mixed widths: built for small stacks only (128-token tiles, single CTAs)
+      *cg_out = 1;
+      return 128;
+    }
   bool wide = false;
   int64_t tiles256 = 0, tiles_pair = 0;
   for (int i = 0; i < count; ++i) {
@@ -1029,10 +1034,15 @@ static int choose_token_tile(const qb_linear_desc* d, const int* idx, int count,
   *cg_out = 1;
   if (wide && sm_count >= 2 && tiles_pair >= sm_count / 2 && g_pair_mode != 0) {
     *cg_out = 2;
-    // 192 tokens per tile when that leaves the pairs less idle at the end.  Measured per tile (12 and 16 full rounds of
-    // all pairs, 4 bits, hundredths of a microsecond): 283 + 37 per K block at 256 tokens, 222 + 31 at 192, that
-    // is 8-10 % more per token; 6144 x 4096 x 1024 (5.2 rounds of 256-token tiles) 41.2 -> 38.9 us,
-    // 6144 x 1024 x 4096 (1.3 rounds) 33.8 -> 29.5 us.
+    // 192 tokens per tile when that leaves the pairs less idle at the end: 6144 x 4096 x 1024 (4 bits, 5.2 rounds of
+    // 256-token tiles) 35.4 -> 34.7 us, 6144 x 1024 x 4096 (1.3 rounds) 28.9 -> 26.3 us.  Costs of a tile in hundredths of
+    // a microsecond, fitted to 72 shapes of one linear (M = 1,280 to 24,576, K = 768 to 4,096) at every width and output
+    // type: a part that the output type decides, and a part per K block that the width decides (at 3 bits the
+    // expanders bound it, so that a narrower tile saves little).  One set of costs for all, taken at 4 bits and fp32,
+    // chose 192 where it lost up to 9 % (24576 x 1024 x 4096, 3 bits).  192 has to be cheaper by 2 %: over those shapes it
+    // then loses 2.9 % at most (7000 x 4096 x 1024, 3 bits, int8), where 256 alone would lose up to 14.6 %.
+    constexpr int kFixed[3][2] = {{292, 228}, {262, 203}, {366, 279}};  // [output][256, 192 tokens]
+    const auto per_block = [](int bits, int w) { return bits == 3 ? (w ? 41 : 43) : (bits == 8 ? (w ? 31 : 35) : (w ? 27 : 30)); };
     const int pairs = sm_count / 2;
     int64_t est[2];
     for (int w = 0; w < 2; ++w) {
@@ -1042,7 +1052,7 @@ static int choose_token_tile(const qb_linear_desc* d, const int* idx, int count,
       for (int i = 0; i < count; ++i) {
         const qb_linear_desc& q = d[idx[i]];
         const int64_t n = ((q.N + 2 * kTileN - 1) / (2 * kTileN)) * ((q.M + bt - 1) / bt);
-        const int64_t cost = w ? 222 + 31 * (q.K / kBlockK) : 283 + 37 * (q.K / kBlockK);
+        const int64_t cost = kFixed[out][w] + per_block(q.bits, w) * (q.K / kBlockK);
         tiles += n;
         sum += n * cost;
         longest = std::max(longest, cost);
@@ -1051,7 +1061,7 @@ static int choose_token_tile(const qb_linear_desc* d, const int* idx, int count,
       // tiles of one length: whole rounds; of several: the balanced lists end about half a long tile apart
       est[w] = uniform ? (tiles + pairs - 1) / pairs * longest : sum / pairs + longest / 2;
     }
-    return est[1] < est[0] ? 192 : 256;
+    return est[1] * 100 < est[0] * 98 ? 192 : 256;
   }
   // a launch that cannot give every SM a 256-token tile uses 128-token tiles: twice the CTAs at work,
   // half the epilogue per tile
@@ -1156,11 +1166,7 @@ static qb_status launch_group(const qb_linear_desc* d, const int* idx, int count
   for (int i = 1; i < count; ++i)
     if (d[idx[i]].bits != bits) bits = 0;
   int cg = 1;
-  int bt = choose_token_tile(d, idx, count, sm_count, &cg);
-  if (bits == 0) {  // mixed widths: built for small stacks only (128-token tiles, single CTAs)
-    cg = 1;
-    bt = 128;
-  }
+  const int bt = choose_token_tile(d, idx, count, sm_count, out, &cg);
   const int group_n = kTileN * cg;
   GP gp;  // every field that the kernel reads for `count` linears is written below
   gp.ws = ws;
@@ -1396,6 +1402,18 @@ extern "C" int32_t qb_layer_linears_launch_count(const qb_linear_desc* descs, in
   qb::require_sm100(&sms);  // without a device: the plan for a 148-SM part
   qb::plan_stack(descs, count, sms, order, groups);
   return (int32_t)groups.size();
+}
+
+extern "C" int32_t qb_layer_linears_tile_tokens(const qb_linear_desc* descs, int32_t count, int32_t out, int32_t launch) {
+  if (!descs || count <= 0 || out < 0 || out > 2 || launch < 0) return 0;
+  int sms = 148;
+  qb::require_sm100(&sms);  // without a device: the plan for a 148-SM part
+  std::vector<int> order;
+  std::vector<qb::StackGroup> groups;
+  qb::plan_stack(descs, count, sms, order, groups);
+  if (launch >= (int)groups.size()) return 0;
+  int cg = 1;
+  return qb::choose_token_tile(descs, order.data() + groups[launch].begin, groups[launch].count, sms, out, &cg);
 }
 
 extern "C" qb_status qb_layer_linears(const qb_linear_desc* descs, int32_t count, void* ws, size_t ws_bytes,
