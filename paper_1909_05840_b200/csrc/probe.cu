@@ -37,7 +37,9 @@ __global__ void __launch_bounds__(128, 1) probe_i8_kernel(int k_blocks) {
   __syncthreads();
   ptx::tcgen05_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  if (threadIdx.x == 0) {
+  // The issuing thread is elected, as in the GEMM: its operands then stay in uniform registers.  (From threadIdx.x == 0
+  // every width took about 500 cycles a K block: the issue was what the probe measured.)
+  if (threadIdx.x < 32 && ptx::elect_one()) {
     const uint32_t idesc = (2u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TOKENS >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
     const uint64_t a_desc = probe_desc(a_addr), b_desc = probe_desc(b_addr);
     const long long t0 = clock64();
