@@ -140,7 +140,7 @@ def test_weight_launch_count_is_host_arithmetic(lib):
     mixed = [(N, K, (2, 3, 4, 8)[l % 4], G, False) for l in range(12) for (N, K, G) in base]
     assert lib.qb_quantize_pack_weights_launch_count(arr_of(mixed), len(mixed)) == 1      # a mixed-precision stack: one launch
     assert lib.qb_quantize_pack_weights_launch_count(arr_of(mixed * 3), 3 * len(mixed)) == 2  # 144 matrices: 96 + 48
-    assert lib.qb_quantize_pack_weights_launch_count(arr_of([(768, 768, 4, 1, False)]), 1) == 2  # one range per tensor: two passes
+    assert lib.qb_quantize_pack_weights_launch_count(arr_of([(768, 768, 4, 1, False)]), 1) == 2  # one range per tensor: clear and ring
     both = [(768, 768, 4, 128, False), (768, 768, 4, 1, False)]
     assert lib.qb_quantize_pack_weights_launch_count(arr_of(both), 2) == 3
     clustered = [(768, 768, 4, 12, False), (3072, 768, 2, 12, False), (768, 768, 3, 128, False)]  # clusters of 2 and 6, and single CTAs

@@ -23,7 +23,7 @@ def ws():
 @pytest.mark.parametrize("N,K,groups", [(768, 768, 12), (264, 384, 11), (96, 3072, 96), (128, 128, 1), (3072, 768, 128),
                                         (70, 256, 70),     # two units per group: nine groups per warp, a last warp with fewer
                                         (12, 30720, 2),    # 1,440 units per group: a cluster of five CTAs
-                                        (74, 8192, 2)])    # 2,368 units per group: the two-pass path
+                                        (74, 8192, 2)])    # 2,368 units per group: the ring
 def test_fake_quantize_matches_oracle(ws, bits, N, K, groups):
     w = synth.weights(N, K, seed=3 * N + K + groups + bits)
     wq = gu.poison(torch.empty((N, K), dtype=torch.float32, device="cuda"))
@@ -64,7 +64,7 @@ def test_fake_quantize_clipped_ranges_constant_group_and_nonfinite(ws):
 
 def test_fake_quantize_batch_equals_single_calls_and_the_oracle():
     # a stack in one call: mixed bit widths, groups held by one CTA, by clusters, several per warp, caller
-    # ranges, and one matrix whose groups take the two passes
+    # ranges, and one matrix whose groups take the ring
     shapes = [(768, 768, 4, 128, False), (3072, 768, 2, 128, False), (768, 3072, 3, 128, False), (70, 256, 8, 70, False),
               (768, 768, 3, 12, False), (12, 30720, 4, 2, False), (74, 8192, 2, 2, False), (264, 384, 4, 11, True),
               (768, 768, 8, 1, True)]

@@ -27,7 +27,7 @@ def ws():
 
 def test_quantizers_at_max_k(ws):
     # activations: three rows of 65536; weights: rows of 512 units in groups held by a cluster of four CTAs
-    # (2 rows per group), by a cluster of two (1 row per group), and by the two passes (one range per tensor)
+    # (2 rows per group), by a cluster of two (1 row per group), and by the ring (one range per tensor)
     x = synth.activations(3, MAX_K, seed=1)
     xq, sc, rs = gu.gpu_quantize_act(x, ws)
     st, o_xq, o_s, o_rs = oracle.quantize_act(x)

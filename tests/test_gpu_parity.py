@@ -182,7 +182,7 @@ def test_quantize_weights_register_path_shapes():
 def test_quantize_weights_cluster_path_shapes():
     # groups of 289 to 2,304 units are held by a thread-block cluster of 2 to 8 CTAs: every cluster size, slices
     # with ragged ends and warps that get nothing, more groups than resident clusters (several items per
-    # cluster), all bit widths; 2,368 units is past the largest cluster and takes the two passes
+    # cluster), all bit widths; 2,368 units is past the largest cluster and takes the ring
     _check_weight_batch([(34, 2176, 4, 2), (36, 4096, 2, 2), (40, 3712, 3, 2), (12, 30720, 8, 2), (72, 8192, 4, 2),
                          (74, 8192, 3, 2), (2560, 1536, 2, 80), (2048, 9600, 4, 512), (2640, 1536, 8, 80),
                          (1000, 2560, 3, 50), (1400, 1408, 2, 40), (96, 16384, 4, 8), (36, 4096, 3, 1), (63, 4096, 4, 1)], seed0=9)

@@ -6,8 +6,8 @@ calls, so the test makes two calls in a row -- the second on a different matrix,
 count -- and compares each with qb_quantize_pack_weights (caller workspace) on the same input and with
 the CPU oracle's quantizer and packer.  Packed words, Delta and q0 are integer / byte-exact results in
 this library's tests, so they must be equal.  The shapes are chosen so that each of the quantizer's paths
-runs against the built-in scratch (status word, and the range tables of the two-pass path): several groups
-per warp, groups cut over the warps of a CTA, a group held by a thread-block cluster, and the two passes.
+runs against the built-in scratch (status word, and the slots of the ring): several groups
+per warp, groups cut over the warps of a CTA, a group held by a thread-block cluster, and the ring.
 """
 import numpy as np
 import pytest
@@ -34,7 +34,7 @@ def test_noalloc_matches_workspace_entry_point_twice_in_a_row():
     ws = qb.workspace(groups=qb.NOALLOC_MAX_GROUPS)
     status = torch.full((1,), 77, dtype=torch.int32, device="cuda")
     # second call: fewer groups, other width and shape, so that stale ranges of call 1 would show
-    # (768, 768, 12 groups): 384 units per group -> a cluster of two CTAs; (768, 3072, 1 group): the two passes
+    # (768, 768, 12 groups): 384 units per group -> a cluster of two CTAs; (768, 3072, 1 group): the ring
     for call, (N, K, bits, groups) in enumerate([(768, 768, 3, 768), (264, 384, 4, 11), (3072, 768, 2, 128),
                                                  (768, 768, 4, 12), (768, 3072, 8, 1)]):
         w_host = synth.weights(N, K, seed=900 + call)
