@@ -84,9 +84,9 @@ qb_status qb_read_status(const void* ws /*dev*/, void* cuda_stream);
  *   xq        dev, int8 [M][K], 16-byte aligned          (written)
  *   act_scale dev, fp32 [1]                              (written)
  *   rowsum    dev, int32 [M]                             (written)
- * One kernel for tensors of up to 32 segments (of up to 1,024 elements of a row) per SM, which stay in registers
- * while the blocks agree on the maximum; else two: a grid-wide max-abs reduction into the workspace, then
- * round/store.
+ * One kernel for tensors of up to 16 segments (of up to 1,024 elements of a row) per SM and 3,072 in all, which stay in
+ * registers while the blocks agree on the maximum; else, and where the stream has too few SMs for all of these blocks
+ * at once (a green context), two: a grid-wide max-abs reduction into the workspace, then round/store.
  */
 qb_status qb_quantize_act(const float* x, int64_t M, int64_t K, int8_t* xq, float* act_scale,
                           int32_t* rowsum, void* ws, size_t ws_bytes, void* cuda_stream);
@@ -110,8 +110,8 @@ qb_status qb_quantize_act(const float* x, int64_t M, int64_t K, int8_t* xq, floa
  * 36,864 weights are held by a thread-block cluster), and always with caller-supplied ranges
  * (nothing is reduced then).  Otherwise two: for groups of up to about 27 MB one that clears slots in the
  * workspace and one that reads the weights once, held on the chip between the range and the rounding (with
- * qb_workspace_bytes() bytes of workspace); beyond, a per-group min/max reduction into the workspace, then
- * round/clamp/pack.
+ * qb_workspace_bytes() bytes of workspace, on a stream that has all SMs); beyond, a per-group min/max reduction into the
+ * workspace, then round/clamp/pack.
  */
 qb_status qb_quantize_pack_weights(const float* w, int64_t N, int64_t K, int bits, int groups,
                                    const float* range_lo, const float* range_hi, uint32_t* packed,
@@ -322,8 +322,8 @@ qb_status qb_layer_linears_i8(const qb_linear_desc* descs /*host*/, const float*
  *   wq       dev fp32 [N][K], 16-byte aligned                     (written)
  *   delta,q0 dev fp32 [G]                                         (written)
  *   range_lo, range_hi: dev fp32 [G] or both NULL, as for qb_quantize_pack_weights.
- * One kernel (W read once) in the cases where qb_quantize_pack_weights takes one; otherwise two:
- * per-group min/max reduction into the workspace, then round/clamp/dequantize.
+ * The launches are those of qb_quantize_pack_weights, with dequantize in the place of pack: W is read once for groups of up
+ * to about 27 MB and with caller-supplied ranges, twice beyond.
  *
  * Backward: grad_w = grad_wq where Clamp passes the weight through (range_lo[g] <= w <= range_hi[g],
  * both ends included), 0 where Clamp holds it at an end of the range; the rounding is treated as the
@@ -409,7 +409,7 @@ qb_status qb_sensitivity_bits(const double* lambda, int32_t layers, int32_t samp
 /*
  * Diagnostic: the rate the tensor cores sustain for the GEMM's own instruction (tcgen05.mma kind::i8,
  * s8 x s8 -> s32, 128 x `tokens` x 32) with both operands resident in shared memory, no global
- * traffic, four K blocks in flight, one CTA per SM on the default stream.  (No counterpart in the
+ * traffic, four K blocks in flight, issued by one elected thread, one CTA per SM on the default stream.  (No counterpart in the
  * paper; it gives the denominator for the tensor-bound shapes of qb_gemm.)
  *   tokens    128 or 256 (the N of the instruction)
  *   k_blocks  K blocks of 128 per CTA (8 .. 2^22); the run lasts about k_blocks * 0.3 us

@@ -5,7 +5,7 @@
 //   * the 128 rows of the MMA's A operand are 128 output neurons (weight rows), expanded from the
 //     packed k-bit words to signed 8-bit values in shared memory (Section 4: low-bit values are
 //     loaded and cast to 8 bits for execution);
-//   * the MMA's B operand is a tile of BT tokens (128 or 256) of the int8 activations, staged by TMA;
+//   * the MMA's B operand is a tile of BT tokens (128, 192 or 256) of the int8 activations, staged by TMA;
 //   * the int32 accumulator tile lives in tensor memory: TMEM lane = output neuron, column = token.
 // With this orientation the per-neuron dequantization constants are per-thread registers in the
 // epilogue and, for a fixed token, the 32 lanes of a warp hold 32 consecutive outputs of one row of
@@ -24,8 +24,8 @@
 //                 running index is g mod 4, thread r of a team owns weight row r of the tile
 //   warps 20..27  epilogue: TMEM -> registers -> fp32 -> shared memory -> TMA store; two warps per
 //                 TMEM lane quarter, each taking every other chunk of 32 tokens
-// Large launches run as CTA pairs (clusters of two, tcgen05 cta_group::2): the tile is 256 neurons x 256
-// tokens, each CTA expands its own 128 weight rows and stages its own 128 tokens, the pair's first CTA
+// Large launches run as CTA pairs (clusters of two, tcgen05 cta_group::2): the tile is 256 neurons x 256 or 192
+// tokens, each CTA expands its own 128 weight rows and stages its own half of the tokens, the pair's first CTA
 // issues one MMA for both.  That halves the token bytes each SM pulls from L2 and writes to and reads from
 // shared memory per MMA, and lets the ring be five K blocks deep instead of three.  No load is multicast.
 // One launch serves up to kMaxProblems independent linears that share the token tile: their tiles form
@@ -1097,7 +1097,9 @@ static void balance_tiles(GroupedParams& gp, int tiles, int grid, bool mixed_bit
   bool uniform = !mixed_bits;
   for (int i = 1; i < gp.count; ++i) uniform = uniform && gp.prob[i].K == gp.prob[0].K;
   if (uniform || tiles > kMaxOrder || tiles >= (int)kNoTile) return;
-  constexpr int kEpilogueCost = 5;  // a tile's fixed cost in units of one K block
+  // a tile's fixed cost in units of one K block, as measured on the launches that this was made for, stacks at M = 128 with
+  // 128-token tiles (3 or 8 instead of 5: the same times)
+  constexpr int kEpilogueCost = 5;
   // the tiles of a problem cost the same: sort the problems, not the tiles
   int by_cost[kMaxProblems], cost[kMaxProblems];
   for (int i = 0; i < gp.count; ++i) {

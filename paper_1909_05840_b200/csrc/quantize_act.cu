@@ -35,7 +35,7 @@ constexpr int kActBlocksPerSm = 4;
 constexpr int kActMaxCluster = 8;     // act_fused_kernel: CTAs of a cluster (the portable size)
 constexpr int kActMaxThreads = 1024;  // and threads of such a CTA
 constexpr int kSegUnits = 8;      // float4 per lane and segment
-constexpr int kMaxActBatch = 64;  // tensors per launch (descriptors travel as kernel parameters, 4 KB)
+constexpr int kMaxActBatch = 64;  // tensors per launch (descriptors travel as kernel parameters, 4.6 KB)
 
 struct ActItem {
   const float* x;

@@ -1,15 +1,18 @@
 // qb_quantize_pack_weights(_batch): group-wise uniform quantizer Q (Section 3.3, Appendix A) and dense
 // k-bit packing (Table 1 counts exactly k bits per weight), for one matrix or a batch of matrices.
 //
-// Two paths, chosen per matrix on the host:
+// Three paths, chosen per matrix on the host (a unit is 128 consecutive elements of one row):
 //   weight_regs_kernel   one read of W; any bit widths in one launch.  With the group's own [min, max]: groups
 //                        of up to 288 units stay in the registers of one CTA between the range and the
 //                        rounding, groups of up to 2,304 units in those of a thread-block cluster.  With
 //                        caller-supplied ranges: groups of any size (nothing to reduce).
-//   two passes           own ranges of larger groups (a range per tensor, say), below.
+//   weight_ring_kernel   one read of W: own ranges of larger groups (a range per tensor, say) of up to eleven chunks of
+//                        16 KB per SM (27 MB on 148), held in the shared memory and registers of the whole device.
+//   two passes           own ranges of groups beyond that, or where the workspace has no room for the ring's
+//                        slots, or where the stream has too few SMs for the ring's blocks at once.
 //
-// Two-pass path, first pass: the matrices of a launch are walked as one sequence of "units" of 128
-// consecutive elements of one row (one float4 per lane, fully coalesced; K % 128 == 0 so a unit never
+// Two-pass path, first pass: the matrices of a launch are walked as one sequence of units (one float4
+// per lane, fully coalesced; K % 128 == 0 so a unit never
 // crosses a row).  Each warp owns a contiguous run of units, so it crosses few group (and matrix)
 // boundaries: weight_range_kernel keeps a running min/max per lane, reduces over the warp when the group
 // changes and publishes with atomicMax on order-preserving integer encodings in the workspace (block-level
@@ -556,11 +559,6 @@ __device__ __forceinline__ uint32_t cluster_size() {
   return r;
 }
 
-// CLUSTER = false: the kernel described above.  CLUSTER = true: groups of 289 to 2,304 units; a thread-block
-// cluster of 2 to 8 CTAs (the launch's cluster size) holds one group, every CTA reduces its 16 slices,
-// writes its range into every CTA's shared memory and the cluster's barrier publishes them.  Every CTA of a
-// cluster runs the same number of items, so the barriers pair up; the last one also keeps a CTA's shared
-// memory alive until no peer writes to it any more.
 // Supplied range of group g: the caller's floats, or the encodings the range pass of the two-pass path left.
 __device__ __forceinline__ GroupParams supplied_group(const RegsItem& m, int g, int L, bool publish, void* ws) {
   if (m.encoded) {
@@ -571,6 +569,11 @@ __device__ __forceinline__ GroupParams supplied_group(const RegsItem& m, int g, 
   return finish_group(m.range_lo[g], m.range_hi[g], true, L, g, m.delta, m.q0, publish, ws);
 }
 
+// CLUSTER = false: the kernel described above.  CLUSTER = true: groups of 289 to 2,304 units; a thread-block
+// cluster of 2 to 8 CTAs (the launch's cluster size) holds one group, every CTA reduces its 16 slices,
+// writes its range into every CTA's shared memory and the cluster's barrier publishes them.  Every CTA of a
+// cluster runs the same number of items, so the barriers pair up; the last one also keeps a CTA's shared
+// memory alive until no peer writes to it any more.
 // FAKE: the fp32 fake-quantized matrix is written instead of packed words (`packed` of the item points to it).
 // CLAMP: the ranges are supplied (`range_lo`, `range_hi` of the item: the caller's, or what the range pass of
 // the two-pass path found): no reduction and no exchange, the weights are clamped into the range, and the pass
@@ -756,9 +759,9 @@ weight_regs_kernel(const __grid_constant__ RegsBatch b) {
 // a CTA holds chunks (sixteen), so the loads and ranges that a team waits for never depend on that team.
 // A chunk is held from its load until its group's range has gone round, and 37 MB are held at once: the exchange's
 // latency bounds the rate.  So a slot's two words carry their own tag: no fence, no count, no atomic; one
-// store by the writer, one load by the reader.  (The set below with atomicMax, a release count and a
-// polling lane per CTA: 97.8 us; with those per warp and chunk, which met on three words of one L2 slice: 299.)
-// Memory-bound: 4 + k/8 B per weight.
+// store by the writer, one load by the reader.  Memory-bound: 4 + k/8 B per weight.  The BERT-base set at one range
+// per matrix, 4 bits (382 MB): 74.3 us; with an atomicMax, a release count and a polling lane per CTA instead of slots
+// 97.8, with those per warp and chunk, which met on three words of one L2 slice, 299; two passes 132.5.
 constexpr int kRingUnits = 32;                 // per chunk: 16 KB
 constexpr int kRingStages = 12;
 constexpr int kRingRangeWarps = 4;
