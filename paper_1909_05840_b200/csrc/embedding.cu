@@ -105,10 +105,10 @@ emb_range_kernel(const float4* e, int64_t V, int d4, int slots, int cols_per_gro
   }
 }
 
-// Range of group g -> q0, 1/Delta, Delta; `report`: the one thread that says that the table is not finite.
-__device__ __forceinline__ void embed_group(int g, int levels, const uint32_t* g_hi, const uint32_t* g_lo_inv,
-                                            float* lo, float* inv, float* d, bool report, void* ws) {
-  float l = ordered_to_float(~g_lo_inv[g]), h = ordered_to_float(g_hi[g]);
+// Encoded range of a group -> q0, 1/Delta, Delta; `report`: the one thread that says that the table is not finite.
+__device__ __forceinline__ void embed_group(uint32_t hi_enc, uint32_t lo_inv, int levels, float* lo, float* inv, float* d,
+                                            bool report, void* ws) {
+  float l = ordered_to_float(~lo_inv), h = ordered_to_float(hi_enc);
   if (!(finite_f(l) && finite_f(h))) {
     if (report) report_status(ws, QB_ERR_NONFINITE);
     l = 0.0f;
@@ -170,12 +170,18 @@ emb_pack_kernel(const float4* e, int64_t V, int d4, int slots, int cols_per_grou
       if (i + j * step < V) v[j] = ldg_policy(e + (V - 1 - (i + j * step)) * d4 + q, pol);
     if (first) {  // the parameters, while the first rows are on their way
       first = false;
+      uint32_t eh[4], el[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {  // all of them before the first store below, which may not be passed by a load
+        eh[k] = g_hi[(4 * q + k) / cols_per_group];
+        el[k] = g_lo_inv[(4 * q + k) / cols_per_group];
+      }
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const int c = 4 * q + k, g = c / cols_per_group;
         const bool publish = blockIdx.x == 0 && slot == 0 && c == g * cols_per_group;  // first column of a group
         float d;
-        embed_group(g, L, g_hi, g_lo_inv, &lo[k], &inv[k], &d, publish, ws);
+        embed_group(eh[k], el[k], L, &lo[k], &inv[k], &d, publish, ws);
         if (publish) {
           delta[g] = d;
           q0[g] = lo[k];
