@@ -21,8 +21,8 @@
 //                      per thread: 40.0 and 48.8 us against 35.0 for the lookups below)
 // All three are streams: 4 B, 4 B + k/8 B per table element, and k/8 B + 4 B (8 B) per looked-up element.
 // 30,522 x 768 at 4 bits, 128 groups (94 MB): 52.6 us with 36 scalar operations per float4, an
-// atomic per column and a memset, 36.5 now.  24,576 tokens, word table at 4 bits then position table at 8 bits
-// accumulated: 41.4 -> 35.0 us.
+// atomic per column and a memset, 35.5 now.  24,576 tokens, word table at 4 bits then position table at 8 bits
+// accumulated: 41.4 -> 34.3 us.
 #include <algorithm>
 #include <atomic>
 
