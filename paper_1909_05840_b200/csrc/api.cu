@@ -1,4 +1,6 @@
 // Host-side plumbing of libqbert: version, status text, workspace helpers, device check.
+#include <cuda.h>
+
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -45,6 +47,30 @@ qb_status require_sm100(int* sm_count) {
   }
   if (sm_count) *sm_count = cached_sms[dev];
   return QB_OK;
+}
+
+bool stream_has_sms(cudaStream_t stream, int sms) {
+  struct Driver {
+    CUresult (*green_ctx)(CUstream, CUgreenCtx*) = nullptr;
+    CUresult (*resource)(CUgreenCtx, CUdevResource*, CUdevResourceType) = nullptr;
+    Driver() {
+      void *a = nullptr, *b = nullptr;
+      cudaDriverEntryPointQueryResult qa, qb;
+      if (cudaGetDriverEntryPoint("cuStreamGetGreenCtx", &a, cudaEnableDefault, &qa) == cudaSuccess && qa == cudaDriverEntryPointSuccess &&
+          cudaGetDriverEntryPoint("cuGreenCtxGetDevResource", &b, cudaEnableDefault, &qb) == cudaSuccess &&
+          qb == cudaDriverEntryPointSuccess) {
+        green_ctx = reinterpret_cast<decltype(green_ctx)>(a);
+        resource = reinterpret_cast<decltype(resource)>(b);
+      } else {
+        cudaGetLastError();  // a driver without green contexts
+      }
+    }
+  };
+  static const Driver driver;
+  CUgreenCtx ctx = nullptr;
+  if (!driver.green_ctx || driver.green_ctx(stream, &ctx) != CUDA_SUCCESS || !ctx) return true;
+  CUdevResource res;
+  return driver.resource(ctx, &res, CU_DEV_RESOURCE_TYPE_SM) == CUDA_SUCCESS && (int)res.sm.smCount >= sms;
 }
 
 }  // namespace qb

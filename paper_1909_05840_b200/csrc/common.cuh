@@ -105,6 +105,11 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned b
   return cudaLaunchKernelEx(&cfg, kernel, std::decay_t<P>(args)...);
 }
 
+// Does work on this stream have `sms` SMs?  Asked before a cooperative launch whose grid is made for the whole device: a
+// stream of a green context may have fewer.  Outside a capture the driver refuses such a launch (below); under capture
+// it does not, and the graph waits for room that never comes.
+bool stream_has_sms(cudaStream_t stream, int sms);
+
 // Was a launch refused because its blocks (of a cooperative launch, of a cluster) cannot be resident together?  The
 // grids are made for the whole device; a green context or an MPS client may have fewer SMs.  The forms that need
 // residency have one beside them that does not, which such a launch falls back to.

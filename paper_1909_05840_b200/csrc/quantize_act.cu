@@ -365,7 +365,8 @@ static qb_status launch_act_batch(const qb_act_desc* d, int count, void* ws, uin
         QB_CUDA_TRY(e);
         return QB_OK;
       }
-    } else if (segs <= (int64_t)sm_count * (kActBlocksPerSm * kActWarps / 2) && segs <= kWsClusters * kActMaxCluster * 2 * kActWarps) {
+    } else if (segs <= (int64_t)sm_count * (kActBlocksPerSm * kActWarps / 2) && segs <= kWsClusters * kActMaxCluster * 2 * kActWarps &&
+               stream_has_sms(stream, sm_count)) {
       // Several clusters while they need no more than half of the warps that the device holds, so that clusters of CTAs
       // of 8 or 16 warps find their place: 1,024 x 768 12.4 us, 14.3 as two launches; 1,500 x 1,024 14.0, 15.0;
       // 2,368 x 1,024 14.4, 15.2.  A segment per warp for all the warps there are (one CTA a cluster, cooperative) is the

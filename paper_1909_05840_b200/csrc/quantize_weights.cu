@@ -1442,7 +1442,7 @@ static std::vector<LargeJob> plan_large_groups(const std::vector<HostWeight>& m,
 static qb_status launch_large_groups(const std::vector<HostWeight>& m, void* ws, size_t ws_bytes, int sm_count,
                                      cudaStream_t stream, bool fake) {
   for (const LargeJob& j : plan_large_groups(m, sm_count)) {
-    bool two_pass = !j.ring || kWsRangeOff + ring_table_bytes((size_t)j.groups) > ws_bytes;
+    bool two_pass = !j.ring || kWsRangeOff + ring_table_bytes((size_t)j.groups) > ws_bytes || !stream_has_sms(stream, sm_count);
     qb_status st = QB_OK;
     if (!two_pass) st = launch_ring(j.m.data(), (int)j.m.size(), ws, sm_count, stream, fake, &two_pass);
     if (st == QB_OK && two_pass) st = launch_two_pass(j.m.data(), (int)j.m.size(), ws, sm_count, stream, fake);

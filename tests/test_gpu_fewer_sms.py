@@ -68,3 +68,44 @@ def test_quantize_weights(part, groups):
     whole = qb.quantize_pack_weights(wd, 3, groups, ws)
     assert torch.equal(whole[0], packed)
     assert qb.read_status(ws) == qb.QB_OK
+
+
+# Under capture nothing refuses a cooperative launch that does not fit: the graph would wait for room for ever.
+@pytest.mark.parametrize("what", ("one cluster", "several clusters", "two launches", "registers", "clusters", "ring"))
+def test_captured(part, what):
+    ws = qb.workspace(groups=4096)
+    stream = torch.cuda.ExternalStream(part.Stream().cuda_stream)
+    if what in ("registers", "clusters", "ring"):
+        groups = {"registers": 768, "clusters": 4, "ring": 1}[what]
+        w = gu.dev(synth.weights(768, 768, seed=groups))
+        outs = list(qb.quantize_pack_weights(w, 3, groups, ws))
+        outs.append(qb.fake_quantize_weights(w, 4, groups, ws)[0])
+
+        def call():
+            qb.quantize_pack_weights(w, 3, groups, ws, packed=outs[0], delta=outs[1], q0=outs[2])
+            qb.fake_quantize_weights(w, 4, groups, ws, wq=outs[3])
+    else:
+        M = {"one cluster": 256, "several clusters": 2368, "two launches": 6000}[what]
+        x = gu.dev(synth.activations(M, 768, seed=M))
+        outs = list(qb.quantize_act(x, ws))
+
+        def call():
+            qb.quantize_act(x, ws, *outs)
+
+    expected = [o.clone() for o in outs]  # the whole device's, which the other tests compare with the oracle
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(stream):
+        g.capture_begin()
+        try:
+            call()
+        finally:
+            g.capture_end()
+        for _ in range(2):
+            for o in outs:
+                gu.poison(o)
+            g.replay()
+            stream.synchronize()  # (synchronising the device does not wait for a green context's stream)
+            assert all(torch.equal(a, b) for a, b in zip(outs, expected))
+            stream.synchronize()
+    assert qb.read_status(ws) == qb.QB_OK
