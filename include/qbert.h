@@ -85,8 +85,8 @@ qb_status qb_read_status(const void* ws /*dev*/, void* cuda_stream);
  *   act_scale dev, fp32 [1]                              (written)
  *   rowsum    dev, int32 [M]                             (written)
  * One kernel for tensors of up to 16 segments (of up to 1,024 elements of a row) per SM and 3,072 in all, which stay in
- * registers while the blocks agree on the maximum; else, and where the stream has too few SMs for all of these blocks
- * at once (a green context), two: a grid-wide max-abs reduction into the workspace, then round/store.
+ * registers while the blocks agree on the maximum; else, and on a stream that has a part of the SMs (a green context),
+ * two: a grid-wide max-abs reduction into the workspace, then round/store.
  */
 qb_status qb_quantize_act(const float* x, int64_t M, int64_t K, int8_t* xq, float* act_scale,
                           int32_t* rowsum, void* ws, size_t ws_bytes, void* cuda_stream);

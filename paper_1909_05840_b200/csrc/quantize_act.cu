@@ -352,12 +352,16 @@ static qb_status launch_act_batch(const qb_act_desc* d, int count, void* ws, uin
   b.segs_total = segs;
   b.keep_fraction = l2_keep_fraction(512.0 * (double)units);
   const int64_t seg_blocks = (segs + kActWarps - 1) / kActWarps;
-  if constexpr (P == 1) {  // (a launch that is refused for want of SMs goes on to the two launches below)
+  if constexpr (P == 1) {
+    // A part of the device takes the two launches below, as does a launch that is refused for want of SMs: they need no
+    // blocks resident together, neither a grid's nor a cluster's (the CTAs of a cluster need SMs of one GPC).
+    const bool together = segs <= (int64_t)sm_count * (kActBlocksPerSm * kActWarps / 2) &&
+                          segs <= kWsClusters * kActMaxCluster * 2 * kActWarps && stream_has_sms(stream, sm_count);
     b.units_per_block = 0;
     // With the GEMM behind it, one cluster of up to 8 CTAs (the portable size; 256 segments) against all blocks
     // resident and one word: M = 128 x 768 9.4 us, 14.3; 256 x 768 10.2, 14.3.  CTAs of at least 1, 4 or 16 warps take as
     // long as those of 8, to 0.3 us.
-    if (segs <= kActMaxCluster * (kActMaxThreads / 32)) {
+    if (together && segs <= kActMaxCluster * (kActMaxThreads / 32)) {
       const unsigned warps = (unsigned)std::max<int64_t>((segs + kActMaxCluster - 1) / kActMaxCluster, kActWarps);
       const unsigned ctas = (unsigned)((segs + warps - 1) / warps);
       const cudaError_t e = launch_kernel(act_fused_kernel<false>, ctas, warps * 32, 0, stream, true, ctas, false, b);
@@ -365,8 +369,7 @@ static qb_status launch_act_batch(const qb_act_desc* d, int count, void* ws, uin
         QB_CUDA_TRY(e);
         return QB_OK;
       }
-    } else if (segs <= (int64_t)sm_count * (kActBlocksPerSm * kActWarps / 2) && segs <= kWsClusters * kActMaxCluster * 2 * kActWarps &&
-               stream_has_sms(stream, sm_count)) {
+    } else if (together) {
       // Several clusters while they need no more than half of the warps that the device holds, so that clusters of CTAs
       // of 8 or 16 warps find their place: 1,024 x 768 12.4 us, 14.3 as two launches; 1,500 x 1,024 14.0, 15.0;
       // 2,368 x 1,024 14.4, 15.2.  A segment per warp for all the warps there are (one CTA a cluster, cooperative) is the

@@ -31,7 +31,7 @@ def in_part(part, call):
         part.pop_context()
 
 
-# one cluster of one and of 8 CTAs; 5 clusters; 152 CTAs of 16 warps, more than 16 SMs hold; two launches
+# on the whole device: one cluster of one and of 8 CTAs; 5 clusters; 152 CTAs of 16 warps, more than 16 SMs hold; two launches
 @pytest.mark.parametrize("M,K", [(3, 256), (256, 1024), (320, 1024), (2368, 1024), (6000, 768)])
 def test_quantize_act(part, M, K):
     ws = qb.workspace(groups=64)
