@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "qbert.h"
@@ -103,6 +104,20 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned b
   cfg.attrs = attr;
   cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kernel, std::decay_t<P>(args)...);
+}
+
+// For kernels that use no shared memory to speak of: the SM's whole data cache is L1.  Without the request such a
+// kernel, set up while one that fills the shared memory drains, runs on under that kernel's split and has little L1 for its
+// loads in flight; with it its blocks come once the SM is free, and the launch itself is still hidden.
+template <class K>
+inline cudaError_t prefer_l1(K kernel) {
+  static std::atomic<bool> done[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess || (dev >= 0 && dev < 64 && done[dev].load(std::memory_order_acquire))) return e;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
+  if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev].store(true, std::memory_order_release);
+  return e;
 }
 
 // Does work on this stream have `sms` SMs?  Asked before a cooperative launch whose grid is made for the whole device: a
