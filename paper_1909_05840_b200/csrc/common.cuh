@@ -109,13 +109,14 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned b
 // For kernels that use no shared memory to speak of: the SM's whole data cache is L1.  Without the request such a
 // kernel, set up while one that fills the shared memory drains, runs on under that kernel's split and has little L1 for its
 // loads in flight; with it its blocks come once the SM is free, and the launch itself is still hidden.
-template <class K>
-inline cudaError_t prefer_l1(K kernel) {
+// The kernel is a template argument, and not one of the call, so that each has flags of its own: several kernels have one type.
+template <auto Kernel>
+inline cudaError_t prefer_l1() {
   static std::atomic<bool> done[64] = {};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess || (dev >= 0 && dev < 64 && done[dev].load(std::memory_order_acquire))) return e;
-  e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
+  e = cudaFuncSetAttribute(Kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
   if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev].store(true, std::memory_order_release);
   return e;
 }
