@@ -4,7 +4,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <atomic>
 #include <type_traits>
 
 #include "qbert.h"
@@ -77,7 +76,14 @@ inline bool valid_bits(int b) { return b == 2 || b == 3 || b == 4 || b == 8; }
 // each without it, 2.2 us with it.
 // `cluster`: CTAs per cluster; `cooperative`: every block must be resident at once (the blocks wait on
 // one another).
-template <class... P, class... A>
+// `SPLIT`: kMostL1 asks for the SM's data cache as L1, for the kernels that use next to no shared memory and follow a GEMM,
+// which takes nearly all of it.  Without the request such a kernel, set up while the GEMM drains, runs under the GEMM's
+// split and has little L1 for its loads in flight; with it its blocks come once the SM is free.  A preference of the one
+// launch: it can neither fail a call nor outlast it, as one that is set on the function could.
+// Encoder layer at M = 4096, in us with new inputs each pass: first pass of the quantizer launched after the GEMM 78.6, set up
+// under it 84.3, that with the request 77.2; two large layers at M = 24576 1,067, 1,136, 1,066.
+enum CacheSplit { kAnySplit, kMostL1 };
+template <CacheSplit SPLIT = kAnySplit, class... P, class... A>
 inline cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
                                  bool overlap, unsigned cluster, bool cooperative, A&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -85,7 +91,7 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned b
   cfg.blockDim = dim3(block, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cudaLaunchAttribute attr[3];
+  cudaLaunchAttribute attr[4];
   int n = 0;
   if (overlap) {
     attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -101,24 +107,13 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned b
     attr[n].id = cudaLaunchAttributeCooperative;
     attr[n++].val.cooperative = 1;
   }
+  if (SPLIT == kMostL1) {
+    attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[n++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxL1;
+  }
   cfg.attrs = attr;
   cfg.numAttrs = n;
   return cudaLaunchKernelEx(&cfg, kernel, std::decay_t<P>(args)...);
-}
-
-// For kernels that use no shared memory to speak of: the SM's whole data cache is L1.  Without the request such a
-// kernel, set up while one that fills the shared memory drains, runs on under that kernel's split and has little L1 for its
-// loads in flight; with it its blocks come once the SM is free, and the launch itself is still hidden.
-// The kernel is a template argument, and not one of the call, so that each has flags of its own: several kernels have one type.
-template <auto Kernel>
-inline cudaError_t prefer_l1() {
-  static std::atomic<bool> done[64] = {};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess || (dev >= 0 && dev < 64 && done[dev].load(std::memory_order_acquire))) return e;
-  e = cudaFuncSetAttribute(Kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxL1);
-  if (e == cudaSuccess && dev >= 0 && dev < 64) done[dev].store(true, std::memory_order_release);
-  return e;
 }
 
 // Does work on this stream have `sms` SMs?  Asked before a cooperative launch whose grid is made for the whole device: a

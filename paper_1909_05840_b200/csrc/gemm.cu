@@ -1391,9 +1391,8 @@ extern "C" qb_status qb_rowsum_i8(const int8_t* xq, int64_t M, int64_t K, int32_
   if (st != QB_OK) return st;
   int64_t blocks = (M + 7) / 8;
   if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
-  QB_CUDA_TRY(qb::prefer_l1<qb::rowsum_i8_kernel>());
-  QB_CUDA_TRY(qb::launch_kernel(qb::rowsum_i8_kernel, (unsigned)blocks, 256, 0, (cudaStream_t)cuda_stream, true, 1, false,
-                                reinterpret_cast<const int4*>(xq), M, K / 16, rowsum));
+  QB_CUDA_TRY(qb::launch_kernel<qb::kMostL1>(qb::rowsum_i8_kernel, (unsigned)blocks, 256, 0, (cudaStream_t)cuda_stream, true, 1, false,
+                                             reinterpret_cast<const int4*>(xq), M, K / 16, rowsum));
   return QB_OK;
 }
 

@@ -388,10 +388,8 @@ static qb_status launch_act_batch(const qb_act_desc* d, int count, void* ws, uin
   int64_t share = (units + cap - 1) / cap;
   share = (share + kSegUnits - 1) / kSegUnits * kSegUnits;
   b.units_per_block = share;
-  QB_CUDA_TRY(prefer_l1<act_absmax_kernel<P>>());
-  QB_CUDA_TRY(prefer_l1<act_quantize_kernel<P>>());
-  QB_CUDA_TRY(launch_kernel(act_absmax_kernel<P>, (unsigned)((units + share - 1) / share), kActThreads, 0, stream, true, 1, false, b));
-  QB_CUDA_TRY(launch_kernel(act_quantize_kernel<P>, (unsigned)std::min(seg_blocks, cap), kActThreads, 0, stream, true, 1, false, b));
+  QB_CUDA_TRY(launch_kernel<kMostL1>(act_absmax_kernel<P>, (unsigned)((units + share - 1) / share), kActThreads, 0, stream, true, 1, false, b));
+  QB_CUDA_TRY(launch_kernel<kMostL1>(act_quantize_kernel<P>, (unsigned)std::min(seg_blocks, cap), kActThreads, 0, stream, true, 1, false, b));
   return QB_OK;
 }
 

@@ -1,4 +1,4 @@
-"""What the activation quantizer asks the CUDA runtime for, seen from the runtime: the library's own sources are linked with
+"""What the activation quantizer and the row sums ask the CUDA runtime for, seen from the runtime: the library's own sources are linked with
 a runtime that launches nothing and writes down every launch (no GPU)."""
 import ctypes
 import subprocess
@@ -41,8 +41,11 @@ const char* cudaGetErrorString(cudaError_t) { return "fake"; }
 cudaError_t cudaMemcpyAsync(void*, const void*, size_t, cudaMemcpyKind, cudaStream_t) { return cudaErrorUnknown; }
 cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t) { return cudaErrorUnknown; }
 cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaErrorUnknown; }
+static bool refuse;
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
-  if (a == cudaFuncAttributePreferredSharedMemoryCarveout) of_function[f] = v;
+  if (a != cudaFuncAttributePreferredSharedMemoryCarveout) return cudaSuccess;
+  if (refuse) return cudaErrorInvalidValue;
+  of_function[f] = v;
   return cudaSuccess;
 }
 cudaError_t cudaLaunchKernel(const void*, dim3, dim3, void**, size_t, cudaStream_t) { return cudaErrorUnknown; }
@@ -58,6 +61,8 @@ int fake_launches() { return (int)launches.size(); }
 const char* fake_name(int i) { return launches[i].name.c_str(); }
 int fake_l1(int i) { return launches[i].l1; }
 void fake_clear() { launches.clear(); }
+void fake_refuse(int r) { refuse = r; }
+int fake_functions_set() { return (int)of_function.size(); }
 }
 """
 
@@ -66,12 +71,18 @@ void fake_clear() { launches.clear(); }
 def lib(tmp_path_factory):
     d = tmp_path_factory.mktemp("fake_runtime")
     (d / "runtime.cpp").write_text(FAKE_RUNTIME)
-    include = ["-I", str(qb_build.INCLUDE), "-I", str(qb_build.CSRC)]
-    nvcc = [qb_build._nvcc(), "-std=c++17", "-O3", "-gencode", "arch=compute_100a,code=sm_100a", "-Xcompiler", "-fPIC", *include]
-    procs = [subprocess.Popen([*nvcc, "-c", str(qb_build.CSRC / s), "-o", str(d / (s + ".o"))]) for s in ("api.cu", "quantize_act.cu")]
-    procs.append(subprocess.Popen([*nvcc, "-c", str(d / "runtime.cpp"), "-o", str(d / "runtime.o")]))
+    qb_build.build()
+    nvcc = [qb_build._nvcc(), "-std=c++17", "-O3", "-gencode", "arch=compute_100a,code=sm_100a", "-Xcompiler", "-fPIC",
+            "-I", str(qb_build.INCLUDE), "-I", str(qb_build.CSRC)]
+    objects, procs = [], [subprocess.Popen([*nvcc, "-c", str(d / "runtime.cpp"), "-o", str(d / "runtime.o")])]
+    for source in ("api.cu", "quantize_act.cu", "gemm.cu"):
+        obj = qb_build.PKG / "_build" / (source + ".o")
+        if qb_build._stale(obj, "*.cu", "*.cuh"):  # a library that came without its objects
+            obj = d / (source + ".o")
+            procs.append(subprocess.Popen([*nvcc, "-c", str(qb_build.CSRC / source), "-o", str(obj)]))
+        objects.append(str(obj))
     assert all([p.wait() == 0 for p in procs])
-    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic,-z,defs", "-o", str(d / "fake.so"), *(str(o) for o in sorted(d.glob("*.o")))], check=True)
+    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic,-z,defs", "-o", str(d / "fake.so"), str(d / "runtime.o"), *objects], check=True)
     lib = ctypes.CDLL(str(d / "fake.so"))
     lib.fake_name.restype = ctypes.c_char_p
     return lib
@@ -95,6 +106,20 @@ def quantize_batch(lib, shapes):
     for d, (M, K) in zip(descs, shapes):
         d.x, d.M, d.K, d.xq, d.act_scale, d.rowsum = 1 << 32, M, K, 2 << 32, 3 << 32, 4 << 32
     return lib.qb_quantize_act_batch(descs, len(shapes), ctypes.c_void_p(5 << 32), ctypes.c_size_t(1 << 20), ctypes.c_void_p(0))
+
+
+def rowsum(lib, M, K):
+    p = ctypes.c_void_p
+    return lib.qb_rowsum_i8(p(1 << 32), ctypes.c_int64(M), ctypes.c_int64(K), p(2 << 32), p(0))
+
+
+def test_a_preference_neither_fails_a_call_nor_outlasts_it(lib):
+    calls = (lambda: quantize(lib, 6000, 768), lambda: quantize_batch(lib, [(128, 768)] * 3), lambda: rowsum(lib, 6000, 768))
+    for refuse in (1, 0):
+        lib.fake_refuse(refuse)
+        for call in calls:
+            assert all(l1 for _, l1 in launches(lib, call))
+            assert lib.fake_functions_set() == 0  # nothing that later launches of the process would find
 
 
 def test_both_passes_ask_for_l1(lib):
