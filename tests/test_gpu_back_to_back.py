@@ -81,6 +81,81 @@ def test_pack_then_gemm_then_requantize(M, N, K, groups, small_ws):
     assert qb.read_status(ws) == qb.QB_OK
 
 
+# The quantizer's two launches set up under the GEMM that makes their input (more than 2,368 segments), of one and of several
+# segments a row; then under a GEMM that still reads the codes and the row sums which they overwrite.
+@pytest.mark.parametrize("M,K,N", [(3001, 768, 768), (1000, 2304, 3072)])
+def test_gemm_then_two_launch_quantizer(M, K, N):
+    bits, groups = 4, 12
+    ws = qb.workspace(groups=64)
+    xs = [synth.activations(M, K, seed=i) * np.float32(REPS - i) for i in range(REPS)]  # smaller and smaller
+    w = synth.weights(N, K, seed=10)
+    d_x, b = [gu.dev(x) for x in xs], buffers(M, N, K, bits, groups)
+    qb.quantize_pack_weights(gu.dev(w), bits, groups, ws, packed=b["packed"], delta=b["delta"], q0=b["q0"])
+    y = torch.empty((M, N), device="cuda")
+    kept, ys = [torch.empty_like(y) for _ in range(REPS)], [torch.empty_like(y) for _ in range(REPS)]
+    again = [buffers(M, N, N, bits, groups) for _ in range(REPS)]
+    torch.cuda.synchronize()
+    for i in range(REPS):
+        qb.quantize_act(d_x[i], ws, b["xq"], b["sc"], b["rs"])
+        qb.gemm(b["xq"], b["sc"], b["rs"], b["packed"], b["delta"], b["q0"], None, N, bits, groups, ws, y=y)
+        qb.quantize_act(y, ws, again[i]["xq"], again[i]["sc"], again[i]["rs"])
+        kept[i].copy_(y)
+    for i in range(REPS):
+        qb.quantize_act(d_x[i], ws, b["xq"], b["sc"], b["rs"])
+        qb.gemm(b["xq"], b["sc"], b["rs"], b["packed"], b["delta"], b["q0"], None, N, bits, groups, ws, y=ys[i])
+    torch.cuda.synchronize()
+    _, codes, o_delta, o_q0 = oracle.quantize_weights(w, bits, groups)
+    sel = gu.sample_rows(M)
+    for i in range(REPS):
+        _, o_xq, o_s, o_rs = oracle.quantize_act(xs[i])
+        gu.assert_y_close(kept[i].cpu().numpy()[sel], oracle.dequant_epilogue(oracle.int_gemm(o_xq[sel], codes), o_rs[sel], o_s, o_delta,
+                                                                              o_q0, None, bits, groups))
+        assert torch.equal(ys[i], kept[i]), i
+        _, o_xq, o_s, o_rs = oracle.quantize_act(kept[i].cpu().numpy())
+        assert again[i]["sc"].item() == o_s, i
+        assert np.array_equal(again[i]["xq"].cpu().numpy(), o_xq) and np.array_equal(again[i]["rs"].cpu().numpy(), o_rs), i
+    assert qb.read_status(ws) == qb.QB_OK
+
+
+@pytest.mark.parametrize("M", (33, 128))
+def test_stack_then_batch_quantizer(M):
+    bits, groups = 4, 8
+    ws = qb.workspace(groups=64)
+    shapes = [(768, 768), (3072, 768), (768, 3072)]
+    xs = [[synth.activations(M, K, seed=3 * i + j) * np.float32(REPS - i) for j, (_, K) in enumerate(shapes)] for i in range(REPS)]
+    w = [synth.weights(N, K, seed=40 + j) for j, (N, K) in enumerate(shapes)]
+    b = [buffers(M, N, K, bits, groups) for N, K in shapes]
+    for wj, bj in zip(w, b):
+        qb.quantize_pack_weights(gu.dev(wj), bits, groups, ws, packed=bj["packed"], delta=bj["delta"], q0=bj["q0"])
+    ys = [torch.empty((M, N), device="cuda") for N, _ in shapes]
+    kept = [[torch.empty_like(y) for y in ys] for _ in range(REPS)]
+    again = [[buffers(M, N, N, bits, groups) for N, _ in shapes] for _ in range(REPS)]
+    d_x = [[gu.dev(x) for x in rep] for rep in xs]
+    first = [qb.make_act_desc_array([(x, bj["xq"], bj["sc"], bj["rs"]) for x, bj in zip(rep, b)]) for rep in d_x]
+    linears = qb.make_desc_array([qb.LinearDesc(bj["xq"], bj["sc"], bj["rs"], bj["packed"], bj["delta"], bj["q0"], None, N, bits, groups, y)
+                                  for bj, y, (N, _) in zip(b, ys, shapes)])
+    second = [qb.make_act_desc_array([(y, a["xq"], a["sc"], a["rs"]) for y, a in zip(ys, rep)]) for rep in again]
+    torch.cuda.synchronize()
+    for i in range(REPS):
+        qb.quantize_act_batch(first[i], ws)
+        qb.layer_linears(linears, ws)
+        qb.quantize_act_batch(second[i], ws)
+        for k, y in zip(kept[i], ys):
+            k.copy_(y)
+    torch.cuda.synchronize()
+    for j in range(len(shapes)):
+        _, codes, o_delta, o_q0 = oracle.quantize_weights(w[j], bits, groups)
+        for i in range(REPS):
+            _, o_xq, o_s, o_rs = oracle.quantize_act(xs[i][j])
+            y = kept[i][j].cpu().numpy()
+            gu.assert_y_close(y, oracle.dequant_epilogue(oracle.int_gemm(o_xq, codes), o_rs, o_s, o_delta, o_q0, None, bits, groups))
+            _, o_xq, o_s, o_rs = oracle.quantize_act(y)
+            a = again[i][j]
+            assert a["sc"].item() == o_s, (i, j)
+            assert np.array_equal(a["xq"].cpu().numpy(), o_xq) and np.array_equal(a["rs"].cpu().numpy(), o_rs), (i, j)
+    assert qb.read_status(ws) == qb.QB_OK
+
+
 @pytest.mark.parametrize("N,K,groups,small_ws", [(128, 256, 8, False), (768, 768, 4, False), (768, 768, 1, False), (768, 768, 1, True)])
 def test_fake_quantize_then_pack_then_backward(N, K, groups, small_ws):
     ws = qb.workspace(groups=4096)
