@@ -71,9 +71,9 @@ inline bool valid_bits(int b) { return b == 2 || b == 3 || b == 4 || b == 8; }
   } while (0)
 
 // Launch of a kernel that begins with pdl_begin.
-// `overlap`: programmatic stream serialization: the kernel's blocks may be set up while the kernel before it on
-// the stream drains, and wait in pdl_begin for its completion.  Back to back launches of 592 blocks: 4.1 us
-// each without it, 2.2 us with it.
+// Programmatic stream serialization: the kernel's blocks may be set up while the kernel before it on the stream
+// drains, and wait in pdl_begin for its completion.  Back to back launches of 592 blocks: 4.1 us each without it, 2.2 us
+// with it.
 // `cluster`: CTAs per cluster; `cooperative`: every block must be resident at once (the blocks wait on
 // one another).
 // `SPLIT`: kMostL1 asks for the SM's data cache as L1, for the kernels that use next to no shared memory and follow a GEMM,
@@ -85,18 +85,16 @@ inline bool valid_bits(int b) { return b == 2 || b == 3 || b == 4 || b == 8; }
 enum CacheSplit { kAnySplit, kMostL1 };
 template <CacheSplit SPLIT = kAnySplit, class... P, class... A>
 inline cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,
-                                 bool overlap, unsigned cluster, bool cooperative, A&&... args) {
+                                 unsigned cluster, bool cooperative, A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid, 1, 1);
   cfg.blockDim = dim3(block, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[4];
-  int n = 0;
-  if (overlap) {
-    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[n++].val.programmaticStreamSerializationAllowed = 1;
-  }
+  int n = 1;
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
   if (cluster > 1) {
     attr[n].id = cudaLaunchAttributeClusterDimension;
     attr[n].val.clusterDim.x = cluster;

@@ -321,13 +321,13 @@ extern "C" qb_status qb_quantize_embedding(const float* table, int64_t V, int64_
   // two blocks per SM; slots * D <= 4096 columns: at most 32 KB of shared memory
   const unsigned rblocks = (unsigned)std::min((V + slots - 1) / slots, (int64_t)sms * 2);
   QB_CUDA_TRY(qb::launch_kernel(qb::emb_range_kernel, rblocks, (unsigned)block, (size_t)slots * 2 * (size_t)D * sizeof(uint32_t), stream,
-                                true, 1, false, e4, V, d4, slots, cpg, groups, qb::l2_keep_fraction(4.0 * (double)V * (double)D), g_hi,
+                                1, false, e4, V, d4, slots, cpg, groups, qb::l2_keep_fraction(4.0 * (double)V * (double)D), g_hi,
                                 g_lo, ws));
   auto pack = bits == 2 ? qb::emb_pack_kernel<2> : (bits == 3 ? qb::emb_pack_kernel<3> : (bits == 4 ? qb::emb_pack_kernel<4> : qb::emb_pack_kernel<8>));
   unsigned grid = 0;
   st = qb::emb_grid(pack, qb::kEmbPack, bits, d4, V, sms, &grid);
   if (st != QB_OK) return st;
-  QB_CUDA_TRY(qb::launch_kernel(pack, grid, (unsigned)block, 0, stream, true, 1, false, e4, V, d4, slots, cpg, g_hi, g_lo, packed, delta, q0,
+  QB_CUDA_TRY(qb::launch_kernel(pack, grid, (unsigned)block, 0, stream, 1, false, e4, V, d4, slots, cpg, g_hi, g_lo, packed, delta, q0,
                                 ws));
   return QB_OK;
 }
@@ -359,7 +359,7 @@ extern "C" qb_status qb_embedding_lookup(const int32_t* ids, int64_t T, const ui
   unsigned grid = 0;
   st = qb::emb_grid(lookup, accumulate ? qb::kEmbLookupAdd : qb::kEmbLookup, bits, d4, T, sms, &grid);
   if (st != QB_OK) return st;
-  QB_CUDA_TRY(qb::launch_kernel(lookup, grid, (unsigned)block, 0, stream, true, 1, false, ids, T, packed, V, d4, slots, (int)(D / groups),
+  QB_CUDA_TRY(qb::launch_kernel(lookup, grid, (unsigned)block, 0, stream, 1, false, ids, T, packed, V, d4, slots, (int)(D / groups),
                                 delta, q0, reinterpret_cast<float4*>(out), ws));
   return QB_OK;
 }

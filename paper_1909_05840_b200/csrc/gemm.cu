@@ -995,7 +995,7 @@ static qb_status launch_group_inst(const GP& gp, int grid, cudaStream_t stream) 
     QB_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::kSmemBytes));
     if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_release);
   }
-  QB_CUDA_TRY(launch_kernel(kernel, (unsigned)grid, kGemmThreads, Cfg::kSmemBytes, stream, true, CG, false, gp));
+  QB_CUDA_TRY(launch_kernel(kernel, (unsigned)grid, kGemmThreads, Cfg::kSmemBytes, stream, CG, false, gp));
   return QB_OK;
 }
 
@@ -1391,7 +1391,7 @@ extern "C" qb_status qb_rowsum_i8(const int8_t* xq, int64_t M, int64_t K, int32_
   if (st != QB_OK) return st;
   int64_t blocks = (M + 7) / 8;
   if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
-  QB_CUDA_TRY(qb::launch_kernel<qb::kMostL1>(qb::rowsum_i8_kernel, (unsigned)blocks, 256, 0, (cudaStream_t)cuda_stream, true, 1, false,
+  QB_CUDA_TRY(qb::launch_kernel<qb::kMostL1>(qb::rowsum_i8_kernel, (unsigned)blocks, 256, 0, (cudaStream_t)cuda_stream, 1, false,
                                              reinterpret_cast<const int4*>(xq), M, K / 16, rowsum));
   return QB_OK;
 }

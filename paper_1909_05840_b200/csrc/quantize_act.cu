@@ -364,7 +364,7 @@ static qb_status launch_act_batch(const qb_act_desc* d, int count, void* ws, uin
     if (together && segs <= kActMaxCluster * (kActMaxThreads / 32)) {
       const unsigned warps = (unsigned)std::max<int64_t>((segs + kActMaxCluster - 1) / kActMaxCluster, kActWarps);
       const unsigned ctas = (unsigned)((segs + warps - 1) / warps);
-      const cudaError_t e = launch_kernel(act_fused_kernel<false>, ctas, warps * 32, 0, stream, true, ctas, false, b);
+      const cudaError_t e = launch_kernel(act_fused_kernel<false>, ctas, warps * 32, 0, stream, ctas, false, b);
       if (!residency_refused(e)) {
         QB_CUDA_TRY(e);
         return QB_OK;
@@ -376,7 +376,7 @@ static qb_status launch_act_batch(const qb_act_desc* d, int count, void* ws, uin
       // slower one: 4,500 x 768 18.4, 16.4 as two launches; 1,000 x 4,096 26.4, 24.6.
       const int64_t warps = segs <= kWsClusters * kActMaxCluster * kActWarps ? kActWarps : 2 * kActWarps;
       const unsigned clusters = (unsigned)((segs + warps * kActMaxCluster - 1) / (warps * kActMaxCluster));
-      const cudaError_t e = launch_kernel(act_fused_kernel<true>, clusters * kActMaxCluster, (unsigned)warps * 32, 0, stream, true,
+      const cudaError_t e = launch_kernel(act_fused_kernel<true>, clusters * kActMaxCluster, (unsigned)warps * 32, 0, stream,
                                           kActMaxCluster, true, b);
       if (!residency_refused(e)) {
         QB_CUDA_TRY(e);
@@ -388,8 +388,8 @@ static qb_status launch_act_batch(const qb_act_desc* d, int count, void* ws, uin
   int64_t share = (units + cap - 1) / cap;
   share = (share + kSegUnits - 1) / kSegUnits * kSegUnits;
   b.units_per_block = share;
-  QB_CUDA_TRY(launch_kernel<kMostL1>(act_absmax_kernel<P>, (unsigned)((units + share - 1) / share), kActThreads, 0, stream, true, 1, false, b));
-  QB_CUDA_TRY(launch_kernel<kMostL1>(act_quantize_kernel<P>, (unsigned)std::min(seg_blocks, cap), kActThreads, 0, stream, true, 1, false, b));
+  QB_CUDA_TRY(launch_kernel<kMostL1>(act_absmax_kernel<P>, (unsigned)((units + share - 1) / share), kActThreads, 0, stream, 1, false, b));
+  QB_CUDA_TRY(launch_kernel<kMostL1>(act_quantize_kernel<P>, (unsigned)std::min(seg_blocks, cap), kActThreads, 0, stream, 1, false, b));
   return QB_OK;
 }
 

@@ -1169,7 +1169,7 @@ static qb_status launch_two_pass(const HostWeight* m, int count, void* ws, int s
   const int64_t warps = (units + upw - 1) / upw;
   const unsigned blocks = (unsigned)((warps + kWqWarps - 1) / kWqWarps);
 
-  QB_CUDA_TRY(launch_kernel(weight_range_kernel, blocks, kWqThreads, 0, stream, true, 1, false, b));
+  QB_CUDA_TRY(launch_kernel(weight_range_kernel, blocks, kWqThreads, 0, stream, 1, false, b));
   HostWeight second[kMaxWeightBatch];
   for (int i = 0; i < count; ++i) {
     second[i] = m[i];
@@ -1257,7 +1257,7 @@ static qb_status launch_regs_cluster(const HostWeight* m, int count, int cl, voi
     b.total_items = items;
     b.count = n;
     QB_CUDA_TRY(launch_kernel(fake ? weight_regs_kernel<true, true, false> : weight_regs_kernel<true, false, false>,
-                              (unsigned)(std::min(items, max_clusters) * cl), kRgThreads, 0, stream, true, (unsigned)cl, false, b));
+                              (unsigned)(std::min(items, max_clusters) * cl), kRgThreads, 0, stream, (unsigned)cl, false, b));
   }
   return QB_OK;
 }
@@ -1331,7 +1331,7 @@ static qb_status launch_regs_single(const HostWeight* m, int count, bool ranged,
     const unsigned grid = (unsigned)std::min<int64_t>(items, sm_count);
     auto kernel = ranged ? (fake ? weight_regs_kernel<false, true, true> : weight_regs_kernel<false, false, true>)
                          : (fake ? weight_regs_kernel<false, true, false> : weight_regs_kernel<false, false, false>);
-    QB_CUDA_TRY(launch_kernel(kernel, grid, kRgThreads, 0, stream, true, 1, false, b));
+    QB_CUDA_TRY(launch_kernel(kernel, grid, kRgThreads, 0, stream, 1, false, b));
   }
   return QB_OK;
 }
@@ -1373,7 +1373,7 @@ static qb_status launch_ring_form(const RingBatch& b, unsigned grid, cudaStream_
     QB_CUDA_TRY(cudaFuncSetAttribute(weight_ring_kernel<FAKE>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingSmemBytes));
     if (dev >= 0 && dev < 64) attr_set[dev].store(true, std::memory_order_release);
   }
-  const cudaError_t e = launch_kernel(weight_ring_kernel<FAKE>, grid, kRingThreads, kRingSmemBytes, stream, true, 1, true, b);
+  const cudaError_t e = launch_kernel(weight_ring_kernel<FAKE>, grid, kRingThreads, kRingSmemBytes, stream, 1, true, b);
   *refused = residency_refused(e);
   if (!*refused) QB_CUDA_TRY(e);
   return QB_OK;
@@ -1405,7 +1405,7 @@ static qb_status launch_ring(const HostWeight* m, int count, void* ws, int sm_co
   b.count = count;
   const unsigned grid = (unsigned)std::min(chunks, std::min(sm_count, kRingMaxCtas));
   const int slots = groups * (int)grid;
-  QB_CUDA_TRY(launch_kernel(clear_slots_kernel, (unsigned)std::min((slots + 255) / 256, sm_count), 256, 0, stream, true, 1, false,
+  QB_CUDA_TRY(launch_kernel(clear_slots_kernel, (unsigned)std::min((slots + 255) / 256, sm_count), 256, 0, stream, 1, false,
                             b.slots, slots));
   return fake ? launch_ring_form<true>(b, grid, stream, refused) : launch_ring_form<false>(b, grid, stream, refused);
 }
@@ -1641,7 +1641,7 @@ extern "C" qb_status qb_ste_backward(const float* grad_wq, const float* w, int64
     return QB_ERR_INVALID;
   }
   const int64_t blocks = std::min((units + 8 * qb::kSteUnits - 1) / (8 * qb::kSteUnits), (int64_t)sms * 64);
-  QB_CUDA_TRY(qb::launch_kernel(qb::ste_backward_kernel, (unsigned)blocks, 256, 0, stream, true, 1, false,
+  QB_CUDA_TRY(qb::launch_kernel(qb::ste_backward_kernel, (unsigned)blocks, 256, 0, stream, 1, false,
                                 reinterpret_cast<const float4*>(grad_wq), reinterpret_cast<const float4*>(w), units,
                                 (uint32_t)(N / groups * (K / 128)), range_lo, range_hi, reinterpret_cast<float4*>(grad_w)));
   return QB_OK;
