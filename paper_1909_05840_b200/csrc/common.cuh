@@ -80,8 +80,11 @@ inline bool valid_bits(int b) { return b == 2 || b == 3 || b == 4 || b == 8; }
 // which takes nearly all of it.  Without the request such a kernel, set up while the GEMM drains, runs under the GEMM's
 // split and has little L1 for its loads in flight; with it its blocks come once the SM is free.  A preference of the one
 // launch: it can neither fail a call nor outlast it, as one that is set on the function could.
-// Encoder layer at M = 4096, in us with new inputs each pass: first pass of the quantizer launched after the GEMM 78.6, set up
-// under it 84.3, that with the request 77.2; two large layers at M = 24576 1,067, 1,136, 1,066.
+// In us, with new inputs each pass: encoder layer at M = 4096 with the quantizer's first pass launched after the GEMM 78.6,
+// set up under it 84.3, that with the request 77.2; two large layers at M = 24576 1,067, 1,136, 1,066.  On both passes rather
+// than the first alone: the same on one stream; ten quantizer batches beside five such layers' GEMMs on another stream
+// 496, 509 (launched after the GEMM: 509), beside three calls of the ring quantizer 517, 524 (519).
+// The other kernels with little shared memory (embeddings, straight-through backward) have not been tried with it.
 enum CacheSplit { kAnySplit, kMostL1 };
 template <CacheSplit SPLIT = kAnySplit, class... P, class... A>
 inline cudaError_t launch_kernel(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream,

@@ -228,8 +228,8 @@ act_quantize_kernel(const __grid_constant__ ActBatch<P> b) {
 // the cluster.  MANY: the maxima of several clusters, all resident (cooperative launch), meet in the workspace: each
 // is stored with the launch's number, and every block polls for all of them, one release and one acquire in all;
 // no word has to be cleared first.  All blocks resident that met in one word (clear, maximum, count, go-ahead,
-// read: five trips to L2) took, with the GEMM, 12.7 us at M = 32 x 768 (now, one cluster: 9.3), 14.3 at
-// 1,024 x 768 (now, 16 clusters: 12.4).
+// read: five trips to L2) took, with the GEMM, 12.7 us at M = 32 x 768 (now, one cluster: 9.1), 14.3 at
+// 1,024 x 768 (now, 16 clusters: 12.6).
 template <bool MANY>
 __global__ void __launch_bounds__(kActMaxThreads, 1)
 act_fused_kernel(const __grid_constant__ ActBatch<1> b) {
@@ -371,9 +371,12 @@ static qb_status launch_act_batch(const qb_act_desc* d, int count, void* ws, uin
       }
     } else if (together) {
       // Several clusters while they need no more than half of the warps that the device holds, so that clusters of CTAs
-      // of 8 or 16 warps find their place: 1,024 x 768 12.4 us, 14.3 as two launches; 1,500 x 1,024 14.0, 15.0;
-      // 2,368 x 1,024 14.4, 15.2.  A segment per warp for all the warps there are (one CTA a cluster, cooperative) is the
-      // slower one: 4,500 x 768 18.4, 16.4 as two launches; 1,000 x 4,096 26.4, 24.6.
+      // of 8 or 16 warps find their place.  What they give is a launch less for a call that is waited for; in a row of
+      // calls the two launches overlap their neighbours and draw level at about 768 segments of 1,024.  One linear (N = 768),
+      // us, one launch / two; in a row: 320 x 1,024 12.4 / 13.0, 768 x 1,024 13.3 / 13.4, 1,024 x 768 13.1 / 12.7, 1,536 x 1,024
+      // 14.5 / 14.2, 2,368 x 1,024 15.0 / 14.9; each waited for: 20.8 / 22.3, 20.9 / 22.4, 20.4 / 21.9, 22.2 / 23.3, 22.6 / 24.1.
+      // A segment per warp for all the warps there are (one CTA a cluster, cooperative) was slower than two launches even
+      // before these overlapped: 4,500 x 768 18.4 / 16.4; 1,000 x 4,096 26.4 / 24.6.
       const int64_t warps = segs <= kWsClusters * kActMaxCluster * kActWarps ? kActWarps : 2 * kActWarps;
       const unsigned clusters = (unsigned)((segs + warps * kActMaxCluster - 1) / (warps * kActMaxCluster));
       const cudaError_t e = launch_kernel(act_fused_kernel<true>, clusters * kActMaxCluster, (unsigned)warps * 32, 0, stream,
